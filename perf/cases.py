@@ -87,7 +87,7 @@ def _most_replicas(R, L, N):
     16) rebuild by N^2 / 2 binary64 adds per replica: fewer replicas."""
     m = L // 3 if L % 3 == 0 else L
     fast = m & (m - 1) == 0 or (L % 16 == 0 and R >= 8)
-    return R if fast else max(1, min(R, int(1.0e9 / (N * N / 2.0))))
+    return R if fast else max(1, min(R, 64, int(1.0e9 / (N * N / 2.0))))
 
 
 def draw(rng):
