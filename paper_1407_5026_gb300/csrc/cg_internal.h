@@ -41,6 +41,17 @@ struct alignas(16) DevCounters {
 constexpr int kGuideBits = 12;
 constexpr int kGuide = 1 << kGuideBits;
 
+// Guide table of the single-hop lattice kernel (cg_pr_lattice.cuh): bucket
+// b = x1 >> (32 - kLatGuideBits) holds v - lat_guide_base(V) when every x1 of
+// the bucket selects the same vector v and that difference is in [0, 254],
+// else 255 (the kernel then searches the thresholds between the bounds of
+// x1's top kLatHintBits bits).  The vectors are ordered dy outer, dx inner, so
+// the probable ones lie in the middle of the list: the base centres the 255
+// representable ones there.
+constexpr int kLatGuideBits = 14;
+constexpr int kLatHintBits = 7;
+__host__ __device__ inline int lat_guide_base(int V) { return V <= 255 ? 0 : (V - 255) / 2; }
+
 // Everything one CTA needs to run one replica.
 struct alignas(16) DevReplica {
     int L, N, H1, V;          // side, sites, folded extent L/2+1, hop vectors
@@ -64,6 +75,7 @@ struct alignas(16) DevReplica {
     const double *tinv_r2_64; // cubic lattice: 1/r by r^2 = fx^2+fy^2+fz^2, 3 (L/2)^2 + 1
     const float *tinv_r2_32;  // entries (the folded table's values); null on the square one
     const unsigned short *guide; // kGuide entries
+    const unsigned char *guide8; // 2^kLatGuideBits entries
     // state (device)
     void *eps;                // N binary64 (CG_FP64) or binary32 (CG_FP32)
     unsigned int *occ;        // occupation bitmask, bit s%32 of word s/32
@@ -110,6 +122,7 @@ struct RunArgs {
     int time_mode;                 // CG_TIME_DETERMINISTIC or CG_TIME_GAUSSIAN
     int pair;                      // 1: two-electron hops (the kPair instances)
     int smem_guide;                // random sites, one CTA: guide records in shared memory
+    int guide_bits;                // single hops on one CTA: log2 of the guide table's entries
     double toy_A0;
 };
 
@@ -138,6 +151,50 @@ __host__ __device__ inline SmemLayout smem_layout(int N, int tab_entries, int V,
     s.off_cv32 = o;  o = cg_align16(o + V * 4);
     s.total = o;
     return s;
+}
+
+// Shared-memory carve-up of the single-hop lattice kernel (cg_pr_lattice.cuh)
+// with a guide table of 2^gbits entries.
+struct LatLayout {
+    int off_eps, off_tinv, off_occ, off_guide, off_hint, off_thr, off_rec;
+    int off_vr64, off_edx64, total;
+};
+
+__host__ __device__ inline LatLayout lat_layout(int N, int tab_entries, int V, int words,
+                                                int real_bytes, int gbits)
+{
+    LatLayout s;
+    int o = 0;
+    s.off_eps = o;   o = cg_align16(o + N * real_bytes);
+    s.off_tinv = o;  o = cg_align16(o + tab_entries * real_bytes);
+    s.off_occ = o;   o = cg_align16(o + words * 4);
+    s.off_guide = o; o = cg_align16(o + (1 << gbits));
+    s.off_hint = o;  o = cg_align16(o + ((1 << kLatHintBits) + 1) * 2);
+    s.off_thr = o;   o = cg_align16(o + V * 4);
+    s.off_rec = o;   o = cg_align16(o + V * 8);
+    s.off_vr64 = o;  o = cg_align16(o + V * 8);
+    s.off_edx64 = o; o = cg_align16(o + V * 8);
+    s.total = o;
+    return s;
+}
+
+// Guide bits of that kernel: a finer table sends fewer labels to the search
+// (about 0.5% of x1's range at 14 bits, 1% at 13 for r_max = 8), so the
+// largest of 14, 13 and 12 that costs no CTA per SM (228 KiB of shared memory,
+// at most four CTAs of 256 threads by registers) and fits the 227 KiB of one
+// CTA with room for the static part.  12 bits take less than the two-electron
+// kernel's layout, so a lattice that fits that one fits this.
+inline int lat_guide_bits(int N, int tab_entries, int V, int words, int real_bytes)
+{
+    auto total = [&](int b) { return lat_layout(N, tab_entries, V, words, real_bytes, b).total; };
+    auto ctas = [&](int b) {
+        const int c = (228 * 1024) / (total(b) + 3072);
+        return c < 4 ? c : 4;
+    };
+    const int most = 227 * 1024 - 2048;
+    for (int b = kLatGuideBits; b > 12; --b)
+        if (total(b) <= most && ctas(b) == ctas(12)) return b;
+    return 12;
 }
 
 // Random sites (cg_pr_random.cu): the coupling matrix from the positions,

@@ -116,6 +116,7 @@ struct Tables {
     std::vector<int> disp;
     std::vector<double> tinvd;
     std::vector<unsigned short> guide;
+    std::vector<unsigned char> guide8;
     std::vector<uint32_t> split;      // hi | lo << 16 of each 1/r entry: BF16 of 1/r on the
                                       // square lattice, binary16 of 2^10 / r on the cubic one
     // cubic lattice: the folded table's values indexed by r^2 = fx^2 + fy^2 +
@@ -131,6 +132,7 @@ struct Tables {
     float *d_ghat = nullptr;
     float2 *d_tw = nullptr;
     unsigned short *d_guide = nullptr;
+    unsigned char *d_guide8 = nullptr;
     uint32_t *d_split = nullptr;
     double *d_t64 = nullptr;
     float *d_t32 = nullptr;
@@ -245,6 +247,18 @@ int build_tables(Tables &t, int L, double xi, int r_max, int dim)
         const bool multi = scan && v + 1 < t.V && t.thr[v + 1] < hi;
         t.guide[b] = (unsigned short)(v | (scan ? 0x8000 : 0) | (multi ? 0x4000 : 0));
     }
+    // guide table of the single-hop lattice kernel: the bucket's vector when it
+    // holds no threshold inside and none of its words is a null proposal
+    const int shift8 = 32 - kLatGuideBits, base = lat_guide_base(t.V);
+    t.guide8.assign((size_t)1 << kLatGuideBits, 255);
+    v = 0;
+    for (int b = 0; b < (1 << kLatGuideBits); ++b) {
+        const unsigned long long lo = (unsigned long long)b << shift8;
+        const unsigned long long hi = lo + (1ull << shift8) - 1;
+        while (v < t.V - 1 && t.thr[v] < lo) ++v;
+        const int g = v - base;
+        if (t.thr[v] >= hi && g >= 0 && g < 255) t.guide8[b] = (unsigned char)g;
+    }
     return CG_OK;
 }
 
@@ -279,6 +293,7 @@ struct Group {
     int dim = 2;                     // 2: square lattice, 3: cubic lattice
     bool random = false;             // random-site replicas (pr_random)
     bool sguide = false;             // their guide records in shared memory
+    int gbits = kLatGuideBits;       // guide bits of the single-hop lattice kernel
     int cluster = 1;                 // CTAs per replica
     unsigned M = 4096;               // labels per round when cg_run is given M = 0
     bool tuned = false;
@@ -516,6 +531,13 @@ double gamma_of(const Rep &r, const cg_opts &o)
     return Tp ? g / (1.0 - (double)Tp * 0x1p-32) : g;
 }
 
+// Guide bits of a lattice replica on the single-hop kernel.
+int guide_bits_of(const Rep &r, int precision)
+{
+    return lat_guide_bits(r.N, (int)r.tab->t64.size(), r.tab->V, r.words,
+                          precision == CG_FP64 ? 8 : 4);
+}
+
 // The single-hop cluster kernel on the cubic lattice keeps 1/r indexed by
 // r^2 (3 (L/2)^2 + 1 entries) instead of the (L/2+1)^3 folded table.
 int persistent_smem(const Rep &r, int precision, int cluster = 1)
@@ -524,6 +546,8 @@ int persistent_smem(const Rep &r, int precision, int cluster = 1)
     const int rb = precision == CG_FP64 ? 8 : 4;
     const bool r2 = dim_of(r.d) == 3 && cluster > 1 && !r.pair;
     const int ntab = r2 ? (int)r.tab->r2_64.size() : (int)r.tab->t64.size();
+    if (cluster == 1 && !r.pair)
+        return lat_layout(r.N, ntab, r.tab->V, r.words, rb, guide_bits_of(r, precision)).total;
     return smem_layout(r.N / cluster, ntab, r.tab->V, r.words, rb).total;
 }
 
@@ -591,6 +615,7 @@ void fill_dev(const Rep &r, const cg_opts &o, DevReplica &dr, cg_hop *log)
     dr.tinv_r2_64 = t.d_r2_64; dr.tinv_r2_32 = t.d_r2_32;
     dr.tinvd = t.d_tinvd;
     dr.guide = t.d_guide;
+    dr.guide8 = t.d_guide8;
     dr.C0 = t.C0;
     dr.eps = r.d_eps; dr.occ = r.d_occ; dr.phi = r.d_phi; dr.ctr = r.d_ctr;
     dr.log = log;
@@ -919,7 +944,7 @@ size_t plan_bytes(int R, const cg_replica_desc *reps, const cg_opts &o)
                         if (r2 > 0 && r2 <= d.r_max * d.r_max) ++V;
                     }
             total += up(tab * 8) + up(tab * 4) + up(V * 4) + up(V * 4) + up(V * 8) +
-                     up((size_t)kGuide * 2) + up(tab * 4);
+                     up((size_t)kGuide * 2) + up((size_t)1 << kLatGuideBits) + up(tab * 4);
             if (dim_of(d) == 3) {
                 const size_t n2 = 3 * (size_t)(d.L / 2) * (d.L / 2) + 1;
                 total += up(n2 * 8) + up(n2 * 4);
@@ -1055,6 +1080,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
             dalloc(h.get(), (void **)&t->d_disp, t->disp.size() * 4) ||
             dalloc(h.get(), (void **)&t->d_tinvd, t->tinvd.size() * 8) ||
             dalloc(h.get(), (void **)&t->d_guide, t->guide.size() * 2) ||
+            dalloc(h.get(), (void **)&t->d_guide8, t->guide8.size()) ||
             dalloc(h.get(), (void **)&t->d_split, t->split.size() * 4)) { destroy_partial(); return nullptr; }
         if (!t->ghat.empty()) {
             if (dalloc(h.get(), (void **)&t->d_ghat, t->ghat.size() * 4) ||
@@ -1075,6 +1101,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         cudaMemcpyAsync(t->d_disp, t->disp.data(), t->disp.size() * 4, cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(t->d_tinvd, t->tinvd.data(), t->tinvd.size() * 8, cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(t->d_guide, t->guide.data(), t->guide.size() * 2, cudaMemcpyHostToDevice, h->st);
+        cudaMemcpyAsync(t->d_guide8, t->guide8.data(), t->guide8.size(), cudaMemcpyHostToDevice, h->st);
     }
     for (Rep &r : h->reps) {
         if (!r.random) continue;
@@ -1152,6 +1179,10 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         for (int m = k; m < R && gkey(order[m]) == gkey(order[k]); ++m)
             g.sguide = g.sguide && h->reps[order[m]].sguide;
         g.first = k;
+        // one table size for the group: the smallest its replicas take (their
+        // hop disks, and so their other tables, may differ)
+        for (int m = k; !g.random && m < R && gkey(order[m]) == gkey(order[k]); ++m)
+            g.gbits = std::min(g.gbits, guide_bits_of(h->reps[order[m]], o.precision));
         const int key = gkey(order[k]);
         int smem = 0, cluster = 1;
         for (int m = k; m < R && gkey(order[m]) == key; ++m)
@@ -1311,6 +1342,7 @@ int launch_group(cg_handle *h, const Group &g, unsigned long long hops, unsigned
     a.toy_A0 = h->toy_A0;
     a.time_mode = h->opts.time_mode;
     a.pair = h->opts.pair_frac > 0.0 ? 1 : 0;
+    a.guide_bits = g.gbits;
     a.smem_guide = (g.random && g.cluster == 1 && g.sguide) ? 1 : 0;
     if (g.random && g.cluster > 1)
         CG_CUDA(launch_pr_random_cluster(h->d_reps, h->d_index + g.first, g.count, g.cluster,

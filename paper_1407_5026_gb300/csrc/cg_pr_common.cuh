@@ -167,21 +167,11 @@ __device__ __forceinline__ float metropolis_bound_f32(float dE, float invTf)
     return __fmaf_rn(e, 0x1p23f, -0.5f);
 }
 
-// Step 2 (accept test) for a proposal whose theta holds, from the two local
-// energies (read from this CTA's shared memory or a cluster peer's).
-template <typename Real>
-__device__ __forceinline__ bool accept_vals(Real ei, Real ej, const Shared &S, const Prop &p,
-                                            double T, float invTf, double &dE_out);
-
-template <>
-__device__ __forceinline__ bool accept_vals<double>(double ei, double ej, const Shared &S,
-                                                    const Prop &p, double T, float invTf,
-                                                    double &dE_out)
+// The Metropolis decision u < e^(-dH/T) for dH > 0 in binary64 semantics: a
+// binary32 estimate of e^(-dH/T) with a relative margin decides most cases,
+// the binary64 exponential the rest.
+__device__ __forceinline__ bool metropolis64(double dE, uint32_t x2, double T, float invTf)
 {
-    double d = d_sub(ej, ei);
-    d = d_sub(d, S.vr64[p.v]);
-    const double dE = d_sub(d, S.edx64[p.v]);
-    dE_out = dE;
     if (dE <= 0.0) return true;
     // binary32 estimate of y = -dE/T and of e^y, then a margin test
     const float df = approx_f32(dE);
@@ -192,60 +182,64 @@ __device__ __forceinline__ bool accept_vals<double>(double ei, double ej, const 
         // u ~ x2 2^-32 differs from (x2 + 1/2) 2^-32 by at most 2^-33 plus a
         // relative 2^-24: the absolute slack 2^-31 covers the first, the
         // relative margin the second and the exponential's error
-        const float u = __uint2float_rn(p.x2) * 0x1p-32f;
+        const float u = __uint2float_rn(x2) * 0x1p-32f;
         if (u + 0x1p-31f < e * (1.0f - 2e-4f)) return true;
         if (u > e * (1.0f + 2e-4f) + 0x1p-31f) return false;
     }
-    const double u = d_mul(d_add((double)p.x2, 0.5), 0x1p-32);
+    const double u = d_mul(d_add((double)x2, 0.5), 0x1p-32);
     return u < cg_exp_accept(d_div(-dE, T));
 }
 
-template <>
-__device__ __forceinline__ bool accept_vals<float>(float ei, float ej, const Shared &S,
-                                                   const Prop &p, double T, float invTf,
-                                                   double &dE_out)
+// The binary32 Metropolis decision: u = (m + 1/2) 2^-23 with m = x2 >> 9
+// (exact in binary32), and u < e^(-dH/T) tested as m < e 2^23 - 1/2.
+__device__ __forceinline__ bool metropolis_f32(float dE, uint32_t x2, float invTf)
 {
-    const float dEf = __fsub_rn(__fsub_rn(ej, ei), S.cv32[p.v]);
+    return dE <= 0.0f || (float)(x2 >> 9) < metropolis_bound_f32(dE, invTf);
+}
+
+// Step 2 (accept test) of a label whose theta holds, from the two local
+// energies, 1/r_v and E dx_v (binary64) and their binary32 sum.
+template <typename Real>
+__device__ __forceinline__ bool metropolis_label(Real ei, Real ej, double vr, double edx, float cv,
+                                                 uint32_t x2, double T, float invTf,
+                                                 double &dE_out);
+
+template <>
+__device__ __forceinline__ bool metropolis_label<double>(double ei, double ej, double vr,
+                                                         double edx, float cv, uint32_t x2,
+                                                         double T, float invTf, double &dE_out)
+{
+    const double dE = d_sub(d_sub(d_sub(ej, ei), vr), edx);
+    dE_out = dE;
+    return metropolis64(dE, x2, T, invTf);
+}
+
+template <>
+__device__ __forceinline__ bool metropolis_label<float>(float ei, float ej, double vr, double edx,
+                                                        float cv, uint32_t x2, double T,
+                                                        float invTf, double &dE_out)
+{
+    const float dEf = __fsub_rn(__fsub_rn(ej, ei), cv);
     if (fabsf(dEf) < 1e-5f) {
         // near tie: decide in binary64 from the widened energies
-        double d = d_sub((double)ej, (double)ei);
-        d = d_sub(d, S.vr64[p.v]);
-        const double dE = d_sub(d, S.edx64[p.v]);
+        const double dE = d_sub(d_sub(d_sub((double)ej, (double)ei), vr), edx);
         dE_out = dE;
         if (dE <= 0.0) return true;
-        const double u = d_mul(d_add((double)p.x2, 0.5), 0x1p-32);
+        const double u = d_mul(d_add((double)x2, 0.5), 0x1p-32);
         return u < cg_exp_accept(d_div(-dE, T));
     }
     dE_out = 0.0;   // widened for the executed hop only
-    if (dEf <= 0.0f) return true;
-    // u = (m + 1/2) 2^-23 with m = x2 >> 9 (exact in binary32); u < e^(-dH/T)
-    // tested as m < e 2^23 - 1/2
-    return (float)(p.x2 >> 9) < metropolis_bound_f32(dEf, invTf);
+    return metropolis_f32(dEf, x2, invTf);
 }
 
-// Step 2 for the two labels of a thread in the binary32 form, without a
-// branch per label: the energies are read for every label (its sites are
-// valid even when theta fails) and theta masks the result, so the two
-// dependency chains interleave.  Near ties (|dH| < 1e-5) are re-decided in
-// binary64 by accept_vals<float>.
-__device__ __forceinline__ void accept2_f32(const Shared &S, const Prop &p0, const Prop &p1,
-                                            double T, float invTf, bool &acc0, bool &acc1,
-                                            double &dE0, double &dE1)
+// Step 2 for a proposal of propose() whose theta holds (energies read from
+// this CTA's shared memory or a cluster peer's).
+template <typename Real>
+__device__ __forceinline__ bool accept_vals(Real ei, Real ej, const Shared &S, const Prop &p,
+                                            double T, float invTf, double &dE_out)
 {
-    const float *eps = reinterpret_cast<const float *>(S.eps);
-    const float d0 = __fsub_rn(__fsub_rn(eps[p0.j], eps[p0.i]), S.cv32[p0.v]);
-    const float d1 = __fsub_rn(__fsub_rn(eps[p1.j], eps[p1.i]), S.cv32[p1.v]);
-    const float t0 = metropolis_bound_f32(d0, invTf);
-    const float t1 = metropolis_bound_f32(d1, invTf);
-    acc0 = p0.theta && (d0 <= 0.0f || (float)(p0.x2 >> 9) < t0);
-    acc1 = p1.theta && (d1 <= 0.0f || (float)(p1.x2 >> 9) < t1);
-    dE0 = 0.0;
-    dE1 = 0.0;
-    const bool tie0 = p0.theta && fabsf(d0) < 1e-5f, tie1 = p1.theta && fabsf(d1) < 1e-5f;
-    if (tie0 || tie1) {
-        if (tie0) acc0 = accept_vals<float>(eps[p0.i], eps[p0.j], S, p0, T, invTf, dE0);
-        if (tie1) acc1 = accept_vals<float>(eps[p1.i], eps[p1.j], S, p1, T, invTf, dE1);
-    }
+    return metropolis_label<Real>(ei, ej, S.vr64[p.v], S.edx64[p.v], S.cv32[p.v], p.x2, T, invTf,
+                                  dE_out);
 }
 
 // ---------------------------------------------------------------------------
@@ -393,24 +387,6 @@ __device__ __forceinline__ double pair_dE64(const Shared &S, const double *tab64
     return d_add(d_add(d1, d2), d_sub(d_sub(tlj, tli), d_sub(tkj, tki)));
 }
 
-// The Metropolis decision u < e^(-dH/T) for dH > 0 in binary64 semantics
-// (a binary32 estimate with a margin decides most cases).
-__device__ __forceinline__ bool metropolis64(double dE, uint32_t x2, double T, float invTf)
-{
-    if (dE <= 0.0) return true;
-    const float df = approx_f32(dE);
-    if (df > 0.0f) {
-        const float y = -df * invTf;
-        if (y < -23.01f) return false;
-        const float e = __expf(y);
-        const float u = __uint2float_rn(x2) * 0x1p-32f;
-        if (u + 0x1p-31f < e * (1.0f - 2e-4f)) return true;
-        if (u > e * (1.0f + 2e-4f) + 0x1p-31f) return false;
-    }
-    const double u = d_mul(d_add((double)x2, 0.5), 0x1p-32);
-    return u < cg_exp_accept(d_div(-dE, T));
-}
-
 // Step 2 for a pair whose theta holds.  Binary64: exact dH.  Binary32: the
 // same sum in binary32 from the binary32 table, re-decided in binary64 from
 // the widened energies and the binary64 table when |dH| < 1e-5 (dE_out is
@@ -507,17 +483,6 @@ __device__ __forceinline__ double hop_dE(const Shared &S, const Prop &p, double 
 {
     const Real *eps = reinterpret_cast<const Real *>(S.eps);
     return hop_dE_vals<Real>(eps[p.i], eps[p.j], S, p, dE);
-}
-
-// dH of an accepting label in binary64, redone for the executed hop from its
-// proposal: the value the accept test computed (binary64 form; binary32 near
-// ties) or the binary32 dH widened.
-template <typename Real>
-__device__ __forceinline__ double winner_dE(const Shared &S, const Prop &p, double T, float invTf)
-{
-    double dE = 0.0;
-    accept<Real>(S, p, T, invTf, dE);
-    return hop_dE<Real>(S, p, dE);
 }
 
 }  // namespace cg

@@ -1,8 +1,8 @@
 // cg_pr_kernel.cu -- launches of the persistent parallel-rejection kernel
-// (cg_pr_persistent.cuh) on the square lattice, with L = 32, 48, 64, 96 and
+// (cg_pr_lattice.cuh) on the square lattice, with L = 32, 48, 64, 96 and
 // 128 fixed at compile time and any other L at run time; cubic lattices go
 // to cg_pr_kernel3d.cu.
-#include "cg_pr_persistent.cuh"
+#include "cg_pr_lattice.cuh"
 
 namespace cg {
 
@@ -12,31 +12,31 @@ static void launch_tt(const DevReplica *d_reps, const int *d_index, int n_ctas, 
 {
     switch (L) {
     case 32:
-        pr_persistent<Real, kThreads, 5, kTime>
+        pr_lattice<Real, kThreads, 5, kTime>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
         break;
     case 48:
-        pr_persistent<Real, kThreads, -48, kTime>
+        pr_lattice<Real, kThreads, -48, kTime>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
         break;
     case 96:
-        pr_persistent<Real, kThreads, -96, kTime>
+        pr_lattice<Real, kThreads, -96, kTime>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
         break;
     case 64:
-        pr_persistent<Real, kThreads, 6, kTime>
+        pr_lattice<Real, kThreads, 6, kTime>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
         break;
     case 128:
-        pr_persistent<Real, kThreads, 7, kTime>
+        pr_lattice<Real, kThreads, 7, kTime>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
         break;
     default:
         if ((L & (L - 1)) == 0)
-            pr_persistent<Real, kThreads, 0, kTime>
+            pr_lattice<Real, kThreads, 0, kTime>
                 <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
         else
-            pr_persistent<Real, kThreads, -1, kTime>
+            pr_lattice<Real, kThreads, -1, kTime>
                 <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     }
 }
@@ -56,23 +56,23 @@ template <typename Real, int kThreads, bool kTime>
 static cudaError_t set_smem_tt(int bytes)
 {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(pr_persistent<Real, kThreads, 5, kTime>,
+    if ((e = cudaFuncSetAttribute(pr_lattice<Real, kThreads, 5, kTime>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) ||
-        (e = cudaFuncSetAttribute(pr_persistent<Real, kThreads, -48, kTime>,
+        (e = cudaFuncSetAttribute(pr_lattice<Real, kThreads, -48, kTime>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) ||
-        (e = cudaFuncSetAttribute(pr_persistent<Real, kThreads, -96, kTime>,
+        (e = cudaFuncSetAttribute(pr_lattice<Real, kThreads, -96, kTime>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)))
         return e;
-    if ((e = cudaFuncSetAttribute(pr_persistent<Real, kThreads, 6, kTime>,
+    if ((e = cudaFuncSetAttribute(pr_lattice<Real, kThreads, 6, kTime>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)))
         return e;
-    if ((e = cudaFuncSetAttribute(pr_persistent<Real, kThreads, 7, kTime>,
+    if ((e = cudaFuncSetAttribute(pr_lattice<Real, kThreads, 7, kTime>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)))
         return e;
-    if ((e = cudaFuncSetAttribute(pr_persistent<Real, kThreads, 0, kTime>,
+    if ((e = cudaFuncSetAttribute(pr_lattice<Real, kThreads, 0, kTime>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)))
         return e;
-    return cudaFuncSetAttribute(pr_persistent<Real, kThreads, -1, kTime>,
+    return cudaFuncSetAttribute(pr_lattice<Real, kThreads, -1, kTime>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 

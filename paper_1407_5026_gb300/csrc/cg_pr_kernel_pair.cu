@@ -14,10 +14,10 @@ static cudaError_t launch_pair_t(const DevReplica *d_reps, const int *d_index, i
         return launch_pr_persistent_pair_time(sizeof(Real) == 8 ? CG_FP64 : CG_FP32, d_reps,
                                               d_index, n_ctas, kThreads, smem_bytes, args, st, L);
     if ((L & (L - 1)) == 0)
-        pr_persistent<Real, kThreads, 0, false, 2, true>
+        pr_persistent<Real, kThreads, 0, false, 2>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     else
-        pr_persistent<Real, kThreads, -1, false, 2, true>
+        pr_persistent<Real, kThreads, -1, false, 2>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     return cudaGetLastError();
 }
@@ -25,8 +25,8 @@ static cudaError_t launch_pair_t(const DevReplica *d_reps, const int *d_index, i
 template <typename Real, int kThreads>
 static cudaError_t set_pair_one(int bytes)
 {
-    const void *k[2] = {(const void *)pr_persistent<Real, kThreads, 0, false, 2, true>,
-                        (const void *)pr_persistent<Real, kThreads, -1, false, 2, true>};
+    const void *k[2] = {(const void *)pr_persistent<Real, kThreads, 0, false, 2>,
+                        (const void *)pr_persistent<Real, kThreads, -1, false, 2>};
     for (const void *f : k) {
         const cudaError_t e =
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

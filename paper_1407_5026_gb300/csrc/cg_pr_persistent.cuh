@@ -40,7 +40,7 @@
 // |dH| < 1e-5), exp from the fast intrinsic.
 #pragma once
 
-#include "cg_pr_common.cuh"
+#include "cg_pr_update.cuh"
 
 namespace cg {
 
@@ -56,7 +56,7 @@ namespace cg {
 // 2 b of the chunk rule C ~ sqrt(2 m b) (b: a chunk's fixed cost in labels)
 constexpr float kChunkCost = 128.0f;
 
-template <typename Real, int kThreads, int kLog2L, bool kTime, int kDim = 2, bool kPair = false>
+template <typename Real, int kThreads, int kLog2L, bool kTime, int kDim = 2>
 __global__ void __launch_bounds__(kThreads, (kThreads >= 1024 ? 1 : 1024 / kThreads))
 pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index, RunArgs a)
 {
@@ -67,7 +67,7 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int s_wlabel[32];
     __shared__ Cand s_cand[32];
-    __shared__ PairProp s_pcand[kPair ? 32 : 1];   // the second electron of a pair candidate
+    __shared__ PairProp s_pcand[32];   // the second electron of a pair candidate
     // step-3c deviates of the next hops (CG_TIME_GAUSSIAN): warp 0 draws 32
     // at a time, one per lane, so the binary64 Box-Muller chain runs once
     // per 32 hops instead of on thread 0's path at every commit
@@ -175,26 +175,19 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
         if (tid == 0) s_c.t0 = clock64();
         // labels per chunk ~ sqrt(2 m b) for m expected labels and a chunk's
         // fixed cost (the OR barrier and the warps' imbalance before it) worth
-        // b labels: nl = 4 or 2 labels per thread (C = nl blockDim) when that
-        // exceeds blockDim, else one per thread for the first C threads (C a
-        // power of two >= 64); m_ema is identical in every thread, so the
-        // choice is uniform and idle warps skip the labels whole.  Pair
-        // instances take at most two labels per thread.
+        // b labels: two labels per thread (C = 2 blockDim) when that exceeds
+        // blockDim, else one per thread for the first C threads (C a power of
+        // two >= 64); m_ema is identical in every thread, so the choice is
+        // uniform and idle warps skip the labels whole
         const float want = sqrtf(kChunkCost * s_c.m_ema);
-        unsigned C, nl;
-        if (!kPair && want > 2.0f * (float)kThreads) {
-            nl = 4;
-            C = 4u * kThreads;
-        } else if (want > (float)kThreads) {
-            nl = 2;
+        unsigned C = 64;
+        const bool two = want > (float)kThreads;
+        if (two) {
             C = 2u * kThreads;
         } else {
-            nl = 1;
-            C = 64;
             while (C < (unsigned)kThreads && (float)C < want) C <<= 1;
             if (C > (unsigned)kThreads) C = kThreads;
         }
-        const bool two = nl > 1;
         const bool act = (unsigned)tid < C;
         unsigned long long p = 0;
         unsigned q = 0, win = 0, kb_hit = 0;
@@ -203,79 +196,8 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
             ++p;
             const PhiloxPrefix PP =
                 philox_prefix((uint32_t)rounds, (uint32_t)(rounds >> 32), rep, key0, key1);
-            PhiloxPrefix PP2{};
-            if (kPair)
-                PP2 = philox_prefix((uint32_t)rounds, (uint32_t)(rounds >> 32) | 0x80000000u, rep,
-                                    key0, key1);
-            if constexpr (!kPair) {
-            for (unsigned kb = 0; kb < M; kb += C) {
-                // bit u of accm: label kb + u blockDim + tid accepts; only the
-                // decisions stay live, the winning lane redoes its proposal
-                unsigned accm = 0;
-                if (act) {
-#pragma unroll
-                    for (unsigned u = 0; u < 4; u += 2) {
-                        if (u < nl) {
-                            const unsigned ka = kb + u * (unsigned)kThreads + (unsigned)tid;
-                            const unsigned kc = ka + (unsigned)kThreads;
-                            const bool hasc = u + 1 < nl;
-                            const bool va = ka < M, vc = hasc && kc < M;
-                            const Prop pa = propose<kPow2, kDim>(S, ka, PP, key0, key1, L, log2L,
-                                                                 (unsigned)N, magic, thr_last, va);
-                            Prop pc{};
-                            if (hasc)
-                                pc = propose<kPow2, kDim>(S, kc, PP, key0, key1, L, log2L,
-                                                          (unsigned)N, magic, thr_last, vc);
-                            bool aa = false, ac = false;
-                            double da = 0.0, dc = 0.0;
-                            if (a.toy) {
-                                aa = va && d_mul(d_add((double)pa.x2, 0.5), 0x1p-32) < a.toy_A0;
-                                ac = vc && d_mul(d_add((double)pc.x2, 0.5), 0x1p-32) < a.toy_A0;
-                            } else if (sizeof(Real) == 4 && hasc) {
-                                accept2_f32(S, pa, pc, T, invTf, aa, ac, da, dc);
-                            } else {
-                                if (pa.theta) aa = accept<Real>(S, pa, T, invTf, da);
-                                if (pc.theta) ac = accept<Real>(S, pc, T, invTf, dc);
-                            }
-                            accm |= (aa ? 1u : 0u) << u;
-                            accm |= (ac ? 1u : 0u) << (u + 1);
-                        }
-                    }
-                }
-                const int any = __syncthreads_or(accm != 0u);
-                if (any) {
-                    // the warp's lowest accepting label: the first sub-chunk
-                    // u with an accept, then the lowest lane
-                    unsigned off = 0xffffffffu;
-                    for (unsigned u = 0; u < nl; ++u) {
-                        const unsigned bu = __ballot_sync(0xffffffffu, (accm >> u) & 1u);
-                        if (bu) {
-                            off = u * (unsigned)kThreads + (unsigned)(warp * 32) +
-                                  (unsigned)(__ffs(bu) - 1);
-                            break;
-                        }
-                    }
-                    if (off != 0xffffffffu && (unsigned)lane == (off & 31u)) {
-                        const Prop pw = propose<kPow2, kDim>(S, kb + off, PP, key0, key1, L, log2L,
-                                                             (unsigned)N, magic, thr_last, true);
-                        s_cand[warp].i = pw.i;
-                        s_cand[warp].j = pw.j;
-                        s_cand[warp].dxy = pw.dxy;
-                        s_cand[warp].dE = a.toy ? 0.0 : winner_dE<Real>(S, pw, T, invTf);
-                    }
-                    if (lane == 0) s_wlabel[warp] = off;
-                    __syncthreads();
-                    unsigned wl = (lane < kThreads / 32) ? s_wlabel[lane] : 0xffffffffu;
-#pragma unroll
-                    for (int o = 16; o; o >>= 1) wl = min(wl, __shfl_xor_sync(0xffffffffu, wl, o));
-                    q = kb + wl + 1;                 // 1-based label in the round
-                    kb_hit = kb;
-                    win = (wl % (unsigned)kThreads) >> 5;
-                    found = true;
-                    break;
-                }
-            }
-            } else {
+            const PhiloxPrefix PP2 = philox_prefix(
+                (uint32_t)rounds, (uint32_t)(rounds >> 32) | 0x80000000u, rep, key0, key1);
             for (unsigned kb = 0; kb < M; kb += C) {
                 const unsigned k0 = kb + (unsigned)tid, k1 = k0 + (unsigned)kThreads;
                 const bool v0 = k0 < M, v1 = two && k1 < M;
@@ -289,7 +211,7 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
                     if (two)
                         p1 = propose<kPow2, kDim>(S, k1, PP, key0, key1, L, log2L, (unsigned)N, magic,
                                             thr_last, v1);
-                    if (kPair && !a.toy) {
+                    if (!a.toy) {
                         q0 = pair_extend<kPow2, kDim>(S, p0, k0, PP2, key0, key1, L, log2L, magic,
                                                 thr_last, Rg.pair_T, Rg.pair_R);
                         if (two)
@@ -301,7 +223,7 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
                         const double u1 = d_mul(d_add((double)p1.x2, 0.5), 0x1p-32);
                         acc0 = v0 && u0 < a.toy_A0;
                         acc1 = v1 && u1 < a.toy_A0;
-                    } else if (kPair) {
+                    } else {
                         if (p0.theta)
                             acc0 = q0.pair ? accept_pair<Real, kPow2, kDim>(S, Rg, p0, q0, T, invTf, dE0,
                                                                      L, log2L, magic, H1)
@@ -310,11 +232,6 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
                             acc1 = q1.pair ? accept_pair<Real, kPow2, kDim>(S, Rg, p1, q1, T, invTf, dE1,
                                                                      L, log2L, magic, H1)
                                            : accept<Real>(S, p1, T, invTf, dE1);
-                    } else if (sizeof(Real) == 4 && two) {
-                        accept2_f32(S, p0, p1, T, invTf, acc0, acc1, dE0, dE1);
-                    } else {
-                        if (p0.theta) acc0 = accept<Real>(S, p0, T, invTf, dE0);
-                        if (p1.theta) acc1 = accept<Real>(S, p1, T, invTf, dE1);
                     }
                 }
                 const int any = __syncthreads_or(acc0 || acc1);
@@ -329,16 +246,12 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
                             s_cand[warp].i = p0.i;
                             s_cand[warp].j = p0.j;
                             s_cand[warp].dxy = p0.dxy;
-                            if (kPair) {
-                                s_pcand[warp] = q0;
-                                s_cand[warp].dE =
-                                    a.toy ? 0.0
-                                    : q0.pair ? pair_hop_dE<Real, kPow2, kDim>(S, Rg, p0, q0, dE0, L,
-                                                                         log2L, magic, H1)
-                                              : hop_dE<Real>(S, p0, dE0);
-                            } else {
-                                s_cand[warp].dE = a.toy ? 0.0 : hop_dE<Real>(S, p0, dE0);
-                            }
+                            s_pcand[warp] = q0;
+                            s_cand[warp].dE =
+                                a.toy ? 0.0
+                                : q0.pair ? pair_hop_dE<Real, kPow2, kDim>(S, Rg, p0, q0, dE0, L,
+                                                                     log2L, magic, H1)
+                                          : hop_dE<Real>(S, p0, dE0);
                         }
                     } else if (b1) {
                         const int first = __ffs(b1) - 1;
@@ -347,16 +260,12 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
                             s_cand[warp].i = p1.i;
                             s_cand[warp].j = p1.j;
                             s_cand[warp].dxy = p1.dxy;
-                            if (kPair) {
-                                s_pcand[warp] = q1;
-                                s_cand[warp].dE =
-                                    a.toy ? 0.0
-                                    : q1.pair ? pair_hop_dE<Real, kPow2, kDim>(S, Rg, p1, q1, dE1, L,
-                                                                         log2L, magic, H1)
-                                              : hop_dE<Real>(S, p1, dE1);
-                            } else {
-                                s_cand[warp].dE = a.toy ? 0.0 : hop_dE<Real>(S, p1, dE1);
-                            }
+                            s_pcand[warp] = q1;
+                            s_cand[warp].dE =
+                                a.toy ? 0.0
+                                : q1.pair ? pair_hop_dE<Real, kPow2, kDim>(S, Rg, p1, q1, dE1, L,
+                                                                     log2L, magic, H1)
+                                          : hop_dE<Real>(S, p1, dE1);
                         }
                     }
                     if (lane == 0) s_wlabel[warp] = off;
@@ -370,7 +279,6 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
                     found = true;
                     break;
                 }
-            }
             }
             if (!found) {
                 if (tid == 0) {
@@ -401,9 +309,8 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
         const int cdx = kDim == 3 ? (c.dxy << 22) >> 22 : (int)(short)(c.dxy & 0xffff);
         const int cdy = kDim == 3 ? (c.dxy << 12) >> 22 : c.dxy >> 16;
         // second electron of an executed pair (toy mode has none)
-        PairProp cq{};
-        if (kPair) cq = s_pcand[win];
-        const bool cpair = kPair && !a.toy && cq.pair;
+        const PairProp cq = s_pcand[win];
+        const bool cpair = !a.toy && cq.pair;
         const int cdx2 = !cpair ? 0 : kDim == 3 ? (cq.dxy2 << 22) >> 22 : (int)(short)(cq.dxy2 & 0xffff);
         const int cdy2 = !cpair ? 0 : kDim == 3 ? (cq.dxy2 << 12) >> 22 : cq.dxy2 >> 16;
         long long t1 = 0;
@@ -444,131 +351,21 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
             }
         }
         rounds += 1;
+        __syncwarp();     // or warp 0 would run the update twice, once for this lane
 
         // ---- local-energy update (step 3b) ----
-        if (kDim == 3) {
-            // thread -> base column bx < L/2 and base (y, z) planes p0, p0 + rpp,
-            // ...; each base site (x, y, z) < L/2 serves the eight sites
-            // (x + a L/2, y + b L/2, z + c L/2), a, b, c in {0, 1}
-            const int Lh = L >> 1;
-            const int rpp = kThreads / Lh;
-            // an executed pair applies the second electron's update after the
-            // first one's (each site rounds twice, in the serial order)
-            const int passes3 = (kPair && cpair) ? 2 : 1;
+        // an executed pair applies the second electron's update after the first
+        // one's (each site rounds twice, in the serial order; a thread owns
+        // the same sites in both)
 #pragma unroll 1
-            for (int pass = 0; pass < passes3; ++pass)
-            if (!a.toy && tid < rpp * Lh) {
-                const unsigned ui = pass ? cq.k : ci, uj = pass ? cq.l : cj;
-                const int bx = tid % Lh, p0 = tid / Lh;
-                int xi, yi, zi, xj, yj, zj;
-                if (kPow2) {
-                    const int m = L - 1;
-                    xi = (int)ui & m; yi = (int)(ui >> log2L) & m; zi = (int)(ui >> (2 * log2L));
-                    xj = (int)uj & m; yj = (int)(uj >> log2L) & m; zj = (int)(uj >> (2 * log2L));
-                } else {
-                    const unsigned qi = __umulhi(ui, magic), qj = __umulhi(uj, magic);
-                    xi = (int)(ui - qi * (unsigned)L); zi = (int)__umulhi(qi, magic);
-                    yi = (int)qi - zi * L;
-                    xj = (int)(uj - qj * (unsigned)L); zj = (int)__umulhi(qj, magic);
-                    yj = (int)qj - zj * L;
-                }
-                const int fxj = fold_axis(bx - xj, L), fxi = fold_axis(bx - xi, L);
-                const Real *cj0 = tinv + fxj, *cj1 = tinv + (Lh - fxj);
-                const Real *ci0 = tinv + fxi, *ci1 = tinv + (Lh - fxi);
-                const int LL = L * L;
-#pragma unroll 2
-                for (int pz = p0; pz < Lh * Lh; pz += rpp) {
-                    int by, bz, fyj, fyi, fzj, fzi;
-                    if (kPow2) {
-                        // power-of-two L: shifts, masks and a min for the folds
-                        by = pz & (Lh - 1);
-                        bz = pz >> (log2L - 1);
-                        const int m = L - 1;
-                        const int dyj = (by - yj) & m, dyi = (by - yi) & m;
-                        const int dzj = (bz - zj) & m, dzi = (bz - zi) & m;
-                        fyj = min(dyj, L - dyj); fyi = min(dyi, L - dyi);
-                        fzj = min(dzj, L - dzj); fzi = min(dzi, L - dzi);
-                    } else {
-                        by = pz % Lh;
-                        bz = pz / Lh;
-                        fyj = fold_axis(by - yj, L); fyi = fold_axis(by - yi, L);
-                        fzj = fold_axis(bz - zj, L); fzi = fold_axis(bz - zi, L);
-                    }
-                    // rows (fz H1 + fy) H1 of the folded table for the four
-                    // (z, y) images of the base site, relative to j and to i
-                    int oj[2][2], oi[2][2];
-#pragma unroll
-                    for (int cz = 0; cz < 2; ++cz)
-#pragma unroll
-                        for (int cy = 0; cy < 2; ++cy) {
-                            oj[cz][cy] = ((cz ? Lh - fzj : fzj) * H1 + (cy ? Lh - fyj : fyj)) * H1;
-                            oi[cz][cy] = ((cz ? Lh - fzi : fzi) * H1 + (cy ? Lh - fyi : fyi)) * H1;
-                        }
-                    Real *e = eps + (bz * L + by) * L + bx;
-                    // odd base rows take the two x-images in swapped order, so
-                    // the half-warps of consecutive rows (L/2 = 16) touch
-                    // opposite halves of the banks at each access
-                    const int sw = p0 & 1;
-#pragma unroll
-                    for (int cz = 0; cz < 2; ++cz)
-#pragma unroll
-                        for (int cy = 0; cy < 2; ++cy)
-#pragma unroll
-                            for (int c = 0; c < 2; ++c) {
-                                const int cx = c ^ sw;
-                                const Real ta = (cx ? cj1 : cj0)[oj[cz][cy]];
-                                const Real tb = (cx ? ci1 : ci0)[oi[cz][cy]];
-                                Real *ep = e + cz * Lh * LL + cy * Lh * L + cx * Lh;
-                                *ep = Prec<Real>::add(*ep, Prec<Real>::sub(ta, tb));
-                            }
-                }
-            }
-        } else {
-            // thread -> base column bx < L/2, base rows by0, by0 + rpp, ...
-            const int Lh = L >> 1;
-            const int rpp = kThreads / Lh;
-            // an executed pair applies the second electron's update after the
-            // first one's (each site rounds twice, in the serial order)
-            const int passes = (kPair && cpair) ? 2 : 1;
-#pragma unroll 1
-            for (int pass = 0; pass < passes; ++pass) {
+        for (int pass = 0; pass < (cpair ? 2 : 1); ++pass) {
             const unsigned ui = pass ? cq.k : ci, uj = pass ? cq.l : cj;
-            if (!a.toy && tid < rpp * Lh) {
-                const int bx = tid % Lh, by0 = tid / Lh;
-                const int yi = kPow2 ? (int)(ui >> log2L) : (int)__umulhi(ui, magic);
-                const int yj = kPow2 ? (int)(uj >> log2L) : (int)__umulhi(uj, magic);
-                const int xi = (int)ui - yi * L, xj = (int)uj - yj * L;
-                const int fxj = fold_axis(bx - xj, L), fxi = fold_axis(bx - xi, L);
-                // columns of (x, .) and (x + L/2, .) relative to j and to i
-                const Real *cj0 = tinv + fxj, *cj1 = tinv + (Lh - fxj);
-                const Real *ci0 = tinv + fxi, *ci1 = tinv + (Lh - fxi);
-                const int LhH1 = Lh * H1, LhL = Lh * L;
-                Real *e = eps + by0 * L + bx;
-#pragma unroll 4
-                for (int y = by0; y < Lh; y += rpp, e += rpp * L) {
-                    int fyj, fyi;
-                    if (kPow2) {
-                        const int dj = (y - yj) & (L - 1), di = (y - yi) & (L - 1);
-                        fyj = min(dj, L - dj);
-                        fyi = min(di, L - di);
-                    } else {
-                        fyj = fold_axis(y - yj, L);
-                        fyi = fold_axis(y - yi, L);
-                    }
-                    // rows fold(y - .) and L/2 - fold(y - .) = fold(y + L/2 - .)
-                    const int oj0 = fyj * H1, oj1 = LhH1 - oj0;
-                    const int oi0 = fyi * H1, oi1 = LhH1 - oi0;
-                    const Real a00 = cj0[oj0], b00 = ci0[oi0];
-                    const Real a10 = cj1[oj0], b10 = ci1[oi0];
-                    const Real a01 = cj0[oj1], b01 = ci0[oi1];
-                    const Real a11 = cj1[oj1], b11 = ci1[oi1];
-                    e[0] = Prec<Real>::add(e[0], Prec<Real>::sub(a00, b00));
-                    e[Lh] = Prec<Real>::add(e[Lh], Prec<Real>::sub(a10, b10));
-                    e[LhL] = Prec<Real>::add(e[LhL], Prec<Real>::sub(a01, b01));
-                    e[LhL + Lh] = Prec<Real>::add(e[LhL + Lh], Prec<Real>::sub(a11, b11));
-                }
-            }
-            }
+            if (kDim == 3)
+                update_cubic<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
+                                                    log2L, magic);
+            else
+                update_square<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
+                                                     log2L, magic);
         }
         __syncthreads();
         if (tid == 0) s_c.cyc_upd += (unsigned long long)(clock64() - t1);
