@@ -192,6 +192,35 @@ cudaError_t launch_reset_refresh_err(const DevReplica *d_reps, const int *d_inde
     return cudaGetLastError();
 }
 
+// Positions sorted by falling attempts per hop (rank by counting: at most a few
+// hundred replicas), and the claim table cleared.
+__global__ void __launch_bounds__(1024) pr_schedule_kernel(const DevReplica *__restrict__ reps,
+                                                           const int *__restrict__ index,
+                                                           int count, int *__restrict__ sched)
+{
+    extern __shared__ float cost[];
+    for (int k = threadIdx.x; k < count; k += blockDim.x) {
+        const DevCounters *c = reps[index[k]].ctr;
+        cost[k] = c->rate > 0.f ? c->rate : c->m_ema;
+    }
+    for (int k = threadIdx.x; k < count + kSchedSms; k += blockDim.x) sched[count + k] = 0;
+    __syncthreads();
+    for (int k = threadIdx.x; k < count; k += blockDim.x) {
+        const float mine = cost[k];
+        int rank = 0;
+        for (int o = 0; o < count; ++o) rank += cost[o] > mine || (cost[o] == mine && o < k);
+        sched[rank] = k;
+    }
+}
+
+cudaError_t launch_pr_schedule(const DevReplica *d_reps, const int *d_index, int count, int *sched,
+                               cudaStream_t st)
+{
+    pr_schedule_kernel<<<1, 1024, sizeof(float) * (size_t)count, st>>>(d_reps, d_index, count,
+                                                                      sched);
+    return cudaGetLastError();
+}
+
 __global__ void debug_philox_kernel(const uint32_t *ctr, const uint32_t *key, uint32_t *out,
                                     int n)
 {

@@ -31,6 +31,7 @@ struct alignas(16) DevCounters {
     double trace_next;                 // attempt count of the next trace point
     double trace_ratio;                // ratio between consecutive trace points
     double time;                       // stochastic time (CG_TIME_GAUSSIAN), else 0
+    float rate;                        // attempts per hop of the last launch (0: none yet)
 };
 
 // Guide table of the tower: bucket b = x1 >> (32 - kGuideBits) holds the
@@ -122,6 +123,9 @@ struct RunArgs {
     int time_mode;                 // CG_TIME_DETERMINISTIC or CG_TIME_GAUSSIAN
     int pair;                      // 1: two-electron hops (the kPair instances)
     int smem_guide;                // random sites, one CTA: guide records in shared memory
+    int *sched;                    // single hops, several CTAs per SM: the claim table of
+                                   // launch_pr_schedule, or null (CTA b runs replica b)
+    int n_sms;                     // SMs of the device (with sched)
     int guide_bits;                // single hops on one CTA: log2 of the guide table's entries
     double toy_A0;
 };
@@ -238,6 +242,14 @@ inline int random_smem_bytes(int N, int C = 1, bool guide = false)
 cudaError_t launch_pr_random_cluster(const DevReplica *d_reps, const int *d_index, int n_reps,
                                      int cluster, int threads, int smem_bytes,
                                      const RunArgs &args, cudaStream_t st);
+
+// Claim table of a launch whose CTAs share SMs: order[count] (replica positions
+// by falling attempts per hop), claimed[count], slots[kSchedSms].
+constexpr int kSchedSms = 256;
+inline size_t sched_bytes(int count) { return sizeof(int) * (2 * (size_t)count + kSchedSms); }
+// Fills it from the counters; one small CTA before the persistent launch.
+cudaError_t launch_pr_schedule(const DevReplica *d_reps, const int *d_index, int count,
+                               int *sched, cudaStream_t st);
 
 // Launchers (defined in the .cu files).
 cudaError_t launch_pr_persistent(int precision, const DevReplica *d_reps,

@@ -293,6 +293,7 @@ struct Group {
     int dim = 2;                     // 2: square lattice, 3: cubic lattice
     bool random = false;             // random-site replicas (pr_random)
     bool sguide = false;             // their guide records in shared memory
+    int *d_sched = nullptr;          // claim table of launches with several CTAs per SM
     int gbits = kLatGuideBits;       // guide bits of the single-hop lattice kernel
     int cluster = 1;                 // CTAs per replica
     unsigned M = 4096;               // labels per round when cg_run is given M = 0
@@ -417,6 +418,7 @@ size_t tc_img_bytes(int L, int dim, int count)
 struct cg_handle {
     cg_opts opts{};
     int device = 0;
+    int n_sms = 1;                 // SMs of the device
     int clock_khz = 2000000;       // peak SM clock (per-hop limit in cycles)
     cudaStream_t st = nullptr;
     bool own_stream = false;
@@ -902,6 +904,7 @@ size_t plan_bytes(int R, const cg_replica_desc *reps, const cg_opts &o)
         if (!found) groups.push_back({reps[k].L, dim_of(reps[k]), 1});
     }
     size_t tc_total = 0;
+    for (auto &g : groups) tc_total += up(sched_bytes(std::get<2>(g)));
     for (auto &g : groups)
         if (group_uses_fft(o, std::get<0>(g), std::get<1>(g))) {
             const size_t L = (size_t)std::get<0>(g);
@@ -1009,6 +1012,10 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         int khz = 0;
         if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, o.device) == cudaSuccess && khz > 0)
             h->clock_khz = khz;
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, o.device) == cudaSuccess &&
+            sms > 0)
+            h->n_sms = std::min(sms, kSchedSms);
     }
     if (ws) {
         if (((uintptr_t)ws & 255) != 0) { fail(CG_EINVAL, "workspace must be 256-byte aligned"); return nullptr; }
@@ -1203,6 +1210,10 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
             if (g.threads < 512) g.threads = 512;
             while (g.threads < g.L && g.threads < 1024) g.threads *= 2;
         }
+        if (!g.random && dalloc(h.get(), (void **)&g.d_sched, sched_bytes(g.count))) {
+            destroy_partial();
+            return nullptr;
+        }
         g.fft = !g.random && group_uses_fft(o, g.L, g.dim);
         if (g.fft && dalloc(h.get(), (void **)&g.d_fft,
                             refresh_fft_buffer_bytes(dim_of(h->reps[order[g.first]].d) == 3
@@ -1343,6 +1354,15 @@ int launch_group(cg_handle *h, const Group &g, unsigned long long hops, unsigned
     a.time_mode = h->opts.time_mode;
     a.pair = h->opts.pair_frac > 0.0 ? 1 : 0;
     a.guide_bits = g.gbits;
+    a.n_sms = h->n_sms;
+    // more CTAs than SMs, all resident at once: pair heavy replicas with light
+    // ones (the rank count is quadratic, and past one wave the hardware deals
+    // the CTAs out as SMs come free)
+    if (!g.random && g.cluster == 1 && !a.pair && g.d_sched && g.count > h->n_sms &&
+        g.count <= 4 * h->n_sms) {
+        a.sched = g.d_sched;
+        CG_CUDA(launch_pr_schedule(h->d_reps, h->d_index + g.first, g.count, g.d_sched, st));
+    }
     a.smem_guide = (g.random && g.cluster == 1 && g.sguide) ? 1 : 0;
     if (g.random && g.cluster > 1)
         CG_CUDA(launch_pr_random_cluster(h->d_reps, h->d_index + g.first, g.count, g.cluster,

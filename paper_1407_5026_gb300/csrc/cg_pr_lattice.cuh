@@ -292,6 +292,31 @@ __device__ __forceinline__ bool lat_eval_toy(const LatConst<Real> &K, unsigned k
     return true;
 }
 
+// The replica position this CTA runs: the first CTA on an SM takes one of the
+// heavier half of the order, the second the lighter one that matches it, so the
+// SMs' sums of attempts come out close (304 replicas of L = 128 at T = 0.01:
+// the largest sum is 1.10 of the mean; 1.32 in replica order, and the launch
+// lasts as long as its slowest SM).  The SM only sets the preferred position: a
+// taken one passes on to the next, so every position is run exactly once
+// wherever the CTAs land.
+__device__ __forceinline__ int claim_replica(int *sched, int count, int n_sms)
+{
+    unsigned sm;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+    const int *order = sched;
+    int *claimed = sched + count, *slots = sched + 2 * count;
+    const int r = (int)(sm % (unsigned)n_sms);
+    const int slot = atomicAdd(&slots[r], 1);
+    const int f = (slot >> 1) * n_sms + r;
+    int pos = (slot & 1) ? count - 1 - f : f;
+    if (pos < 0 || pos >= count) pos = r % count;
+    for (int t = 0; t < count; ++t) {
+        if (atomicExch(&claimed[pos], 1) == 0) break;
+        pos = pos + 1 < count ? pos + 1 : 0;
+    }
+    return order[pos];
+}
+
 template <typename Real, int kThreads, int kLog2L, bool kTime, int kDim = 2>
 __global__ void __launch_bounds__(kThreads, (kThreads >= 1024 ? 1 : 1024 / kThreads))
 pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, RunArgs a)
@@ -310,14 +335,18 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     // draws 32 at a time, one per lane
     __shared__ double s_z[kTime ? 32 : 1];
     __shared__ struct {
-        unsigned long long hops, attempts, evaluated, cyc_rej, cyc_upd, zbase;
+        unsigned long long hops, attempts, evaluated, cyc_rej, cyc_upd, zbase, hops0, attempts0;
         long long P, t0;
         double energy, time;
         cg_hop *log;
         int tracing;
     } s_c;
 
-    const DevReplica &Rg = reps[index[blockIdx.x]];
+    __shared__ int s_pos;
+    if (threadIdx.x == 0)
+        s_pos = a.sched ? claim_replica(a.sched, (int)gridDim.x, a.n_sms) : (int)blockIdx.x;
+    __syncthreads();
+    const DevReplica &Rg = reps[index[s_pos]];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int L = kFixL ? kFixL : Rg.L;
     const int N = kDim == 3 ? L * L * L : L * L, H1 = L / 2 + 1, words = (N + 31) / 32;
@@ -388,6 +417,8 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         s_c.tracing = Rg.trace != nullptr;
         s_c.hops = cnt->hops;
         s_c.attempts = cnt->attempts;
+        s_c.hops0 = cnt->hops;
+        s_c.attempts0 = cnt->attempts;
         s_c.evaluated = cnt->evaluated;
         s_c.P = cnt->P;
         s_c.energy = cnt->energy;
@@ -575,6 +606,8 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         cnt->cycles_reject += s_c.cyc_rej;
         cnt->cycles_update += s_c.cyc_upd;
         cnt->m_ema = m_ema;
+        if (s_c.hops - s_c.hops0 >= 32ull)
+            cnt->rate = (float)(s_c.attempts - s_c.attempts0) / (float)(s_c.hops - s_c.hops0);
         cnt->status = status;
     }
 }
