@@ -39,6 +39,8 @@
 // L = 32 to 96 mixed 3.16 -> 1.78; 32^3 2.24 -> 2.06.
 #pragma once
 
+#include <type_traits>
+
 #include "cg_pr_update.cuh"
 
 namespace cg {
@@ -155,7 +157,6 @@ __device__ __forceinline__ float hi_to_f32(int hi, bool &ok)
 }
 
 // What a label's evaluation reads that stays fixed over a launch.
-template <typename Real>
 struct LatConst {
     LatLayout S;
     Cand *cand;                // per warp: its lowest accepting label's proposal
@@ -166,15 +167,27 @@ struct LatConst {
     double T;
 };
 
+// eps_s as binary64.
+template <typename Store>
+__device__ __forceinline__ double lat_energy(int off_eps, unsigned s)
+{
+    if constexpr (std::is_same<Store, long long>::value)
+        return fix_to_double(sm<long long>(off_eps, s));
+    else
+        return (double)sm<Store>(off_eps, s);
+}
+
 // The warp's block of 32 NL labels from kb on: label kb + 32 n + lane, n < NL.
 // Only labels whose theta holds and whose dH is below the cut go through the
 // accept test; the lowest accepting lane writes the warp's candidate and
 // lowers the CTA's best label.  True when the block holds an accept.
-template <typename Real, bool kPow2, int kDim, int NL>
-__device__ __forceinline__ bool lat_eval(const LatConst<Real> &K, unsigned kb,
-                                         const PhiloxPrefix &PP, unsigned *best)
+// Store: the type of the energies in shared memory (long long: binary64 in
+// fixed point).
+template <typename Store, bool kPow2, int kDim, int NL>
+__device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const PhiloxPrefix &PP,
+                                         unsigned *best)
 {
-    constexpr bool kF64 = sizeof(Real) == 8;
+    constexpr bool kF64 = sizeof(Store) == 8, kFix = std::is_same<Store, long long>::value;
     uint32_t x1[NL], x2[NL];
     unsigned si[NL], sj[NL];
     int v[NL];
@@ -211,7 +224,14 @@ __device__ __forceinline__ bool lat_eval(const LatConst<Real> &K, unsigned kb,
         sj[n] = hop_target<kPow2, kDim>(si[n], rc.y, K.L, K.log2L, K.N, K.magic);
         const unsigned wj = sm<unsigned>(K.S.off_occ, sj[n] >> 5);
         const bool theta = on[n] && !((wj >> (sj[n] & 31u)) & 1u);
-        if constexpr (kF64) {
+        if constexpr (kFix) {
+            // the high words: units of 2^-28, cut and rounded by at most
+            // 2^-28 + 2^-22 each below 4; the cut's slack covers it
+            const float fi = __int2float_rn(sm<int>(K.S.off_eps, 2 * si[n] + 1));
+            const float fj = __int2float_rn(sm<int>(K.S.off_eps, 2 * sj[n] + 1));
+            d[n] = fmaf(fj - fi, 0x1p-28f, -cv[n]);
+            cand[n] = theta && d[n] < K.cut;
+        } else if constexpr (kF64) {
             bool oi, oj;
             const float fi = hi_to_f32(sm<int>(K.S.off_eps, 2 * si[n] + 1), oi);
             const float fj = hi_to_f32(sm<int>(K.S.off_eps, 2 * sj[n] + 1), oj);
@@ -233,7 +253,8 @@ __device__ __forceinline__ bool lat_eval(const LatConst<Real> &K, unsigned kb,
         dE[n] = 0.0;
         if constexpr (kF64) {
             acc[n] = cand[n] && metropolis_label<double>(
-                                    sm<double>(K.S.off_eps, si[n]), sm<double>(K.S.off_eps, sj[n]),
+                                    lat_energy<Store>(K.S.off_eps, si[n]),
+                                    lat_energy<Store>(K.S.off_eps, sj[n]),
                                     sm<double>(K.S.off_vr64, v[n]), sm<double>(K.S.off_edx64, v[n]),
                                     cv[n], x2[n], K.T, K.invTf, dE[n]);
         } else {
@@ -266,10 +287,9 @@ __device__ __forceinline__ bool lat_eval(const LatConst<Real> &K, unsigned kb,
 
 // Constant-acceptance test mode: label kb + lane accepts iff its variate is
 // below A0.
-template <typename Real, bool kPow2, int kDim>
-__device__ __forceinline__ bool lat_eval_toy(const LatConst<Real> &K, unsigned kb,
-                                             const PhiloxPrefix &PP, int V, double A0,
-                                             unsigned *best)
+template <bool kPow2, int kDim>
+__device__ __forceinline__ bool lat_eval_toy(const LatConst &K, unsigned kb, const PhiloxPrefix &PP,
+                                             int V, double A0, unsigned *best)
 {
     const unsigned k = kb + (unsigned)K.lane;
     uint32_t x[4];
@@ -323,6 +343,8 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
 {
     constexpr bool kPow2 = kLog2L >= 0;
     constexpr bool kF64 = sizeof(Real) == 8;
+    // the fixed-point form of binary64 energies (binary32 has none)
+    using Fix = typename std::conditional<kF64, long long, Real>::type;
     // L fixed at compile time: 2^kLog2L (kLog2L > 0), or -kLog2L, an even L
     // that is not a power of two (kLog2L < -1); 0 when L is read at run time
     constexpr int kFixL = kLog2L > 0 ? (1 << kLog2L) : (kLog2L < -1 ? -kLog2L : 0);
@@ -437,10 +459,32 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     // variates are at least 2^-24 (ln: -16.64), binary64 ones 2^-33, and the
     // binary64 test calls e^y zero below y = -23.  The binary32 form decides
     // |dH| < 1e-5 apart.  The binary64 bound leaves room for cv's rounding.
-    const float cut = kF64 ? (float)(23.1 * T + (1.0 + fabs(Rg.E) * (double)(L / 2)) * 0x1p-21)
+    const float cut = kF64 ? (float)(23.1 * T + (8.0 + fabs(Rg.E) * (double)(L / 2)) * 0x1p-21)
                            : fmaxf((float)(17.0 * T), 1.1e-5f);
 
-    LatConst<Real> K;
+    // binary64: the energies and the table in fixed point where that is exact
+    // for every one of them (the configurations' W = 1 and 2 at half filling;
+    // a W that is no short binary fraction leaves small energies finer bits)
+    bool fixed = false;
+    if constexpr (kF64) {
+        // from 1024 sites on: below, the update waits for latency, not for the
+        // binary64 pipe, and the decoding costs more (L = 24: 3.4 against 3.2 us
+        // a hop, L = 32: 2.95 and 2.99, L = 64: 2.9 and 4.2)
+        bool ok = N >= 1024;
+        for (int l = tid; ok && l < N; l += kThreads) fix_from_double(sm<double>(lay.off_eps, l), ok);
+        for (int l = tid; ok && l < ntab; l += kThreads)
+            fix_from_double(sm<double>(lay.off_tinv, l), ok);
+        fixed = !__syncthreads_or(!ok);
+        if (fixed) {
+            for (int l = tid; l < N; l += kThreads)
+                sm<long long>(lay.off_eps, l) = fix_from_double(sm<double>(lay.off_eps, l), ok);
+            for (int l = tid; l < ntab; l += kThreads)
+                sm<long long>(lay.off_tinv, l) = fix_from_double(sm<double>(lay.off_tinv, l), ok);
+            __syncthreads();
+        }
+    }
+
+    LatConst K;
     K.S = lay; K.cand = s_cand;
     K.L = L; K.log2L = log2L; K.vbase = vbase; K.vlast = V - 1; K.gshift = gshift;
     K.warp = warp; K.lane = lane;
@@ -490,8 +534,16 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                     if (a.toy) {
                         for (unsigned k = k0; k < kb + C && !hit; k += nw * step)
                             for (unsigned n = 0; n < step && !hit; n += 32u)
-                                hit = lat_eval_toy<Real, kPow2, kDim>(K, k + n, PP, V, a.toy_A0,
+                                hit = lat_eval_toy<kPow2, kDim>(K, k + n, PP, V, a.toy_A0,
                                                                       &s_best[par]);
+                    } else if (kF64 && fixed) {
+                        if (two) {
+#pragma unroll 1
+                            for (unsigned k = k0; k < kb + C && !hit; k += nw * step)
+                                hit = lat_eval<Fix, kPow2, kDim, 2>(K, k, PP, &s_best[par]);
+                        } else {
+                            hit = lat_eval<Fix, kPow2, kDim, 1>(K, k0, PP, &s_best[par]);
+                        }
                     } else if (two) {
 #pragma unroll 1
                         for (unsigned k = k0; k < kb + C && !hit; k += nw * step)
@@ -548,13 +600,37 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         __syncwarp();     // or that warp would run the update twice, once for this lane
 
         // ---- local-energy update (step 3b) ----
-        if (kDim == 3)
-            update_cubic<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L, log2L,
-                                                magic);
-        else
-            update_square<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L, log2L,
-                                                 magic);
-        __syncthreads();
+        unsigned big = 0;
+        if (kF64 && fixed) {
+            if (kDim == 3)
+                update_cubic<Fix, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
+                                                   log2L, magic, big);
+            else
+                update_square<Fix, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
+                                                    log2L, magic, big);
+        } else {
+            if (kDim == 3)
+                update_cubic<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
+                                                    log2L, magic, big);
+            else
+                update_square<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
+                                                     log2L, magic, big);
+        }
+        if (kF64 && fixed) {
+            // an energy has reached 4 in size: back to binary64 before the
+            // next hop could leave the integers' range (one hop moves it by
+            // at most 1)
+            if (__syncthreads_or((int)(big >> 30) & 1)) {
+                for (int l = tid; l < N; l += kThreads)
+                    sm<double>(lay.off_eps, l) = fix_to_double(sm<long long>(lay.off_eps, l));
+                for (int l = tid; l < ntab; l += kThreads)
+                    sm<double>(lay.off_tinv, l) = fix_to_double(sm<long long>(lay.off_tinv, l));
+                fixed = false;
+                __syncthreads();
+            }
+        } else {
+            __syncthreads();
+        }
         // the books of this hop, beside the next hop's first labels
         if (tid == kBook) {
             int cdx, cdy;
@@ -591,7 +667,9 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     // ---- store the replica back ----
     {
         Real *eps_g = reinterpret_cast<Real *>(Rg.eps);
-        for (int l = tid; l < N; l += kThreads) eps_g[l] = sm<Real>(lay.off_eps, l);
+        for (int l = tid; l < N; l += kThreads)
+            eps_g[l] = kF64 && fixed ? (Real)lat_energy<Fix>(lay.off_eps, l)
+                                     : sm<Real>(lay.off_eps, l);
         for (int l = tid; l < words; l += kThreads) Rg.occ[l] = sm<unsigned>(lay.off_occ, l);
     }
     if (tid == kBook) {

@@ -359,13 +359,14 @@ pr_persistent(const DevReplica *__restrict__ reps, const int *__restrict__ index
         // the same sites in both)
 #pragma unroll 1
         for (int pass = 0; pass < (cpair ? 2 : 1); ++pass) {
+            unsigned big = 0;
             const unsigned ui = pass ? cq.k : ci, uj = pass ? cq.l : cj;
             if (kDim == 3)
                 update_cubic<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
-                                                    log2L, magic);
+                                                    log2L, magic, big);
             else
                 update_square<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
-                                                     log2L, magic);
+                                                     log2L, magic, big);
         }
         __syncthreads();
         if (tid == 0) s_c.cyc_upd += (unsigned long long)(clock64() - t1);

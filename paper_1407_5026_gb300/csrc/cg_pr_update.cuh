@@ -18,13 +18,94 @@ __device__ __forceinline__ T &sm(int off, int i = 0)
     return reinterpret_cast<T *>(smem + off)[i];
 }
 
+// ---- binary64 energies in fixed point ----
+// GB300 adds binary64 numbers at 1/64 of its binary32 rate, and the update's
+// two adds per site were 63% of a hop of the L = 128 batch.  An energy that is
+// a multiple of 2^-60 below 4 in size, and the table's 1/r (a multiple of 2^-60
+// for r <= 256), are exact in a 64-bit integer of that unit, so the two
+// roundings of eps + (1/r_lj - 1/r_li) become integer shifts and adds with the
+// same bits: an integer sum, rounded to 53 significant bits, ties to even.
+constexpr int kFixBits = 60;
+
+// Both conversions in integer arithmetic (the binary64 pipe is the slow one).
+__device__ __forceinline__ double fix_to_double(long long e)
+{
+    if (e == 0) return 0.0;
+    const unsigned long long u = (unsigned long long)(e < 0 ? -e : e);
+    const int k = 63 - __clzll((long long)u);          // leading bit; at most 53 follow
+    const unsigned long long m = k > 52 ? u >> (k - 52) : u << (52 - k);
+    const unsigned long long ex = (unsigned long long)(1023 - kFixBits + k) << 52;
+    return __longlong_as_double((long long)((e < 0 ? 1ull << 63 : 0ull) | ex |
+                                            (m & 0x000fffffffffffffull)));
+}
+
+// x as an integer of 2^-60; ok is cleared unless that is exact, sign of zero
+// included, and |x| < 4.
+__device__ __forceinline__ long long fix_from_double(double x, bool &ok)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    if (b == 0) return 0;
+    const int ex = (int)((b >> 52) & 0x7ffull), sh = ex - (1023 - kFixBits + 52);
+    const unsigned long long m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    // ex <= 1024: below 4 (inf and NaN fail here); sh > -53: not below 2^-60
+    // (subnormals and -0 fail here); no bit below 2^-60
+    if (ex > 1024 || sh <= -53 || (sh < 0 && (m & ((1ull << -sh) - 1ull)))) {
+        ok = false;
+        return 0;
+    }
+    const long long e = (long long)(sh >= 0 ? m << sh : m >> -sh);
+    return (b >> 63) ? -e : e;
+}
+
+// s rounded to 53 significant bits, ties to even; big gathers the high words
+// (bit 30 set: |s| >= 2^62).  The position of the leading bit is taken from
+// the one's complement of a negative s: it differs from |s|'s for s = -2^k
+// alone, which either rounding keeps.
+__device__ __forceinline__ long long fix_round53(long long s, unsigned &big)
+{
+    const unsigned lo = (unsigned)s, hi = (unsigned)((unsigned long long)s >> 32);
+    const unsigned h = hi ^ (unsigned)((int)hi >> 31);
+    big |= h;
+    unsigned msb;
+    asm("bfind.u32 %0, %1;" : "=r"(msb) : "r"(h));    // 0xffffffff for h = 0
+    const int sh = max((int)msb - 20, 0);             // bits below the 53 kept (at most 10)
+    const unsigned mask = (1u << sh) - 1u;
+    // half a unit less one, plus the last kept bit (none when nothing is cut)
+    const unsigned r = (mask >> 1) + ((lo >> sh) & mask & 1u);
+    const unsigned long long t = (unsigned long long)s + r;
+    return (long long)((t & 0xffffffff00000000ull) | ((unsigned)t & ~mask));
+}
+
+// e + (a - b), each step rounded to T's precision (fixed point: binary64's).
+__device__ __forceinline__ float site_add(float e, float a, float b, unsigned &)
+{
+    return __fadd_rn(e, __fsub_rn(a, b));
+}
+__device__ __forceinline__ double site_add(double e, double a, double b, unsigned &)
+{
+    return d_add(e, d_sub(a, b));
+}
+__device__ __forceinline__ long long site_add(long long e, long long a, long long b, unsigned &big)
+{
+    long long d = a - b;
+    // |a - b| < 2^53 units (1/128): exact as it is; only sites within about
+    // 11 sqrt(hop length) of the hop need the first rounding
+    if ((unsigned)((unsigned long long)d >> 32) + (1u << 21) >= (1u << 22)) {
+        unsigned none = 0;
+        d = fix_round53(d, none);
+    }
+    return fix_round53(e + d, big);
+}
+
 // Square lattice: thread -> base column bx < L/2, base rows by0, by0 + rpp, ...
 // A base site serves (x, y), (x + L/2, y), (x, y + L/2), (x + L/2, y + L/2): on
 // an even ring fold(d + L/2) = L/2 - fold(d), so one folded offset per axis
 // serves all four.
+// big: see fix_round53 (long long energies).
 template <typename Real, int kThreads, bool kPow2>
-__device__ __forceinline__ void update_square(bool on, int off_eps, int off_tinv, unsigned ui, unsigned uj,
-                                              int L, int log2L, unsigned magic)
+__device__ __forceinline__ void update_square(bool on, int off_eps, int off_tinv, unsigned ui,
+                                              unsigned uj, int L, int log2L, unsigned magic,
+                                              unsigned &big)
 {
     const int tid = threadIdx.x;
     const int Lh = L >> 1, H1 = Lh + 1;
@@ -59,10 +140,10 @@ __device__ __forceinline__ void update_square(bool on, int off_eps, int off_tinv
             const Real a10 = cj1[oj0], b10 = ci1[oi0];
             const Real a01 = cj0[oj1], b01 = ci0[oi1];
             const Real a11 = cj1[oj1], b11 = ci1[oi1];
-            e[0] = Prec<Real>::add(e[0], Prec<Real>::sub(a00, b00));
-            e[Lh] = Prec<Real>::add(e[Lh], Prec<Real>::sub(a10, b10));
-            e[LhL] = Prec<Real>::add(e[LhL], Prec<Real>::sub(a01, b01));
-            e[LhL + Lh] = Prec<Real>::add(e[LhL + Lh], Prec<Real>::sub(a11, b11));
+            e[0] = site_add(e[0], a00, b00, big);
+            e[Lh] = site_add(e[Lh], a10, b10, big);
+            e[LhL] = site_add(e[LhL], a01, b01, big);
+            e[LhL + Lh] = site_add(e[LhL + Lh], a11, b11, big);
         }
     }
 }
@@ -71,8 +152,9 @@ __device__ __forceinline__ void update_square(bool on, int off_eps, int off_tinv
 // p0 + rpp, ...; each base site (x, y, z) < L/2 serves the eight sites
 // (x + a L/2, y + b L/2, z + c L/2), a, b, c in {0, 1}.
 template <typename Real, int kThreads, bool kPow2>
-__device__ __forceinline__ void update_cubic(bool on, int off_eps, int off_tinv, unsigned ui, unsigned uj,
-                                             int L, int log2L, unsigned magic)
+__device__ __forceinline__ void update_cubic(bool on, int off_eps, int off_tinv, unsigned ui,
+                                             unsigned uj, int L, int log2L, unsigned magic,
+                                             unsigned &big)
 {
     const int tid = threadIdx.x;
     const int Lh = L >> 1, H1 = Lh + 1;
@@ -139,7 +221,7 @@ __device__ __forceinline__ void update_cubic(bool on, int off_eps, int off_tinv,
                         const Real ta = (cx ? cj1 : cj0)[oj[cz][cy]];
                         const Real tb = (cx ? ci1 : ci0)[oi[cz][cy]];
                         Real *ep = e + cz * Lh * LL + cy * Lh * L + cx * Lh;
-                        *ep = Prec<Real>::add(*ep, Prec<Real>::sub(ta, tb));
+                        *ep = site_add(*ep, ta, tb, big);
                     }
         }
     }
