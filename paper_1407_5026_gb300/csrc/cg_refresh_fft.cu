@@ -163,6 +163,62 @@ __device__ __forceinline__ int out_pos(int k, const FftArgs &a, bool dif_out)
     return dif_out ? (int)bitrev((unsigned)k, a.log2L) : k;
 }
 
+// eps_new = phi + (v + c) rounded once to binary32, and the change
+// |eps_old - eps_new|, in binary32 pairs: phi is split without the binary64
+// pipe (its word cut to a binary32 plus the 29 bits below), the two large terms
+// add with their exact error (Knuth's two-sum) and the error joins the small
+// ones before the last add.  What is lost is below 2^-45 of the sum.  (In
+// binary64, ten operations per site at 1/64 of the binary32 rate, this step
+// took most of the last pass.)
+__device__ __forceinline__ float refresh_site(double phi, float v, float c, float eps_old,
+                                              float &change)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(phi);
+    const int ex = (int)((b >> 52) & 0x7ffull);
+    const unsigned sign = (unsigned)(b >> 63) << 31;
+    if (ex > 1150) {                                     // no binary32 value: inf, or NaN
+        change = __uint_as_float(0x7f800000u);
+        return __uint_as_float(sign | 0x7f800000u |
+                               (ex == 0x7ff && (b & 0x000fffffffffffffull) ? 1u << 22 : 0u));
+    }
+    float hi = 0.0f, lo = 0.0f;                          // below 2^-74: nothing to add
+    if (ex >= 949) {
+        hi = __uint_as_float(sign | ((unsigned)(ex - 896) << 23) |
+                             ((unsigned)(b >> 29) & 0x7fffffu));
+        lo = __uint2float_rn((unsigned)b & 0x1fffffffu) *
+             __uint_as_float(sign | ((unsigned)(ex - 948) << 23));   // 2^(ex - 1075), signed
+    }
+    const float s = __fadd_rn(hi, v), bb = __fsub_rn(s, hi);
+    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb));
+    const float t = __fadd_rn(err, __fadd_rn(lo, c));
+    change = fabsf(__fsub_rn(__fsub_rn(eps_old, s), t));
+    return __fadd_rn(s, t);
+}
+
+// The block's maxima of the changes of two replicas into their counters.
+__device__ __forceinline__ void record_change(float ca, float cb, bool two, bool count,
+                                              DevCounters *da, DevCounters *db, unsigned *s_err)
+{
+    // non-negative floats order as their bits
+    const unsigned ma = __reduce_max_sync(0xffffffffu, __float_as_uint(ca));
+    const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(cb));
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&s_err[0], ma);
+        atomicMax(&s_err[1], mb);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicMax(&da->max_err_bits,
+                  (unsigned long long)__double_as_longlong((double)__uint_as_float(s_err[0])));
+        if (count) atomicAdd(&da->refreshes, 1ull);
+        if (two) {
+            atomicMax(&db->max_err_bits,
+                      (unsigned long long)__double_as_longlong((double)__uint_as_float(s_err[1])));
+            if (count) atomicAdd(&db->refreshes, 1ull);
+        }
+    }
+}
+
 // One pass over W lines of one pair.  kMode: 0 forward x from the bitmasks;
 // 1 forward (buffer to buffer); 2 forward, product with DFT(g)/N, inverse
 // (the last axis); 3 inverse (buffer to buffer); 4 inverse x into eps.
@@ -171,7 +227,7 @@ template <int kMode>
 __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int axis)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned long long s_err[2];
+    __shared__ unsigned s_err[2];
     const int L = a.L, W = a.W, Ls = L + 1;     // padded line stride (banks)
     const int groups = (int)(gridDim.x / (unsigned)((a.R + 1) / 2));
     const int p = blockIdx.x / groups, g = blockIdx.x - p * groups;
@@ -200,7 +256,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         }
         s[w * Ls + (natural_in ? k : (int)bitrev((unsigned)k, a.log2L))] = v;
     }
-    if (kMode == 4 && threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
+    if (kMode == 4 && threadIdx.x < 2) s_err[threadIdx.x] = 0u;
     __syncthreads();
     // ---- transform ----
     float2 *out = s;                                       // where the result lies
@@ -236,7 +292,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         }
     }
     // ---- store ----
-    double err_a = 0.0, err_b = 0.0;
+    float err_a = 0.0f, err_b = 0.0f;
     if (kMode != 4) {
         for (int e = threadIdx.x; e < n; e += kFftThreads) {
             int w, k;
@@ -255,47 +311,361 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps) + site0;
         // the transforms took n - nu with nu rounded to binary32; sum_t g(s-t)
         // = C0 for every s, so (nu_f - nu) C0 restores the exact nu
-        const double ca = d_mul(d_sub((double)(float)Ra.nu, Ra.nu), Ra.C0);
-        const double cb = d_mul(d_sub((double)(float)Rb.nu, Rb.nu), Rb.C0);
+        const float ca = (float)d_mul(d_sub((double)(float)Ra.nu, Ra.nu), Ra.C0);
+        const float cb = (float)d_mul(d_sub((double)(float)Rb.nu, Rb.nu), Rb.C0);
 #pragma unroll 4
         for (int e = threadIdx.x; e < n; e += kFftThreads) {
             const int w = e / L, k = e - w * L;
             const float2 v = out[w * Ls + out_pos(k, a, true)];
-            const double na = d_add(pa[e], d_add((double)v.x, ca));
-            err_a = fmax(err_a, fabs((double)ea[e] - na));
-            ea[e] = __double2float_rn(na);
+            float ch;
+            ea[e] = refresh_site(pa[e], v.x, ca, ea[e], ch);
+            err_a = fmaxf(err_a, ch);
             if (two) {
-                const double nb = d_add(pb[e], d_add((double)v.y, cb));
-                err_b = fmax(err_b, fabs((double)eb[e] - nb));
-                eb[e] = __double2float_rn(nb);
+                eb[e] = refresh_site(pb[e], v.y, cb, eb[e], ch);
+                err_b = fmaxf(err_b, ch);
             }
         }
+        record_change(err_a, err_b, two, g == 0, Ra.ctr, Rb.ctr, s_err);
     }
-    if (kMode == 4) {
-        // block maxima of the non-negative errors through their bit patterns
-        unsigned long long ba = (unsigned long long)__double_as_longlong(err_a);
-        unsigned long long bb = (unsigned long long)__double_as_longlong(err_b);
+}
+
+// ---------------------------------------------------------------------------
+// Square lattices of L = 16 to 128: the whole refresh of a replica pair in one
+// CTA.  Its L x L complex values stay in shared memory (132 KiB at L = 128)
+// through all the transforms, where the passes above write and read the pair's
+// values through L2 between launches and run a barrier per radix-2 stage.
+//
+// A line of L = R1 8 elements transforms in two steps, in place:
+//     X[c + R1 d] = sum_b W_8^(b d) W_L^(b c) sum_a W_R1^(a c) x[8 a + b]
+// step 1, for each b: an R1-point transform over a (elements 8 a + b) times
+// the twiddles; step 2, for each c: an 8-point transform over b (elements
+// 8 c + b), leaving X[c + R1 d] at 8 c + d.  The inverse takes the steps
+// backwards from that order, so nothing is ever reordered: only the product
+// looks DFT(g) up by the permuted wave numbers, between the forward and the
+// inverse 8-point steps of the y axis, in registers.  Seven sweeps of shared
+// memory in all; the first reads the bitmasks, the last writes eps.
+//
+// Element (y, x) lies at y (L + 1) + (x with its low three bits xored by the
+// next three): columns are contiguous across a half-warp, and the 8-element
+// groups of a line spread over the banks.
+// ---------------------------------------------------------------------------
+
+template <bool kInv>
+__device__ __forceinline__ float2 rot90(float2 v)         // times -i (inverse: i)
+{
+    return kInv ? make_float2(-v.y, v.x) : make_float2(v.y, -v.x);
+}
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// v times (wr, -wi) (inverse: its conjugate)
+template <bool kInv>
+__device__ __forceinline__ float2 ctw(float2 v, float wr, float wi)
+{
+    return cmul(v, make_float2(wr, kInv ? wi : -wi));
+}
+
+template <bool kInv>
+__device__ __forceinline__ void dft2(float2 &a, float2 &b)
+{
+    const float2 t = csub(a, b);
+    a = cadd(a, b);
+    b = t;
+}
+
+template <bool kInv>
+__device__ __forceinline__ void dft3(float2 &a, float2 &b, float2 &c)
+{
+    const float h = 0.8660254037844386f;                  // sqrt(3) / 2
+    const float2 s = cadd(b, c), d = rot90<kInv>(csub(b, c));
+    const float2 t = make_float2(fmaf(-0.5f, s.x, a.x), fmaf(-0.5f, s.y, a.y));
+    a = cadd(a, s);
+    b = make_float2(fmaf(h, d.x, t.x), fmaf(h, d.y, t.y));
+    c = make_float2(fmaf(-h, d.x, t.x), fmaf(-h, d.y, t.y));
+}
+
+template <bool kInv>
+__device__ __forceinline__ void dft4(float2 &a, float2 &b, float2 &c, float2 &d)
+{
+    const float2 t0 = cadd(a, c), t1 = csub(a, c), t2 = cadd(b, d), t3 = rot90<kInv>(csub(b, d));
+    a = cadd(t0, t2);
+    b = cadd(t1, t3);
+    c = csub(t0, t2);
+    d = csub(t1, t3);
+}
+
+// R-point transform of v in registers, natural order in and out.
+template <int R, bool kInv>
+__device__ __forceinline__ void dft(float2 (&v)[R])
+{
+    constexpr float kS = 0.7071067811865476f;             // cos(pi / 4)
+    if constexpr (R == 2) {
+        dft2<kInv>(v[0], v[1]);
+    } else if constexpr (R == 3) {
+        dft3<kInv>(v[0], v[1], v[2]);
+    } else if constexpr (R == 4) {
+        dft4<kInv>(v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 6) {
+        // n = 2 a + b, k = c + 3 d
+        dft3<kInv>(v[0], v[2], v[4]);
+        dft3<kInv>(v[1], v[3], v[5]);
+        v[3] = ctw<kInv>(v[3], 0.5f, 0.8660254037844386f);
+        v[5] = ctw<kInv>(v[5], -0.5f, 0.8660254037844386f);
+        float2 o[6];
 #pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            const unsigned long long xa = __shfl_xor_sync(0xffffffffu, ba, o);
-            const unsigned long long xb = __shfl_xor_sync(0xffffffffu, bb, o);
-            ba = ba > xa ? ba : xa;
-            bb = bb > xb ? bb : xb;
+        for (int c = 0; c < 3; ++c) {
+            o[c] = cadd(v[2 * c], v[2 * c + 1]);
+            o[c + 3] = csub(v[2 * c], v[2 * c + 1]);
         }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(&s_err[0], ba);
-            atomicMax(&s_err[1], bb);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = o[k];
+    } else if constexpr (R == 8) {
+        dft4<kInv>(v[0], v[2], v[4], v[6]);
+        dft4<kInv>(v[1], v[3], v[5], v[7]);
+        v[3] = ctw<kInv>(v[3], kS, kS);
+        v[5] = rot90<kInv>(v[5]);
+        v[7] = ctw<kInv>(v[7], -kS, kS);
+        float2 o[8];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            o[c] = cadd(v[2 * c], v[2 * c + 1]);
+            o[c + 4] = csub(v[2 * c], v[2 * c + 1]);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            atomicMax(&Ra.ctr->max_err_bits, s_err[0]);
-            if (g == 0) atomicAdd(&Ra.ctr->refreshes, 1ull);
-            if (two) {
-                atomicMax(&Rb.ctr->max_err_bits, s_err[1]);
-                if (g == 0) atomicAdd(&Rb.ctr->refreshes, 1ull);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = o[k];
+    } else if constexpr (R == 12 || R == 16) {
+        // n = 4 a + b, k = c + (R/4) d: R/4-point transforms over a, the
+        // twiddles W_R^(b c), 4-point transforms over b
+        constexpr int P = R / 4;
+        constexpr float c16[10] = {1.0f, 0.9238795325112867f, kS, 0.3826834323650898f, 0.0f,
+                                   -0.3826834323650898f, -kS, -0.9238795325112867f, -1.0f,
+                                   -0.9238795325112867f};
+        constexpr float s16[10] = {0.0f, 0.3826834323650898f, kS, 0.9238795325112867f, 1.0f,
+                                   0.9238795325112867f, kS, 0.3826834323650898f, 0.0f,
+                                   -0.3826834323650898f};
+        constexpr float c12[7] = {1.0f, 0.8660254037844386f, 0.5f, 0.0f, -0.5f,
+                                  -0.8660254037844386f, -1.0f};
+        constexpr float s12[7] = {0.0f, 0.5f, 0.8660254037844386f, 1.0f, 0.8660254037844386f, 0.5f,
+                                  0.0f};
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            if constexpr (P == 4)
+                dft4<kInv>(v[b], v[4 + b], v[8 + b], v[12 + b]);
+            else
+                dft3<kInv>(v[b], v[4 + b], v[8 + b]);
+#pragma unroll
+            for (int c = 1; c < P; ++c)
+                if (b) {
+                    const int e = b * c;
+                    v[4 * c + b] = P == 4 ? ctw<kInv>(v[4 * c + b], c16[e % 10], s16[e % 10])
+                                          : ctw<kInv>(v[4 * c + b], c12[e % 7], s12[e % 7]);
+                }
+        }
+        float2 o[R];
+#pragma unroll
+        for (int c = 0; c < P; ++c) {
+            dft4<kInv>(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+#pragma unroll
+            for (int d = 0; d < 4; ++d) o[c + P * d] = v[4 * c + d];
+        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = o[k];
+    }
+}
+
+template <int L>
+constexpr int fft_cta_threads()
+{
+    return L == 128 ? 1024 : L == 96 ? 576 : L == 64 ? 512 : L == 48 ? 288 : L == 32 ? 128 : 64;
+}
+
+template <int L>
+__global__ void __launch_bounds__(fft_cta_threads<L>()) fft_cta_kernel(FftArgs a)
+{
+    constexpr int R1 = L / 8, kT = fft_cta_threads<L>(), Ls = L + 1;
+    extern __shared__ float2 s[];
+    __shared__ unsigned s_err[2];
+    float2 *tw = s + L * Ls;                              // exp(-2 pi i k / L)
+    const int tid = threadIdx.x, p = blockIdx.x;
+    const DevReplica &Ra = a.reps[a.index[2 * p]];
+    const bool two = 2 * p + 1 < a.R;
+    const DevReplica &Rb = a.reps[a.index[two ? 2 * p + 1 : 2 * p]];
+    for (int k = tid; k < L; k += kT) tw[k] = a.tw[k];
+    if (tid < 2) s_err[tid] = 0u;
+    __syncthreads();
+    auto at = [&](int y, int x) -> float2 & {
+        return s[y * Ls + (x & ~7) + ((x ^ (x >> 3)) & 7)];
+    };
+    // rows r and r + 8 share a half-warp: their 8-element runs fall in
+    // opposite halves of the banks
+    auto row_of = [](int r) {
+        return L % 16 ? r : (r & ~15) | ((r & 1) << 3) | ((r >> 1) & 7);
+    };
+    // phi and eps, which the last sweep reads, on their way into L2 meanwhile
+    for (int r = 0; r < (two ? 2 : 1); ++r) {
+        const DevReplica &R = r ? Rb : Ra;
+        const char *f = reinterpret_cast<const char *>(R.phi), *e = reinterpret_cast<const char *>(R.eps);
+        for (int k = tid * 128; k < L * L * 8; k += kT * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f + k));
+        for (int k = tid * 128; k < L * L * 4; k += kT * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(e + k));
+    }
+    // x, step 1, from the bitmasks
+    {
+        const float na = (float)Ra.nu, nb = (float)Rb.nu;
+        for (int it = tid; it < L * 8; it += kT) {
+            const int b = it & 7, y = row_of(it >> 3);
+            float2 v[R1];
+#pragma unroll
+            for (int k = 0; k < R1; ++k) {
+                const unsigned site = (unsigned)(y * L + 8 * k + b);
+                const unsigned wa = __ldg(Ra.occ + (site >> 5)), wb = __ldg(Rb.occ + (site >> 5));
+                v[k] = make_float2((float)((wa >> (site & 31u)) & 1u) - na,
+                                   two ? (float)((wb >> (site & 31u)) & 1u) - nb : 0.0f);
+            }
+            dft<R1, false>(v);
+#pragma unroll
+            for (int c = 0; c < R1; ++c) at(y, 8 * c + b) = c ? cmul(v[c], tw[b * c]) : v[c];
+        }
+    }
+    __syncthreads();
+    // item -> (row, c) of the 8-element groups of the rows
+    auto group_of = [](int it, int &y, int &c) {
+        if (R1 % 8 == 0) {
+            const int rest = it >> 4;
+            c = (it & 7) + 8 * (rest % (R1 / 8));
+            y = 2 * (rest / (R1 / 8)) + ((it >> 3) & 1);
+        } else {
+            c = it % R1;
+            y = it / R1;
+        }
+    };
+    // x, step 2
+    for (int it = tid; it < L * R1; it += kT) {
+        int y, c;
+        group_of(it, y, c);
+        float2 v[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) v[b] = at(y, 8 * c + b);
+        dft<8, false>(v);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) at(y, 8 * c + d) = v[d];
+    }
+    __syncthreads();
+    // y, step 1
+    for (int it = tid; it < L * 8; it += kT) {
+        const int x = it % L, b = it / L;
+        float2 v[R1];
+#pragma unroll
+        for (int k = 0; k < R1; ++k) v[k] = at(8 * k + b, x);
+        dft<R1, false>(v);
+#pragma unroll
+        for (int c = 0; c < R1; ++c) at(8 * c + b, x) = c ? cmul(v[c], tw[b * c]) : v[c];
+    }
+    __syncthreads();
+    // y, step 2, the product with DFT(g)/N, and the inverse's first step
+    for (int it = tid; it < L * R1; it += kT) {
+        const int x = it % L, c = it / L, kx = (x >> 3) + R1 * (x & 7);
+        float2 v[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) v[b] = at(8 * c + b, x);
+        dft<8, false>(v);
+#pragma unroll
+        for (int d = 0; d < 8; ++d) {
+            const float g = __ldg(a.ghat + (c + R1 * d) * L + kx);
+            v[d] = make_float2(v[d].x * g, v[d].y * g);
+        }
+        dft<8, true>(v);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            float2 w = tw[b * c];
+            w.y = -w.y;
+            at(8 * c + b, x) = cmul(v[b], w);
+        }
+    }
+    __syncthreads();
+    // y, the inverse's second step
+    for (int it = tid; it < L * 8; it += kT) {
+        const int x = it % L, b = it / L;
+        float2 v[R1];
+#pragma unroll
+        for (int c = 0; c < R1; ++c) v[c] = at(8 * c + b, x);
+        dft<R1, true>(v);
+#pragma unroll
+        for (int k = 0; k < R1; ++k) at(8 * k + b, x) = v[k];
+    }
+    __syncthreads();
+    // x, the inverse's first step
+    for (int it = tid; it < L * R1; it += kT) {
+        int y, c;
+        group_of(it, y, c);
+        float2 v[8];
+#pragma unroll
+        for (int d = 0; d < 8; ++d) v[d] = at(y, 8 * c + d);
+        dft<8, true>(v);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            float2 w = tw[b * c];
+            w.y = -w.y;
+            at(y, 8 * c + b) = cmul(v[b], w);
+        }
+    }
+    __syncthreads();
+    // x, the inverse's second step, into eps
+    float err_a = 0.0f, err_b = 0.0f;
+    {
+        const double *__restrict__ pa = Ra.phi, *__restrict__ pb = Rb.phi;
+        float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps);
+        float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps);
+        // the transforms took n - nu with nu rounded to binary32; sum_t g(s-t)
+        // = C0 for every s, so (nu_f - nu) C0 restores the exact nu
+        const float ca = (float)d_mul(d_sub((double)(float)Ra.nu, Ra.nu), Ra.C0);
+        const float cb = (float)d_mul(d_sub((double)(float)Rb.nu, Rb.nu), Rb.C0);
+        for (int it = tid; it < L * 8; it += kT) {
+            const int b = it & 7, y = row_of(it >> 3), site = y * L + b;
+            float2 v[R1];
+#pragma unroll
+            for (int c = 0; c < R1; ++c) v[c] = at(y, 8 * c + b);
+            dft<R1, true>(v);
+            // four elements' loads in flight at a time
+            constexpr int kBatch = R1 % 4 == 0 ? 4 : R1 % 3 == 0 ? 3 : 2;
+#pragma unroll
+            for (int k0 = 0; k0 < R1; k0 += kBatch) {
+                double fa[kBatch], fb[kBatch];
+                float oa[kBatch], ob[kBatch];
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    const int e = site + 8 * (k0 + k);
+                    fa[k] = pa[e];
+                    oa[k] = ea[e];
+                    fb[k] = two ? pb[e] : 0.0;
+                    ob[k] = two ? eb[e] : 0.0f;
+                }
+#pragma unroll
+                for (int k = 0; k < kBatch; ++k) {
+                    const int e = site + 8 * (k0 + k);
+                    float ch;
+                    ea[e] = refresh_site(fa[k], v[k0 + k].x, ca, oa[k], ch);
+                    err_a = fmaxf(err_a, ch);
+                    if (two) {
+                        eb[e] = refresh_site(fb[k], v[k0 + k].y, cb, ob[k], ch);
+                        err_b = fmaxf(err_b, ch);
+                    }
+                }
             }
         }
     }
+    record_change(err_a, err_b, two, true, Ra.ctr, Rb.ctr, s_err);
+}
+
+template <int L>
+cudaError_t launch_cta(const FftArgs &a, int pairs, cudaStream_t st)
+{
+    const int smem = (L * (L + 1) + L) * (int)sizeof(float2);
+    const cudaError_t e = cudaFuncSetAttribute(fft_cta_kernel<L>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e) return e;
+    fft_cta_kernel<L><<<pairs, fft_cta_threads<L>(), smem, st>>>(a);
+    return cudaGetLastError();
 }
 
 template <int kMode>
@@ -352,6 +722,16 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
     const int groups = lines / a.W;
     cudaError_t e;
     if (dim == 2) {
+        // a pair per CTA where its values fit shared memory
+        switch (L) {
+        case 16: return launch_cta<16>(a, pairs, st);
+        case 24: return launch_cta<24>(a, pairs, st);
+        case 32: return launch_cta<32>(a, pairs, st);
+        case 48: return launch_cta<48>(a, pairs, st);
+        case 64: return launch_cta<64>(a, pairs, st);
+        case 96: return launch_cta<96>(a, pairs, st);
+        case 128: return launch_cta<128>(a, pairs, st);
+        }
         if ((e = launch_pass<0>(a, 0, pairs, groups, st))) return e;
         if ((e = launch_pass<2>(a, 1, pairs, groups, st))) return e;
         return launch_pass<4>(a, 0, pairs, groups, st);
