@@ -103,12 +103,15 @@ cudaError_t launch_eps_init(const DevReplica *d_rep, int N, int ntab, int words,
     return cudaGetLastError();
 }
 
+// blockIdx.y: the replica's position in the group (one launch for all of them:
+// a replica alone fills N/256 CTAs, 7 at L = 42)
 template <bool kTabGlobal>
-__global__ void __launch_bounds__(256) refresh_fp64_kernel(const DevReplica *__restrict__ rp)
+__global__ void __launch_bounds__(256) refresh_fp64_kernel(const DevReplica *__restrict__ reps,
+                                                           const int *__restrict__ index)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ unsigned long long s_max;
-    const DevReplica &R = *rp;
+    const DevReplica &R = reps[index[blockIdx.y]];
     const int L = R.L, N = R.N, H1 = R.H1, words = R.words, ntab = tab_entries(R);
     const int Lz = R.dim == 3 ? L : 1;
     double *tab_s = reinterpret_cast<double *>(sm);
@@ -158,9 +161,15 @@ __global__ void __launch_bounds__(256) refresh_fp64_kernel(const DevReplica *__r
     }
 }
 
-cudaError_t launch_refresh_fp64(const DevReplica *d_rep, int N, int ntab, int words,
-                                cudaStream_t st)
+cudaError_t launch_refresh_fp64(const DevReplica *d_reps, const int *d_index, int count, int N,
+                                int ntab, int words, cudaStream_t st)
 {
+    // grid.y is at most 65535
+    for (; count > 65535; count -= 65535, d_index += 65535) {
+        const cudaError_t e = launch_refresh_fp64(d_reps, d_index, 65535, N, ntab, words, st);
+        if (e) return e;
+    }
+    const dim3 grid((unsigned)((N + 255) / 256), (unsigned)count);
     const int smem = cg_align16(ntab * 8) + words * 4;
     cudaError_t e;
     if (smem > kAuxSmemLimit) {
@@ -168,13 +177,13 @@ cudaError_t launch_refresh_fp64(const DevReplica *d_rep, int N, int ntab, int wo
         if ((e = cudaFuncSetAttribute(refresh_fp64_kernel<true>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, sm2)))
             return e;
-        refresh_fp64_kernel<true><<<(N + 255) / 256, 256, sm2, st>>>(d_rep);
+        refresh_fp64_kernel<true><<<grid, 256, sm2, st>>>(d_reps, d_index);
         return cudaGetLastError();
     }
     if ((e = cudaFuncSetAttribute(refresh_fp64_kernel<false>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem)))
         return e;
-    refresh_fp64_kernel<false><<<(N + 255) / 256, 256, smem, st>>>(d_rep);
+    refresh_fp64_kernel<false><<<grid, 256, smem, st>>>(d_reps, d_index);
     return cudaGetLastError();
 }
 

@@ -292,8 +292,8 @@ cudaError_t launch_pr_cluster_pair(int precision, const DevReplica *d_reps, cons
                                    const RunArgs &args, cudaStream_t st, int L, int dim);
 cudaError_t launch_eps_init(const DevReplica *d_rep, int N, int tab_entries, int words,
                             int precision, cudaStream_t st);
-cudaError_t launch_refresh_fp64(const DevReplica *d_rep, int N, int tab_entries, int words,
-                                cudaStream_t st);
+cudaError_t launch_refresh_fp64(const DevReplica *d_reps, const int *d_index, int count, int N,
+                                int tab_entries, int words, cudaStream_t st);
 cudaError_t launch_debug_philox(const uint32_t *ctr, const uint32_t *key,
                                 uint32_t *out, int n, cudaStream_t st);
 cudaError_t launch_debug_exp(const double *x, double *out, int n, cudaStream_t st);

@@ -1318,11 +1318,10 @@ int refresh_group(cg_handle *h, const Group &g, cudaStream_t st)
                                       g.d_img, g.d_err, st));
         }
     } else {
-        for (int k = g.first; k < g.first + g.count; ++k) {
-            const int ri = h->order[k];
-            const Rep &r = h->reps[ri];
-            CG_CUDA(launch_refresh_fp64(h->d_reps + ri, r.N, (int)r.tab->t64.size(), r.words, st));
-        }
+        // replicas of one group share L and dimension, and so these sizes
+        const Rep &r = h->reps[h->order[g.first]];
+        CG_CUDA(launch_refresh_fp64(h->d_reps, h->d_index + g.first, g.count, r.N,
+                                    (int)r.tab->t64.size(), r.words, st));
     }
     return CG_OK;
 }

@@ -145,3 +145,20 @@ def test_transform_refresh_of_a_pair(B, L, R):
             assert abs(o["max_eps_err_last_refresh"] - np.abs(before[k] - eps).max()) <= 2.5e-7
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("L,dim,R", [(18, 2, 7), (42, 2, 5), (10, 3, 3)])
+def test_binary64_refresh_of_a_group(B, L, dim, R):
+    reps = [dict(BASE, L=L, r_max=3, seed=s, replica=s, dim=dim) for s in range(R)]
+    s = B.System(reps, precision=B.CG_FP32, refresh_kind=B.CG_REFRESH_FP64)
+    try:
+        assert s.run(60, 512) == B.CG_OK
+        B.cg_refresh(s.h)
+        for k in range(R):
+            n, eps, phi, _ = s.state(k)
+            exact = (ref.site_energies_fft3(n, phi, 0.5, L) if dim == 3
+                     else ref.site_energies_fft(n, phi, 0.5, L))
+            assert np.abs(eps - exact).max() <= 2.5e-7
+            assert s.observables(k)["refreshes"] == 1
+    finally:
+        s.close()
