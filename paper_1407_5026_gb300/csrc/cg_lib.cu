@@ -548,9 +548,22 @@ int persistent_smem(const Rep &r, int precision, int cluster = 1)
     const int rb = precision == CG_FP64 ? 8 : 4;
     const bool r2 = dim_of(r.d) == 3 && cluster > 1 && !r.pair;
     const int ntab = r2 ? (int)r.tab->r2_64.size() : (int)r.tab->t64.size();
-    if (cluster == 1 && !r.pair)
+    if (cluster == 1)
         return lat_layout(r.N, ntab, r.tab->V, r.words, rb, guide_bits_of(r, precision)).total;
     return smem_layout(r.N / cluster, ntab, r.tab->V, r.words, rb).total;
+}
+
+// Whether a replica runs on c CTAs: by the layout of the cluster kernels' pair
+// form, which is never the smaller one, so that the guide's size decides neither
+// which lattices are taken nor on how many CTAs.
+bool fits_ctas(const Rep &r, int precision, int c, int budget)
+{
+    if (persistent_smem(r, precision, c) > budget) return false;
+    if (r.random) return true;
+    const bool r2 = dim_of(r.d) == 3 && c > 1 && !r.pair;
+    const int ntab = r2 ? (int)r.tab->r2_64.size() : (int)r.tab->t64.size();
+    return smem_layout(r.N / c, ntab, r.tab->V, r.words, precision == CG_FP64 ? 8 : 4).total <=
+           budget;
 }
 
 // L must be a multiple of this for a cluster of c CTAs: c on the cubic
@@ -575,13 +588,13 @@ int choose_cluster(const cg_opts &o, const Rep &r, int optin)
     if (o.cluster_size > 1) {
         const int c = o.cluster_size;
         if ((c == 2 || c == 4 || c == 8) && r.d.L % cluster_rows_unit(r.d, c) == 0 &&
-            (r.random || r.d.L >= 16) && persistent_smem(r, o.precision, c) <= budget)
+            (r.random || r.d.L >= 16) && fits_ctas(r, o.precision, c, budget))
             return c;
         return 0;
     }
-    if (persistent_smem(r, o.precision, 1) <= budget) return 1;
+    if (fits_ctas(r, o.precision, 1, budget)) return 1;
     for (int c = 2; c <= 8; c *= 2)
-        if (r.d.L % cluster_rows_unit(r.d, c) == 0 && persistent_smem(r, o.precision, c) <= budget)
+        if (r.d.L % cluster_rows_unit(r.d, c) == 0 && fits_ctas(r, o.precision, c, budget))
             return c;
     return 0;
 }
@@ -1357,7 +1370,7 @@ int launch_group(cg_handle *h, const Group &g, unsigned long long hops, unsigned
     // more CTAs than SMs, all resident at once: pair heavy replicas with light
     // ones (the rank count is quadratic, and past one wave the hardware deals
     // the CTAs out as SMs come free)
-    if (!g.random && g.cluster == 1 && !a.pair && g.d_sched && g.count > h->n_sms &&
+    if (!g.random && g.cluster == 1 && g.d_sched && g.count > h->n_sms &&
         g.count <= 4 * h->n_sms) {
         a.sched = g.d_sched;
         CG_CUDA(launch_pr_schedule(h->d_reps, h->d_index + g.first, g.count, g.d_sched, st));
@@ -1848,9 +1861,13 @@ static std::vector<std::pair<int, int>> cluster_candidates(const cg_handle *h, c
     for (int c = 1; c <= 8; c *= 2) {
         if (c > 1 && !g.random && (g.L % (g.dim == 3 ? c : 2 * c) != 0 || g.L < 16)) continue;
         int sm = 0;
-        for (int k = 0; k < g.count; ++k)
-            sm = std::max(sm, persistent_smem(h->reps[h->order[g.first + k]], h->opts.precision, c));
-        if (sm <= budget) out.push_back({c, sm});
+        bool fits = true;
+        for (int k = 0; k < g.count; ++k) {
+            const Rep &r = h->reps[h->order[g.first + k]];
+            sm = std::max(sm, persistent_smem(r, h->opts.precision, c));
+            fits = fits && fits_ctas(r, h->opts.precision, c, budget);
+        }
+        if (fits) out.push_back({c, sm});
     }
     return out;
 }

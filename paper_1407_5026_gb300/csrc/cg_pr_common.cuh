@@ -373,18 +373,30 @@ __device__ __forceinline__ T tinv_sites(const T *tab, unsigned a, unsigned b, in
 // dH of the pair i -> j, k -> l in binary64, in the serial chain's order:
 // (dH1 + dH2) + ((1/r_lj - 1/r_li) - (1/r_kj - 1/r_ki)), each dH as R9.
 template <bool kPow2, int kDim = 2>
+__device__ __forceinline__ double pair_dE64_vals(const double *tab64, double ei, double ej,
+                                                 double ek, double el, double vr1, double edx1,
+                                                 double vr2, double edx2, unsigned i, unsigned j,
+                                                 unsigned k, unsigned l, int L, int log2L,
+                                                 unsigned magic, int H1)
+{
+    const double d1 = d_sub(d_sub(d_sub(ej, ei), vr1), edx1);
+    const double d2 = d_sub(d_sub(d_sub(el, ek), vr2), edx2);
+    const double tlj = tinv_sites<double, kPow2, kDim>(tab64, l, j, L, log2L, magic, H1);
+    const double tli = tinv_sites<double, kPow2, kDim>(tab64, l, i, L, log2L, magic, H1);
+    const double tkj = tinv_sites<double, kPow2, kDim>(tab64, k, j, L, log2L, magic, H1);
+    const double tki = tinv_sites<double, kPow2, kDim>(tab64, k, i, L, log2L, magic, H1);
+    return d_add(d_add(d1, d2), d_sub(d_sub(tlj, tli), d_sub(tkj, tki)));
+}
+
+template <bool kPow2, int kDim = 2>
 __device__ __forceinline__ double pair_dE64(const Shared &S, const double *tab64, double ei,
                                             double ej, double ek, double el, const Prop &p,
                                             const PairProp &q, int L, int log2L,
                                             unsigned magic, int H1)
 {
-    const double d1 = d_sub(d_sub(d_sub(ej, ei), S.vr64[p.v]), S.edx64[p.v]);
-    const double d2 = d_sub(d_sub(d_sub(el, ek), S.vr64[q.v2]), S.edx64[q.v2]);
-    const double tlj = tinv_sites<double, kPow2, kDim>(tab64, q.l, p.j, L, log2L, magic, H1);
-    const double tli = tinv_sites<double, kPow2, kDim>(tab64, q.l, p.i, L, log2L, magic, H1);
-    const double tkj = tinv_sites<double, kPow2, kDim>(tab64, q.k, p.j, L, log2L, magic, H1);
-    const double tki = tinv_sites<double, kPow2, kDim>(tab64, q.k, p.i, L, log2L, magic, H1);
-    return d_add(d_add(d1, d2), d_sub(d_sub(tlj, tli), d_sub(tkj, tki)));
+    return pair_dE64_vals<kPow2, kDim>(tab64, ei, ej, ek, el, S.vr64[p.v], S.edx64[p.v],
+                                       S.vr64[q.v2], S.edx64[q.v2], p.i, p.j, q.k, q.l, L, log2L,
+                                       magic, H1);
 }
 
 // Step 2 for a pair whose theta holds.  Binary64: exact dH.  Binary32: the

@@ -1,7 +1,7 @@
 // cg_pr_kernel3d_pair.cu -- launches of the persistent parallel-rejection
-// kernel (cg_pr_persistent.cuh) with two-electron hops on the L x L x L cubic
+// kernel (cg_pr_lattice.cuh) with two-electron hops on the L x L x L cubic
 // lattice, L known at run time, both clocks.
-#include "cg_pr_persistent.cuh"
+#include "cg_pr_lattice.cuh"
 
 namespace cg {
 
@@ -10,10 +10,10 @@ static void launch3p_tt(const DevReplica *d_reps, const int *d_index, int n_ctas
                         const RunArgs &args, cudaStream_t st, int L)
 {
     if ((L & (L - 1)) == 0)
-        pr_persistent<Real, kThreads, 0, kTime, 3>
+        pr_lattice<Real, kThreads, 0, kTime, 3, true>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     else
-        pr_persistent<Real, kThreads, -1, kTime, 3>
+        pr_lattice<Real, kThreads, -1, kTime, 3, true>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
 }
 
@@ -31,10 +31,10 @@ static cudaError_t launch3p_t(const DevReplica *d_reps, const int *d_index, int 
 template <typename Real, int kThreads>
 static cudaError_t set3p_one(int bytes)
 {
-    const void *k[4] = {(const void *)pr_persistent<Real, kThreads, 0, false, 3>,
-                        (const void *)pr_persistent<Real, kThreads, -1, false, 3>,
-                        (const void *)pr_persistent<Real, kThreads, 0, true, 3>,
-                        (const void *)pr_persistent<Real, kThreads, -1, true, 3>};
+    const void *k[4] = {(const void *)pr_lattice<Real, kThreads, 0, false, 3, true>,
+                        (const void *)pr_lattice<Real, kThreads, -1, false, 3, true>,
+                        (const void *)pr_lattice<Real, kThreads, 0, true, 3, true>,
+                        (const void *)pr_lattice<Real, kThreads, -1, true, 3, true>};
     for (const void *f : k) {
         const cudaError_t e =
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -1,8 +1,8 @@
 // cg_pr_kernel_pair.cu -- launches of the persistent parallel-rejection kernel
-// (cg_pr_persistent.cuh) with two-electron hops on the L x L square lattice,
+// (cg_pr_lattice.cuh) with two-electron hops on the L x L square lattice,
 // L known at run time (a power of two or any even L), deterministic clock
 // (the stochastic-clock instances are in cg_pr_kernel_pair_time.cu).
-#include "cg_pr_persistent.cuh"
+#include "cg_pr_lattice.cuh"
 
 namespace cg {
 
@@ -13,11 +13,14 @@ static cudaError_t launch_pair_t(const DevReplica *d_reps, const int *d_index, i
     if (args.time_mode)
         return launch_pr_persistent_pair_time(sizeof(Real) == 8 ? CG_FP64 : CG_FP32, d_reps,
                                               d_index, n_ctas, kThreads, smem_bytes, args, st, L);
-    if ((L & (L - 1)) == 0)
-        pr_persistent<Real, kThreads, 0, false, 2>
+    if (L == 64)
+        pr_lattice<Real, kThreads, 6, false, 2, true>
+            <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
+    else if ((L & (L - 1)) == 0)
+        pr_lattice<Real, kThreads, 0, false, 2, true>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     else
-        pr_persistent<Real, kThreads, -1, false, 2>
+        pr_lattice<Real, kThreads, -1, false, 2, true>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     return cudaGetLastError();
 }
@@ -25,8 +28,8 @@ static cudaError_t launch_pair_t(const DevReplica *d_reps, const int *d_index, i
 template <typename Real, int kThreads>
 static cudaError_t set_pair_one(int bytes)
 {
-    const void *k[2] = {(const void *)pr_persistent<Real, kThreads, 0, false, 2>,
-                        (const void *)pr_persistent<Real, kThreads, -1, false, 2>};
+    const void *k[3] = {(const void *)pr_lattice<Real, kThreads, 6, false, 2, true>,(const void *)pr_lattice<Real, kThreads, 0, false, 2, true>,
+                        (const void *)pr_lattice<Real, kThreads, -1, false, 2, true>};
     for (const void *f : k) {
         const cudaError_t e =
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -1,8 +1,8 @@
 // cg_pr_kernel_pair_time.cu -- the two-electron-hop instances of the
-// persistent parallel-rejection kernel (cg_pr_persistent.cuh) with the
+// persistent parallel-rejection kernel (cg_pr_lattice.cuh) with the
 // stochastic clock of step 3c (CG_TIME_GAUSSIAN), square lattice, L known at
 // run time.
-#include "cg_pr_persistent.cuh"
+#include "cg_pr_lattice.cuh"
 
 namespace cg {
 
@@ -11,10 +11,10 @@ static cudaError_t launch_pt(const DevReplica *d_reps, const int *d_index, int n
                              int smem_bytes, const RunArgs &args, cudaStream_t st, int L)
 {
     if ((L & (L - 1)) == 0)
-        pr_persistent<Real, kThreads, 0, true, 2>
+        pr_lattice<Real, kThreads, 0, true, 2, true>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     else
-        pr_persistent<Real, kThreads, -1, true, 2>
+        pr_lattice<Real, kThreads, -1, true, 2, true>
             <<<n_ctas, kThreads, smem_bytes, st>>>(d_reps, d_index, args);
     return cudaGetLastError();
 }
@@ -22,8 +22,8 @@ static cudaError_t launch_pt(const DevReplica *d_reps, const int *d_index, int n
 template <typename Real, int kThreads>
 static cudaError_t set_pt_one(int bytes)
 {
-    const void *k[2] = {(const void *)pr_persistent<Real, kThreads, 0, true, 2>,
-                        (const void *)pr_persistent<Real, kThreads, -1, true, 2>};
+    const void *k[2] = {(const void *)pr_lattice<Real, kThreads, 0, true, 2, true>,
+                        (const void *)pr_lattice<Real, kThreads, -1, true, 2, true>};
     for (const void *f : k) {
         const cudaError_t e =
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);

@@ -1,6 +1,7 @@
-// cg_pr_lattice.cuh -- the persistent parallel-rejection kernel for single
-// hops on one CTA per replica (square lattice: cg_pr_kernel.cu, cubic
-// lattice: cg_pr_kernel3d.cu).  Two-electron hops run on cg_pr_persistent.cuh.
+// cg_pr_lattice.cuh -- the persistent parallel-rejection kernel with one CTA
+// per replica (square lattice: cg_pr_kernel.cu, cubic lattice:
+// cg_pr_kernel3d.cu; with two-electron hops: cg_pr_kernel_pair.cu,
+// cg_pr_kernel_pair_time.cu and cg_pr_kernel3d_pair.cu).
 //
 // One CTA runs one disorder replica for a whole launch.  Its local energies
 // eps (N values), the folded minimum-image 1/r table, the occupation bitmask
@@ -48,13 +49,18 @@ namespace cg {
 // b of the chunk rule C ~ sqrt(m b)
 constexpr float kLatChunkCost = 256.0f;
 
-// Hop vector dx of a packed displacement word (see rec below): with a
-// power-of-two L the low field is dx mod L, otherwise dx | dy << 16 (square)
-// or 10-bit fields (cubic).
+// Hop vector of a packed displacement word (see rec below): with a
+// power-of-two L the fields are dx mod L, dy mod L (and dz mod L), otherwise
+// dx | dy << 16 (square) or 10-bit fields (cubic).
 template <bool kPow2, int kDim>
-__device__ __forceinline__ void vec_fields(unsigned w, int L, int log2L, int &dx, int &dy)
+__device__ __forceinline__ void vec_fields(unsigned w, int L, int log2L, int &dx, int &dy, int &dz)
 {
+    dz = 0;
     if (kPow2) {
+        if (kDim == 3) {
+            dz = (int)(w >> (2 * log2L));
+            dz -= (dz >= (L >> 1)) ? L : 0;
+        }
         dx = (int)(w & (unsigned)(L - 1));
         dx -= (dx >= (L >> 1)) ? L : 0;
         dy = (int)((w >> log2L) & (unsigned)(L - 1));
@@ -62,25 +68,33 @@ __device__ __forceinline__ void vec_fields(unsigned w, int L, int log2L, int &dx
     } else if (kDim == 3) {
         dx = (int)(w << 22) >> 22;
         dy = (int)(w << 12) >> 22;
+        dz = (int)w >> 20;
     } else {
         dx = (int)(short)(w & 0xffffu);
         dy = (int)w >> 16;
     }
 }
 
-// The displacement word of a packed hop vector dxy (cg_internal.h).
+// The displacement word of (dx, dy, dz), and of a packed hop vector dxy
+// (cg_internal.h).
+template <bool kPow2, int kDim>
+__device__ __forceinline__ unsigned vec_word(int dx, int dy, int dz, int L, int log2L)
+{
+    if (!kPow2)
+        return kDim == 3 ? ((unsigned)dx & 0x3ffu) | (((unsigned)dy & 0x3ffu) << 10) |
+                               ((unsigned)dz << 20)
+                         : ((unsigned)dx & 0xffffu) | ((unsigned)dy << 16);
+    const unsigned m = (unsigned)(L - 1);
+    const unsigned yx = (((unsigned)dy & m) << log2L) | ((unsigned)dx & m);
+    return kDim == 3 ? (((unsigned)dz & m) << (2 * log2L)) | yx : yx;
+}
+
 template <bool kPow2, int kDim>
 __device__ __forceinline__ unsigned vec_word(int dxy, int L, int log2L)
 {
-    if (!kPow2) return (unsigned)dxy;
-    const unsigned m = (unsigned)(L - 1);
-    if (kDim == 3) {
-        const unsigned dx = (unsigned)((dxy << 22) >> 22) & m, dy = (unsigned)((dxy << 12) >> 22) & m,
-                       dz = (unsigned)(dxy >> 20) & m;
-        return (((dz << log2L) | dy) << log2L) | dx;
-    }
-    const unsigned dx = (unsigned)(int)(short)(dxy & 0xffff) & m, dy = (unsigned)(dxy >> 16) & m;
-    return (dy << log2L) | dx;
+    if (kDim == 3)
+        return vec_word<kPow2, kDim>((dxy << 22) >> 22, (dxy << 12) >> 22, dxy >> 20, L, log2L);
+    return vec_word<kPow2, kDim>((int)(short)(dxy & 0xffff), dxy >> 16, 0, L, log2L);
 }
 
 // Site i displaced by the vector word w.  Power-of-two L: i + w is right in
@@ -165,7 +179,62 @@ struct LatConst {
     uint32_t key0, key1;
     float cut, invTf;
     double T;
+    // two-electron hops
+    PairProp *pcand;           // per warp: the second electron of its candidate
+    unsigned pair_T;
+    int pair_R;
+    const double *tab64;       // the binary64 table in global memory
 };
+
+// Two-electron hops: a label whose fourth word is below pair_T proposes a pair.
+// From the Philox block of counter (k, r lo, r hi | 2^31, replica), y0, y2 (and
+// y3 on the cubic lattice) give the offset e of the second electron k = i + e,
+// each axis floor(y W / 2^32) - R with W = 2R + 1, and y1 its hop vector d2 by
+// the same tower, l = k + d2.  theta also needs n_k = 1, n_l = 0,
+// 0 < |e|^2 <= R^2 and 0 < |e'|^2 <= R^2 for the reverse offset
+// e' = e + d2 - d1, so that a pair and its reverse are proposed with the same
+// probability.  w1: the displacement word of the first electron's hop.
+struct LatPair {
+    unsigned k, l, w2;
+    int v2;
+    float cv2;
+    bool ok;
+};
+
+template <bool kPow2, int kDim>
+__device__ __forceinline__ LatPair lat_pair(const LatConst &K, unsigned label,
+                                            const PhiloxPrefix &PP2, unsigned i, unsigned w1)
+{
+    LatPair q;
+    uint32_t y[4];
+    philox_finish(label, PP2, K.key0, K.key1, y);
+    const int R = K.pair_R;
+    const unsigned W = (unsigned)(2 * R + 1);
+    const int ex = (int)__umulhi(y[0], W) - R, ey = (int)__umulhi(y[2], W) - R;
+    const int ez = kDim == 3 ? (int)__umulhi(y[3], W) - R : 0;
+    const int g = (int)sm<unsigned char>(K.S.off_guide, y[1] >> K.gshift);
+    q.v2 = g + K.vbase;
+    bool live = true;
+    if (g == 255) {
+        q.v2 = K.vlast;
+        live = lat_search(K.S, y[1], K.thr_last, q.v2);
+    }
+    const uint2 rc = sm<uint2>(K.S.off_rec, q.v2);
+    q.cv2 = __uint_as_float(rc.x);
+    q.w2 = rc.y;
+    int dx1, dy1, dz1, dx2, dy2, dz2;
+    vec_fields<kPow2, kDim>(w1, K.L, K.log2L, dx1, dy1, dz1);
+    vec_fields<kPow2, kDim>(q.w2, K.L, K.log2L, dx2, dy2, dz2);
+    q.k = hop_target<kPow2, kDim>(i, vec_word<kPow2, kDim>(ex, ey, ez, K.L, K.log2L), K.L, K.log2L,
+                                  K.N, K.magic);
+    q.l = hop_target<kPow2, kDim>(q.k, q.w2, K.L, K.log2L, K.N, K.magic);
+    const int fx = ex + dx2 - dx1, fy = ey + dy2 - dy1, fz = ez + dz2 - dz1;
+    const int e2 = ex * ex + ey * ey + ez * ez, f2 = fx * fx + fy * fy + fz * fz, R2 = R * R;
+    const unsigned wk = sm<unsigned>(K.S.off_occ, q.k >> 5), wl = sm<unsigned>(K.S.off_occ, q.l >> 5);
+    q.ok = live && e2 > 0 && e2 <= R2 && f2 > 0 && f2 <= R2 && ((wk >> (q.k & 31u)) & 1u) &&
+           !((wl >> (q.l & 31u)) & 1u);
+    return q;
+}
 
 // eps_s as binary64.
 template <typename Store>
@@ -177,22 +246,59 @@ __device__ __forceinline__ double lat_energy(int off_eps, unsigned s)
         return (double)sm<Store>(off_eps, s);
 }
 
+// Step 2 for a pair whose theta holds; dE is its dH in binary64 (binary32
+// energies: from the widened ones, as for the executed pair).  The binary32
+// form decides by the same sum in binary32, and near ties (|dH| < 1e-5) by the
+// binary64 one.
+template <typename Store, bool kPow2, int kDim>
+__device__ __forceinline__ bool lat_accept_pair(const LatConst &K, const LatPair &q, unsigned i,
+                                                unsigned j, int v, float cv, uint32_t x2,
+                                                double &dE)
+{
+    const int H1 = K.L / 2 + 1;
+    // -1: undecided (binary64 decides), else the binary32 form's decision
+    int take = -1;
+    if constexpr (sizeof(Store) == 4) {
+        const float *t32 = &sm<float>(K.S.off_tinv);
+        const float ei = sm<float>(K.S.off_eps, i), ej = sm<float>(K.S.off_eps, j);
+        const float ek = sm<float>(K.S.off_eps, q.k), el = sm<float>(K.S.off_eps, q.l);
+        const float d1 = __fsub_rn(__fsub_rn(ej, ei), cv);
+        const float d2 = __fsub_rn(__fsub_rn(el, ek), q.cv2);
+        const float cr = __fsub_rn(
+            __fsub_rn(tinv_sites<float, kPow2, kDim>(t32, q.l, j, K.L, K.log2L, K.magic, H1),
+                      tinv_sites<float, kPow2, kDim>(t32, q.l, i, K.L, K.log2L, K.magic, H1)),
+            __fsub_rn(tinv_sites<float, kPow2, kDim>(t32, q.k, j, K.L, K.log2L, K.magic, H1),
+                      tinv_sites<float, kPow2, kDim>(t32, q.k, i, K.L, K.log2L, K.magic, H1)));
+        const float dEf = __fadd_rn(__fadd_rn(d1, d2), cr);
+        if (!(fabsf(dEf) < 1e-5f))
+            take = dEf <= 0.0f ||
+                   (float)(x2 >> 9) < __fmaf_rn(__expf(-dEf * K.invTf), 0x1p23f, -0.5f);
+        if (take == 0) return false;
+    }
+    dE = pair_dE64_vals<kPow2, kDim>(
+        K.tab64, lat_energy<Store>(K.S.off_eps, i), lat_energy<Store>(K.S.off_eps, j),
+        lat_energy<Store>(K.S.off_eps, q.k), lat_energy<Store>(K.S.off_eps, q.l),
+        sm<double>(K.S.off_vr64, v), sm<double>(K.S.off_edx64, v), sm<double>(K.S.off_vr64, q.v2),
+        sm<double>(K.S.off_edx64, q.v2), i, j, q.k, q.l, K.L, K.log2L, K.magic, H1);
+    return take > 0 || metropolis64(dE, x2, K.T, K.invTf);
+}
+
 // The warp's block of 32 NL labels from kb on: label kb + 32 n + lane, n < NL.
 // Only labels whose theta holds and whose dH is below the cut go through the
 // accept test; the lowest accepting lane writes the warp's candidate and
 // lowers the CTA's best label.  True when the block holds an accept.
 // Store: the type of the energies in shared memory (long long: binary64 in
 // fixed point).
-template <typename Store, bool kPow2, int kDim, int NL>
+template <typename Store, bool kPow2, int kDim, int NL, bool kPair>
 __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const PhiloxPrefix &PP,
-                                         unsigned *best)
+                                         const PhiloxPrefix &PP2, unsigned *best)
 {
     constexpr bool kF64 = sizeof(Store) == 8, kFix = std::is_same<Store, long long>::value;
     uint32_t x1[NL], x2[NL];
     unsigned si[NL], sj[NL];
     int v[NL];
     float cv[NL], d[NL];
-    bool on[NL], cand[NL];
+    bool on[NL], cand[NL], pair[NL];
     bool odd = false;
 #pragma unroll
     for (int n = 0; n < NL; ++n) {
@@ -201,6 +307,7 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
         philox_finish(k, PP, K.key0, K.key1, x);
         x1[n] = x[1];
         x2[n] = x[2];
+        pair[n] = kPair && x[3] < K.pair_T;
         si[n] = kPow2 ? (x[0] >> (32 - kDim * K.log2L)) : __umulhi(x[0], K.N);
         const unsigned wi = sm<unsigned>(K.S.off_occ, si[n] >> 5);
         on[n] = ((wi >> (si[n] & 31u)) & 1u) && k < K.M;
@@ -230,21 +337,50 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
             const float fi = __int2float_rn(sm<int>(K.S.off_eps, 2 * si[n] + 1));
             const float fj = __int2float_rn(sm<int>(K.S.off_eps, 2 * sj[n] + 1));
             d[n] = fmaf(fj - fi, 0x1p-28f, -cv[n]);
-            cand[n] = theta && d[n] < K.cut;
+            cand[n] = theta && !pair[n] && d[n] < K.cut;
         } else if constexpr (kF64) {
             bool oi, oj;
             const float fi = hi_to_f32(sm<int>(K.S.off_eps, 2 * si[n] + 1), oi);
             const float fj = hi_to_f32(sm<int>(K.S.off_eps, 2 * sj[n] + 1), oj);
             d[n] = (fj - fi) - cv[n];
-            cand[n] = theta &&
+            cand[n] = theta && !pair[n] &&
                       (fmaf(fabsf(fi) + fabsf(fj), -0x1p-19f, d[n]) < K.cut || !oi || !oj);
         } else {
             d[n] = __fsub_rn(__fsub_rn(sm<float>(K.S.off_eps, sj[n]), sm<float>(K.S.off_eps, si[n])),
                              cv[n]);
-            cand[n] = theta && d[n] < K.cut;
+            cand[n] = theta && !pair[n] && d[n] < K.cut;
+        }
+        pair[n] = pair[n] && theta;
+    }
+    // pair labels whose first electron can hop: one in twenty at half filling,
+    // so a lane rarely has two and the block rarely takes a second turn
+    unsigned pacc = 0;                         // bit n: pair label n accepts
+    LatPair pq;                                // the lane's lowest accepting pair
+    double pdE = 0.0;
+    if constexpr (kPair) {
+        unsigned todo = (pair[0] ? 1u : 0u) | (NL > 1 && pair[NL - 1] ? 2u : 0u);
+        while (__any_sync(0xffffffffu, todo != 0u)) {
+            const bool first = (todo & 1u) || NL == 1;
+            if (todo) {
+                const unsigned i = first ? si[0] : si[NL - 1], j = first ? sj[0] : sj[NL - 1];
+                const int v1 = first ? v[0] : v[NL - 1];
+                const LatPair q = lat_pair<kPow2, kDim>(
+                    K, kb + (first ? 0u : 32u) + (unsigned)K.lane, PP2, i,
+                    sm<uint2>(K.S.off_rec, v1).y);
+                double dE;
+                if (q.ok &&
+                    lat_accept_pair<Store, kPow2, kDim>(K, q, i, j, v1, first ? cv[0] : cv[NL - 1],
+                                                        first ? x2[0] : x2[NL - 1], dE) &&
+                    !pacc) {
+                    pacc = first ? 1u : 2u;
+                    pq = q;
+                    pdE = dE;
+                }
+                todo &= todo - 1u;
+            }
         }
     }
-    if (!__any_sync(0xffffffffu, cand[0] || cand[NL - 1])) return false;
+    if (!__any_sync(0xffffffffu, cand[0] || cand[NL - 1] || pacc)) return false;
     // the accept test of the few labels near or below zero
     bool acc[NL];
     double dE[NL];
@@ -268,8 +404,8 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
     }
     // the warp's lowest accepting label: the first of the NL with an accept,
     // then the lowest lane (NL is 1 or 2)
-    const unsigned b0 = __ballot_sync(0xffffffffu, acc[0]);
-    const unsigned b1 = NL > 1 ? __ballot_sync(0xffffffffu, acc[NL - 1]) : 0u;
+    const unsigned b0 = __ballot_sync(0xffffffffu, acc[0] || (pacc & 1u));
+    const unsigned b1 = NL > 1 ? __ballot_sync(0xffffffffu, acc[NL - 1] || (pacc & 2u)) : 0u;
     if (!(b0 | b1)) return false;
     if (K.lane == __ffs(b0 ? b0 : b1) - 1) {
         Cand c;
@@ -279,6 +415,20 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
         c.dE = b0 ? dE[0] : dE[NL - 1];
         // binary32: the executed hop's dH is the binary32 one, widened
         if (!kF64 && c.dE == 0.0) c.dE = (double)(b0 ? d[0] : d[NL - 1]);
+        if constexpr (kPair) {
+            PairProp out;
+            out.k = out.l = 0xffffffffu;
+            out.v2 = out.dxy2 = 0;
+            out.pair = (b0 ? 1u : 2u) == pacc;
+            if (out.pair) {
+                out.k = pq.k;
+                out.l = pq.l;
+                out.v2 = pq.v2;
+                out.dxy2 = (int)pq.w2;
+                c.dE = pdE;
+            }
+            K.pcand[K.warp] = out;
+        }
         K.cand[K.warp] = c;
         atomicMin(best, kb + (b0 ? 0u : 32u * (unsigned)(NL - 1)) + (unsigned)K.lane);
     }
@@ -337,7 +487,7 @@ __device__ __forceinline__ int claim_replica(int *sched, int count, int n_sms)
     return order[pos];
 }
 
-template <typename Real, int kThreads, int kLog2L, bool kTime, int kDim = 2>
+template <typename Real, int kThreads, int kLog2L, bool kTime, int kDim = 2, bool kPair = false>
 __global__ void __launch_bounds__(kThreads, (kThreads >= 1024 ? 1 : 1024 / kThreads))
 pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, RunArgs a)
 {
@@ -352,6 +502,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     // labels of its own when a chunk is smaller than the CTA
     constexpr int kBook = kThreads - 32, kWarps = kThreads / 32;
     __shared__ Cand s_cand[kWarps];
+    __shared__ PairProp s_pcand[kPair ? kWarps : 1];   // the second electron of a pair candidate
     __shared__ unsigned s_best[2];
     // step-3c deviates of the next hops (CG_TIME_GAUSSIAN): the last warp
     // draws 32 at a time, one per lane
@@ -491,6 +642,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     K.N = (unsigned)N; K.magic = magic; K.M = M; K.thr_last = thr_last;
     K.key0 = key0; K.key1 = key1;
     K.cut = cut; K.invTf = invTf; K.T = T;
+    K.pcand = s_pcand; K.pair_T = Rg.pair_T; K.pair_R = Rg.pair_R; K.tab64 = Rg.tinv64;
 
     unsigned par = 0;
     for (unsigned long long h = 0; h < a.n_hops; ++h) {
@@ -512,7 +664,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         // blockDim, else one block of 32 for the first nw warps (a power of
         // two, at least 2).  m_ema is the same in every thread, so the choice
         // is uniform.
-        const float want = sqrtf(kLatChunkCost * m_ema);
+        const float want = sqrtf((kPair ? 0.5f : 1.0f) * kLatChunkCost * m_ema);
         const bool two = want > (float)kThreads;
         const unsigned nb = want > 2.0f * (float)kThreads ? 2u : 1u;
         unsigned nw = 2;
@@ -527,6 +679,10 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
             ++p;
             const PhiloxPrefix PP =
                 philox_prefix((uint32_t)rounds, (uint32_t)(rounds >> 32), rep, key0, key1);
+            PhiloxPrefix PP2{};
+            if (kPair)
+                PP2 = philox_prefix((uint32_t)rounds, (uint32_t)(rounds >> 32) | 0x80000000u, rep,
+                                    key0, key1);
             for (unsigned kb = 0; kb < M; kb += C) {
                 bool hit = false;
                 if ((unsigned)warp < nw) {
@@ -540,16 +696,20 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                         if (two) {
 #pragma unroll 1
                             for (unsigned k = k0; k < kb + C && !hit; k += nw * step)
-                                hit = lat_eval<Fix, kPow2, kDim, 2>(K, k, PP, &s_best[par]);
+                                hit = lat_eval<Fix, kPow2, kDim, 2, kPair>(K, k, PP, PP2,
+                                                                       &s_best[par]);
                         } else {
-                            hit = lat_eval<Fix, kPow2, kDim, 1>(K, k0, PP, &s_best[par]);
+                            hit = lat_eval<Fix, kPow2, kDim, 1, kPair>(K, k0, PP, PP2,
+                                                                       &s_best[par]);
                         }
                     } else if (two) {
 #pragma unroll 1
                         for (unsigned k = k0; k < kb + C && !hit; k += nw * step)
-                            hit = lat_eval<Real, kPow2, kDim, 2>(K, k, PP, &s_best[par]);
+                            hit = lat_eval<Real, kPow2, kDim, 2, kPair>(K, k, PP, PP2,
+                                                                       &s_best[par]);
                     } else {
-                        hit = lat_eval<Real, kPow2, kDim, 1>(K, k0, PP, &s_best[par]);
+                        hit = lat_eval<Real, kPow2, kDim, 1, kPair>(K, k0, PP, PP2,
+                                                                       &s_best[par]);
                     }
                 }
                 if (__syncthreads_or(hit)) {
@@ -586,6 +746,9 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         const unsigned q = wl + 1;                // 1-based label in the round
         const Cand c = s_cand[(wl - kb_hit) / step % nw];
         const unsigned ci = c.i, cj = c.j;
+        PairProp cq{};                         // second electron (toy mode has none)
+        if (kPair) cq = s_pcand[(wl - kb_hit) / step % nw];
+        const bool cpair = kPair && !a.toy && cq.pair;
         const unsigned long long m_hop = (p - 1) * (unsigned long long)M + q;
         m_ema = 0.9f * m_ema + 0.1f * (float)m_hop;
         long long t1 = 0;
@@ -595,31 +758,42 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
             if (!a.toy) {
                 sm<unsigned>(lay.off_occ, ci >> 5) &= ~(1u << (ci & 31));
                 sm<unsigned>(lay.off_occ, cj >> 5) |= (1u << (cj & 31));
+                if (cpair) {
+                    sm<unsigned>(lay.off_occ, cq.k >> 5) &= ~(1u << (cq.k & 31));
+                    sm<unsigned>(lay.off_occ, cq.l >> 5) |= (1u << (cq.l & 31));
+                }
             }
         }
         __syncwarp();     // or that warp would run the update twice, once for this lane
 
         // ---- local-energy update (step 3b) ----
+        // an executed pair applies the second electron's update after the first
+        // one's (each site rounds twice, in the serial order; a thread owns
+        // the same sites in both)
         unsigned big = 0;
-        if (kF64 && fixed) {
-            if (kDim == 3)
-                update_cubic<Fix, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
-                                                   log2L, magic, big);
-            else
-                update_square<Fix, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
-                                                    log2L, magic, big);
-        } else {
-            if (kDim == 3)
-                update_cubic<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
-                                                    log2L, magic, big);
-            else
-                update_square<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ci, cj, L,
-                                                     log2L, magic, big);
+#pragma unroll 1
+        for (int pass = 0; pass < (cpair ? 2 : 1); ++pass) {
+            const unsigned ui = kPair && pass ? cq.k : ci, uj = kPair && pass ? cq.l : cj;
+            if (kF64 && fixed) {
+                if (kDim == 3)
+                    update_cubic<Fix, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
+                                                       log2L, magic, big);
+                else
+                    update_square<Fix, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
+                                                        log2L, magic, big);
+            } else {
+                if (kDim == 3)
+                    update_cubic<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj, L,
+                                                        log2L, magic, big);
+                else
+                    update_square<Real, kThreads, kPow2>(!a.toy, lay.off_eps, lay.off_tinv, ui, uj,
+                                                         L, log2L, magic, big);
+            }
         }
         if (kF64 && fixed) {
             // an energy has reached 4 in size: back to binary64 before the
-            // next hop could leave the integers' range (one hop moves it by
-            // at most 1)
+            // next hop could leave the integers' range of 8 (a hop moves it by
+            // at most 1 per electron)
             if (__syncthreads_or((int)(big >> 30) & 1)) {
                 for (int l = tid; l < N; l += kThreads)
                     sm<double>(lay.off_eps, l) = fix_to_double(sm<long long>(lay.off_eps, l));
@@ -633,8 +807,10 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         }
         // the books of this hop, beside the next hop's first labels
         if (tid == kBook) {
-            int cdx, cdy;
-            vec_fields<kPow2, kDim>((unsigned)c.dxy, L, log2L, cdx, cdy);
+            int cdx, cdy, cdz, cdx2 = 0, cdy2 = 0;
+            vec_fields<kPow2, kDim>((unsigned)c.dxy, L, log2L, cdx, cdy, cdz);
+            if (kPair && cpair)
+                vec_fields<kPow2, kDim>((unsigned)cq.dxy2, L, log2L, cdx2, cdy2, cdz);
             s_c.cyc_rej += (unsigned long long)(t1 - s_c.t0);
             s_c.cyc_upd += (unsigned long long)(clock64() - t1);
             if (kTime)           // step 3c: Gaussian dt of hop number s_c.hops
@@ -645,7 +821,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
             s_c.evaluated += (kb_hit + C < M) ? (kb_hit + C) : M;
             s_c.hops += 1;
             if (!a.toy) {
-                s_c.P += cdx;
+                s_c.P += cdx + cdx2;
                 s_c.energy = d_add(s_c.energy, c.dE);
             }
             if (s_c.tracing)
@@ -655,8 +831,8 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                 e.i = ci; e.j = cj; e.q = q; e.p = (uint32_t)p; e.round = rounds;
                 e.dx = a.toy ? 0 : cdx; e.dy = a.toy ? 0 : cdy;
                 e.dE = a.toy ? 0.0 : c.dE;
-                e.k = 0xFFFFFFFFu; e.l = 0xFFFFFFFFu;
-                e.dx2 = 0; e.dy2 = 0;
+                e.k = cpair ? cq.k : 0xFFFFFFFFu; e.l = cpair ? cq.l : 0xFFFFFFFFu;
+                e.dx2 = cdx2; e.dy2 = cdy2;
                 s_c.log[a.log_offset + h] = e;
             }
         }
