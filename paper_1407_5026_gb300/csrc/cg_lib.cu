@@ -599,12 +599,32 @@ int choose_cluster(const cg_opts &o, const Rep &r, int optin)
     return 0;
 }
 
-// CTA size of a single-CTA group: the update needs at least L/2 threads (one
-// per base column); 384 is accepted as given.
-int choose_threads(const cg_opts &o, int L, int smem)
+// CTA size of a group: the update needs at least L/2 threads (one per base
+// column); 384 is accepted as given.  Without a wish, on one CTA per replica
+// (us per hop, one replica or the batch named):
+//   binary32: 256 threads, which have 128 registers each with two CTAs per SM
+//   (L = 128, 304 replicas, T = 0.01 and 0.05: 9.5 and 3.8 against 9.7 and 4.2
+//   with 512; L = 64, T = 0.05: 2.03 and 2.36), 512 from 24,576 sites on, where
+//   the update takes most of a hop (32^3: 3.8 against 4.4 with 256);
+//   binary64: 384 below 2048 sites, where a hop is one chain of latencies
+//   (L = 16: 2.9 against 3.4 with 1024), 512 below 12,288 (L = 96: 3.6 against
+//   3.9), else 1024 (L = 128, T = 0.01: 15.1 against 15.6 with 512);
+//   two-electron hops: 256, and 512 from 12,288 sites on: a label holds more
+//   values than 64 registers (L = 64, 304 replicas: 3.7 against 4.6 with 512).
+int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
 {
+    const int L = r.d.L, N = r.N;
     int t = o.block_threads;
-    if (t == 0) t = (o.precision == CG_FP64 || smem > 110 * 1024) ? 1024 : 512;
+    if (t == 0) {
+        if (r.random || cluster > 1)
+            t = (o.precision == CG_FP64 || smem > 110 * 1024) ? 1024 : 512;
+        else if (r.pair)
+            t = N < 12288 ? 256 : 512;
+        else if (o.precision == CG_FP64)
+            t = N < 2048 ? 384 : N < 12288 ? 512 : 1024;
+        else
+            t = N < 24576 ? 256 : 512;
+    }
     while (t < L / 2 && t < 1024) t = (t == 384) ? 512 : 2 * t;
     return t;
 }
@@ -1214,7 +1234,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         g.count = k - g.first;
         g.smem = smem;
         g.cluster = cluster;
-        g.threads = choose_threads(o, g.L, smem);
+        g.threads = choose_threads(o, h->reps[order[g.first]], smem, cluster);
         if (cluster > 1 && g.random) {
             // the random-site cluster kernel takes 256, 512 or 1024 threads
             if (g.threads == 384) g.threads = 512;

@@ -487,8 +487,13 @@ __device__ __forceinline__ int claim_replica(int *sched, int count, int n_sms)
     return order[pos];
 }
 
+// Registers: two CTAs of 256 or 512 threads per SM (128 or 64 each).  A label
+// pair in flight keeps about 90 values; at 256 threads the wider file gains more
+// than the second half of the warps did (four CTAs of 256 at 64 registers help
+// only batches of more than two replicas per SM: 608 of L = 64 2.1 ms against
+// 2.0, 912 2.9 against 3.0).
 template <typename Real, int kThreads, int kLog2L, bool kTime, int kDim = 2, bool kPair = false>
-__global__ void __launch_bounds__(kThreads, (kThreads >= 1024 ? 1 : 1024 / kThreads))
+__global__ void __launch_bounds__(kThreads, (kThreads >= 1024 ? 1 : (kThreads <= 256 ? 512 : 1024) / kThreads))
 pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, RunArgs a)
 {
     constexpr bool kPow2 = kLog2L >= 0;
