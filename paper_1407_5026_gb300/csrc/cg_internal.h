@@ -126,7 +126,8 @@ struct RunArgs {
     int *sched;                    // single hops, several CTAs per SM: the claim table of
                                    // launch_pr_schedule, or null (CTA b runs replica b)
     int n_sms;                     // SMs of the device (with sched)
-    int guide_bits;                // single hops on one CTA: log2 of the guide table's entries
+    int guide_bits;                // log2 of the guide table's entries (LatLayout)
+    int cluster_r2;                // cubic clusters: the update reads 1/r by r^2
     double toy_A0;
 };
 
@@ -188,6 +189,7 @@ __host__ __device__ inline LatLayout lat_layout(int N, int tab_entries, int V, i
 // at most four CTAs of 256 threads by registers) and fits the 227 KiB of one
 // CTA with room for the static part.  12 bits take less than the two-electron
 // kernel's layout, so a lattice that fits that one fits this.
+constexpr int kLatSmemMost = 227 * 1024 - 2048;
 inline int lat_guide_bits(int N, int tab_entries, int V, int words, int real_bytes)
 {
     auto total = [&](int b) { return lat_layout(N, tab_entries, V, words, real_bytes, b).total; };
@@ -195,9 +197,8 @@ inline int lat_guide_bits(int N, int tab_entries, int V, int words, int real_byt
         const int c = (228 * 1024) / (total(b) + 3072);
         return c < 4 ? c : 4;
     };
-    const int most = 227 * 1024 - 2048;
     for (int b = kLatGuideBits; b > 12; --b)
-        if (total(b) <= most && ctas(b) == ctas(12)) return b;
+        if (total(b) <= kLatSmemMost && ctas(b) == ctas(12)) return b;
     return 12;
 }
 

@@ -294,7 +294,8 @@ struct Group {
     bool random = false;             // random-site replicas (pr_random)
     bool sguide = false;             // their guide records in shared memory
     int *d_sched = nullptr;          // claim table of launches with several CTAs per SM
-    int gbits = kLatGuideBits;       // guide bits of the single-hop lattice kernel
+    int gbits = kLatGuideBits;       // lat_tables of the group's cluster size
+    bool r2 = false;
     int cluster = 1;                 // CTAs per replica
     unsigned M = 4096;               // labels per round when cg_run is given M = 0
     bool tuned = false;
@@ -533,24 +534,39 @@ double gamma_of(const Rep &r, const cg_opts &o)
     return Tp ? g / (1.0 - (double)Tp * 0x1p-32) : g;
 }
 
-// Guide bits of a lattice replica on the single-hop kernel.
-int guide_bits_of(const Rep &r, int precision)
+// Tables a lattice replica takes on the kernels that use LatLayout (one CTA, and
+// clusters with single hops): the guide's size, and on cubic clusters 1/r by
+// r^2 (3 (L/2)^2 + 1 entries) where the (L/2+1)^3 folded table does not fit.
+struct LatTables {
+    int gbits;
+    bool r2;
+    int total;       // dynamic shared memory
+};
+
+LatTables lat_tables(const Rep &r, int precision, int cluster)
 {
-    return lat_guide_bits(r.N, (int)r.tab->t64.size(), r.tab->V, r.words,
-                          precision == CG_FP64 ? 8 : 4);
+    const int rb = precision == CG_FP64 ? 8 : 4, folded = (int)r.tab->t64.size(), V = r.tab->V;
+    if (cluster == 1) {
+        const int b = lat_guide_bits(r.N, folded, V, r.words, rb);
+        return {b, false, lat_layout(r.N, folded, V, r.words, rb, b).total};
+    }
+    const bool cubic = dim_of(r.d) == 3;
+    for (int r2 = 0; r2 < (cubic ? 2 : 1); ++r2)
+        for (int b = kLatGuideBits; b >= 12; --b) {
+            const int total = lat_layout(r.N / cluster, r2 ? (int)r.tab->r2_64.size() : folded, V,
+                                         r.words, rb, b).total;
+            if (total <= kLatSmemMost || (b == 12 && r2 == (cubic ? 1 : 0)))
+                return {b, r2 == 1, total};
+        }
+    return {12, cubic, 0};      // not reached
 }
 
-// The single-hop cluster kernel on the cubic lattice keeps 1/r indexed by
-// r^2 (3 (L/2)^2 + 1 entries) instead of the (L/2+1)^3 folded table.
 int persistent_smem(const Rep &r, int precision, int cluster = 1)
 {
     if (r.random) return random_smem_bytes(r.N, cluster, cluster == 1 && r.sguide);
-    const int rb = precision == CG_FP64 ? 8 : 4;
-    const bool r2 = dim_of(r.d) == 3 && cluster > 1 && !r.pair;
-    const int ntab = r2 ? (int)r.tab->r2_64.size() : (int)r.tab->t64.size();
-    if (cluster == 1)
-        return lat_layout(r.N, ntab, r.tab->V, r.words, rb, guide_bits_of(r, precision)).total;
-    return smem_layout(r.N / cluster, ntab, r.tab->V, r.words, rb).total;
+    if (cluster == 1 || !r.pair) return lat_tables(r, precision, cluster).total;
+    return smem_layout(r.N / cluster, (int)r.tab->t64.size(), r.tab->V, r.words,
+                       precision == CG_FP64 ? 8 : 4).total;
 }
 
 // Whether a replica runs on c CTAs: by the layout of the cluster kernels' pair
@@ -990,6 +1006,19 @@ size_t plan_bytes(int R, const cg_replica_desc *reps, const cg_opts &o)
     return total + tc_total;
 }
 
+// One choice of tables for a group: the smallest guide and the r^2 table if any
+// replica takes it (their hop disks, and so their other tables, may differ).
+void set_lat_tables(const cg_handle *h, Group &g)
+{
+    g.gbits = kLatGuideBits;
+    g.r2 = false;
+    for (int k = g.first; !g.random && k < g.first + g.count; ++k) {
+        const LatTables t = lat_tables(h->reps[h->order[k]], h->opts.precision, g.cluster);
+        g.gbits = std::min(g.gbits, t.gbits);
+        g.r2 = g.r2 || t.r2;
+    }
+}
+
 cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, void *ws,
                        size_t ws_bytes)
 {
@@ -1210,6 +1239,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         }
         k = e;
     }
+    h->order = order;
     for (int k = 0; k < R;) {
         Group g;
         g.L = h->reps[order[k]].d.L;
@@ -1219,10 +1249,6 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         for (int m = k; m < R && gkey(order[m]) == gkey(order[k]); ++m)
             g.sguide = g.sguide && h->reps[order[m]].sguide;
         g.first = k;
-        // one table size for the group: the smallest its replicas take (their
-        // hop disks, and so their other tables, may differ)
-        for (int m = k; !g.random && m < R && gkey(order[m]) == gkey(order[k]); ++m)
-            g.gbits = std::min(g.gbits, guide_bits_of(h->reps[order[m]], o.precision));
         const int key = gkey(order[k]);
         int smem = 0, cluster = 1;
         for (int m = k; m < R && gkey(order[m]) == key; ++m)
@@ -1234,6 +1260,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         g.count = k - g.first;
         g.smem = smem;
         g.cluster = cluster;
+        set_lat_tables(h.get(), g);
         g.threads = choose_threads(o, h->reps[order[g.first]], smem, cluster);
         if (cluster > 1 && g.random) {
             // the random-site cluster kernel takes 256, 512 or 1024 threads
@@ -1279,7 +1306,6 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
                 return nullptr;
             }
     }
-    h->order = order;
     h->h_reps.resize(R);
     for (int k = 0; k < R; ++k) fill_dev(h->reps[k], o, h->h_reps[k], nullptr);
     if (cudaMemcpyAsync(h->d_reps, h->h_reps.data(), sizeof(DevReplica) * R,
@@ -1386,6 +1412,7 @@ int launch_group(cg_handle *h, const Group &g, unsigned long long hops, unsigned
     a.time_mode = h->opts.time_mode;
     a.pair = h->opts.pair_frac > 0.0 ? 1 : 0;
     a.guide_bits = g.gbits;
+    a.cluster_r2 = g.r2 ? 1 : 0;
     a.n_sms = h->n_sms;
     // more CTAs than SMs, all resident at once: pair heavy replicas with light
     // ones (the rank count is quadratic, and past one wave the hardware deals
@@ -1927,6 +1954,7 @@ int cg_autotune(cg_handle *h, uint32_t hops_per_trial)
                     g.smem = c.second;
                     g.threads = ct;
                     g.M = cM;
+                    set_lat_tables(h, g);
                     g.tuned = true;
                 }
             if (g.tuned) continue;
@@ -1985,6 +2013,7 @@ int cg_autotune(cg_handle *h, uint32_t hops_per_trial)
                     trial.threads = t;
                     trial.cluster = c;
                     trial.smem = cand.second;
+                    set_lat_tables(h, trial);
                     cudaEventRecord(e0, h->st);
                     int lrc = launch_group(h, trial, hops_per_trial, Ms[mi], 0, h->st);
                     cudaEventRecord(e1, h->st);
@@ -2023,6 +2052,7 @@ int cg_autotune(cg_handle *h, uint32_t hops_per_trial)
         g.M = best_M;
         g.cluster = best_c;
         g.smem = best_smem;
+        set_lat_tables(h, g);
         g.tuned = true;
         found.push_back({key, {best_t, best_M, best_c}});
     }

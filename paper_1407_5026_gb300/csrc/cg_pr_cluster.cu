@@ -4,12 +4,12 @@
 
 namespace cg {
 
-template <typename Real, int kThreads, bool kPow2, int kDim>
+template <typename Real, int kThreads, bool kPow2, int kDim, bool kR2 = false>
 static cudaError_t launch_cluster_d(const DevReplica *d_reps, const int *d_index, int n_reps,
                                     int cluster, int smem_bytes, const RunArgs &args,
                                     cudaStream_t st)
 {
-    auto kern = pr_cluster<Real, kThreads, kPow2, kDim>;
+    auto kern = pr_cluster<Real, kThreads, kPow2, kDim, false, kR2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          smem_bytes);
     if (e) return e;
@@ -33,6 +33,9 @@ static cudaError_t launch_cluster_t(const DevReplica *d_reps, const int *d_index
                                     int cluster, int smem_bytes, const RunArgs &args,
                                     cudaStream_t st, int dim)
 {
+    if (dim == 3 && args.cluster_r2)
+        return launch_cluster_d<Real, kThreads, kPow2, 3, true>(d_reps, d_index, n_reps, cluster,
+                                                                smem_bytes, args, st);
     return dim == 3 ? launch_cluster_d<Real, kThreads, kPow2, 3>(d_reps, d_index, n_reps, cluster,
                                                                  smem_bytes, args, st)
                     : launch_cluster_d<Real, kThreads, kPow2, 2>(d_reps, d_index, n_reps, cluster,

@@ -31,17 +31,19 @@
 // in turn.
 // The wall-clock limit of a hop is decided by rank 0 and published in its
 // exchange slot, so every exit decision is uniform over the cluster.
-// On the cubic lattice with single hops the update reads 1/r indexed by
+// On the cubic lattice with single hops, where the (L/2+1)^3 folded table does
+// not fit beside the CTA's share of eps (kR2), the update reads 1/r indexed by
 // r^2 = fx^2 + fy^2 + fz^2 of the folded offsets (3 (L/2)^2 + 1 entries, the
-// folded table's own values: 1/r depends on r^2 alone) instead of the
-// (L/2+1)^3 folded table: 12 KiB instead of 144 KiB at L = 64 in binary32,
-// where the folded table fits beside no share of eps.  The labels never read
+// folded table's own values: 1/r depends on r^2 alone): 12 KiB instead of
+// 144 KiB at L = 64 in binary32.  Neighbouring x's read the folded table
+// without bank conflicts, the r^2 table with about three per access, so the
+// folded one is taken where it fits (L = 48 on 4 CTAs).  The labels never read
 // either table (their 1/r comes from the per-vector tables).
 #pragma once
 
 #include <cooperative_groups.h>
 
-#include "cg_pr_common.cuh"
+#include "cg_pr_lattice.cuh"
 
 namespace coop = cooperative_groups;
 
@@ -97,12 +99,105 @@ __device__ __forceinline__ Real cluster_eps(coop::cluster_group &cl, Real *local
     return peer[off];
 }
 
-template <typename Real, int kThreads, bool kPow2, int kDim, bool kPair = false>
+// The warp's block of 32 NL labels from kb on in the cluster form of lat_eval:
+// the bitmask is local, the energies of the labels whose theta holds come from
+// the CTAs that own them.  The lowest accepting lane writes the warp's
+// candidate and lowers the CTA's best label.
+template <typename Real, bool kPow2, int kDim, int NL>
+__device__ __forceinline__ void cluster_eval(coop::cluster_group &cl, const LatConst &K, Real *eps,
+                                             int rows_local, unsigned rank, unsigned magicB,
+                                             unsigned kb, const PhiloxPrefix &PP, unsigned *best)
+{
+    constexpr bool kF64 = sizeof(Real) == 8;
+    uint32_t x1[NL], x2[NL];
+    unsigned si[NL], sj[NL];
+    int v[NL];
+    float cv[NL], d[NL];
+    Real ei[NL], ej[NL];
+    bool on[NL], cand[NL];
+    bool odd = false;
+#pragma unroll
+    for (int n = 0; n < NL; ++n) {
+        const unsigned k = kb + 32u * (unsigned)n + (unsigned)K.lane;
+        uint32_t x[4];
+        philox_finish(k, PP, K.key0, K.key1, x);
+        x1[n] = x[1];
+        x2[n] = x[2];
+        si[n] = kPow2 ? (x[0] >> (32 - kDim * K.log2L)) : __umulhi(x[0], K.N);
+        const unsigned wi = sm<unsigned>(K.S.off_occ, si[n] >> 5);
+        on[n] = ((wi >> (si[n] & 31u)) & 1u) && k < K.M;
+        const int g = (int)sm<unsigned char>(K.S.off_guide, x[1] >> K.gshift);
+        odd |= on[n] && g == 255;
+        v[n] = g + K.vbase;
+    }
+    if (odd) {
+#pragma unroll
+        for (int n = 0; n < NL; ++n)
+            if (on[n] && v[n] == 255 + K.vbase) on[n] = lat_search(K.S, x1[n], K.thr_last, v[n]);
+    }
+#pragma unroll
+    for (int n = 0; n < NL; ++n) {
+        v[n] = min(v[n], K.vlast);
+        const uint2 rc = sm<uint2>(K.S.off_rec, v[n]);
+        cv[n] = __uint_as_float(rc.x);
+        sj[n] = hop_target<kPow2, kDim>(si[n], rc.y, K.L, K.log2L, K.N, K.magic);
+        const unsigned wj = sm<unsigned>(K.S.off_occ, sj[n] >> 5);
+        cand[n] = on[n] && !((wj >> (sj[n] & 31u)) & 1u);
+        ei[n] = ej[n] = 0;
+    }
+    // both labels' remote reads in flight together
+#pragma unroll
+    for (int n = 0; n < NL; ++n)
+        if (cand[n]) {
+            ei[n] = cluster_eps<Real, kDim>(cl, eps, si[n], rows_local, K.log2L, K.L, K.magic,
+                                            kPow2, rank, magicB);
+            ej[n] = cluster_eps<Real, kDim>(cl, eps, sj[n], rows_local, K.log2L, K.L, K.magic,
+                                            kPow2, rank, magicB);
+        }
+#pragma unroll
+    for (int n = 0; n < NL; ++n) {
+        if constexpr (kF64) {
+            bool oi, oj;
+            const float fi = hi_to_f32(__double2hiint(ei[n]), oi);
+            const float fj = hi_to_f32(__double2hiint(ej[n]), oj);
+            d[n] = (fj - fi) - cv[n];
+            cand[n] = cand[n] &&
+                      (fmaf(fabsf(fi) + fabsf(fj), -0x1p-19f, d[n]) < K.cut || !oi || !oj);
+        } else {
+            d[n] = __fsub_rn(__fsub_rn(ej[n], ei[n]), cv[n]);
+            cand[n] = cand[n] && d[n] < K.cut;
+        }
+    }
+    if (!__any_sync(0xffffffffu, cand[0] || cand[NL - 1])) return;
+    bool acc[NL];
+    double dE[NL];
+#pragma unroll
+    for (int n = 0; n < NL; ++n) {
+        dE[n] = 0.0;
+        acc[n] = cand[n] && metropolis_label<Real>(ei[n], ej[n], sm<double>(K.S.off_vr64, v[n]),
+                                                   sm<double>(K.S.off_edx64, v[n]), cv[n], x2[n],
+                                                   K.T, K.invTf, dE[n]);
+    }
+    const unsigned b0 = __ballot_sync(0xffffffffu, acc[0]);
+    const unsigned b1 = NL > 1 ? __ballot_sync(0xffffffffu, acc[NL - 1]) : 0u;
+    if (!(b0 | b1)) return;
+    if (K.lane == __ffs(b0 ? b0 : b1) - 1) {
+        Cand c;
+        c.i = b0 ? si[0] : si[NL - 1];
+        c.j = b0 ? sj[0] : sj[NL - 1];
+        c.dxy = (int)sm<uint2>(K.S.off_rec, b0 ? v[0] : v[NL - 1]).y;
+        c.dE = b0 ? dE[0] : dE[NL - 1];
+        // binary32: the executed hop's dH is the binary32 one, widened
+        if (!kF64 && c.dE == 0.0) c.dE = (double)(b0 ? d[0] : d[NL - 1]);
+        K.cand[K.warp] = c;
+        atomicMin(best, kb + (b0 ? 0u : 32u * (unsigned)(NL - 1)) + (unsigned)K.lane);
+    }
+}
+
+template <typename Real, int kThreads, bool kPow2, int kDim, bool kPair = false, bool kR2 = false>
 __global__ void __launch_bounds__(kThreads, 1)
 pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, RunArgs a)
 {
-    // the update's 1/r indexed by r^2 (cubic lattice, single hops)
-    constexpr bool kR2 = kDim == 3 && !kPair;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int s_wlabel[32];
     __shared__ Cand s_cand[32];
@@ -112,6 +207,7 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     __shared__ double s_z[32];
     __shared__ unsigned long long s_zbase;
     __shared__ Slot s_slot[2][8];
+    __shared__ unsigned s_best[2];                        // single hops: lowest accepting label
     __shared__ PairProp s_pcand[kPair ? 32 : 1];          // pair data of each warp's candidate
     __shared__ PairProp s_pslot[kPair ? 2 : 1][kPair ? 8 : 1];   // ... of each CTA's
     __shared__ struct {
@@ -119,6 +215,7 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         long long P, t0;
         double energy, time;
         float m_ema;
+        unsigned late;
     } s_c;
 
     coop::cluster_group cl = coop::this_cluster();
@@ -141,19 +238,24 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         (kDim == 3 || Bq < 2) ? 0u : (unsigned)(4294967296ull / (unsigned)Bq + 1ull);
     const int ntab = kR2 ? 3 * (L >> 1) * (L >> 1) + 1 : kDim == 3 ? H1 * H1 * H1 : H1 * H1;
 
-    const SmemLayout lay = smem_layout(N_local, ntab, V, words, (int)sizeof(Real));
+    // two-electron hops keep the label code and the tables of smem_layout,
+    // single hops those of the one-CTA kernel
+    const SmemLayout layp = smem_layout(N_local, ntab, V, words, (int)sizeof(Real));
+    const LatLayout lay = lat_layout(N_local, ntab, V, words, (int)sizeof(Real), a.guide_bits);
+    const int off_eps = kPair ? layp.off_eps : lay.off_eps;
+    const int off_tinv = kPair ? layp.off_tinv : lay.off_tinv;
     Shared S;
-    S.eps = smem + lay.off_eps;
-    S.tinv = smem + lay.off_tinv;
-    S.occ = reinterpret_cast<unsigned *>(smem + lay.off_occ);
-    S.guide = reinterpret_cast<unsigned short *>(smem + lay.off_guide);
-    S.thr = reinterpret_cast<unsigned *>(smem + lay.off_thr);
-    S.disp = reinterpret_cast<int *>(smem + lay.off_disp);
-    S.vr64 = reinterpret_cast<double *>(smem + lay.off_vr64);
-    S.edx64 = reinterpret_cast<double *>(smem + lay.off_edx64);
-    S.cv32 = reinterpret_cast<float *>(smem + lay.off_cv32);
-    Real *eps = reinterpret_cast<Real *>(S.eps);
-    const Real *tinv = reinterpret_cast<const Real *>(S.tinv);
+    S.eps = smem + off_eps;
+    S.tinv = smem + off_tinv;
+    S.occ = reinterpret_cast<unsigned *>(smem + (kPair ? layp.off_occ : lay.off_occ));
+    S.guide = reinterpret_cast<unsigned short *>(smem + layp.off_guide);
+    S.thr = reinterpret_cast<unsigned *>(smem + layp.off_thr);
+    S.disp = reinterpret_cast<int *>(smem + layp.off_disp);
+    S.vr64 = reinterpret_cast<double *>(smem + layp.off_vr64);
+    S.edx64 = reinterpret_cast<double *>(smem + layp.off_edx64);
+    S.cv32 = reinterpret_cast<float *>(smem + layp.off_cv32);
+    Real *eps = reinterpret_cast<Real *>(smem + off_eps);
+    const Real *tinv = reinterpret_cast<const Real *>(smem + off_tinv);
 
     // ---- stage: own rows of eps, full tables and bitmask ----
     {
@@ -175,16 +277,20 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
         Real *tab_s = reinterpret_cast<Real *>(S.tinv);
         for (int l = tid; l < ntab; l += kThreads) tab_s[l] = tab_g[l];
         for (int l = tid; l < words; l += kThreads) S.occ[l] = Rg.occ[l];
-        for (int l = tid; l < kGuide; l += kThreads) S.guide[l] = Rg.guide[l];
-        for (int l = tid; l < V; l += kThreads) {
-            const int dxy = Rg.disp[l];
-            // dx of the packed vector (10-bit fields on the cubic lattice)
-            const int dx = kDim == 3 ? (dxy << 22) >> 22 : (int)(short)(dxy & 0xffff);
-            S.thr[l] = Rg.thr[l];
-            S.disp[l] = dxy;
-            S.vr64[l] = Rg.tinvd[l];
-            S.edx64[l] = d_mul(E, (double)dx);
-            S.cv32[l] = (float)d_add(Rg.tinvd[l], S.edx64[l]);   // one rounding to binary32
+        if (kPair) {
+            for (int l = tid; l < kGuide; l += kThreads) S.guide[l] = Rg.guide[l];
+            for (int l = tid; l < V; l += kThreads) {
+                const int dxy = Rg.disp[l];
+                // dx of the packed vector (10-bit fields on the cubic lattice)
+                const int dx = kDim == 3 ? (dxy << 22) >> 22 : (int)(short)(dxy & 0xffff);
+                S.thr[l] = Rg.thr[l];
+                S.disp[l] = dxy;
+                S.vr64[l] = Rg.tinvd[l];
+                S.edx64[l] = d_mul(E, (double)dx);
+                S.cv32[l] = (float)d_add(Rg.tinvd[l], S.edx64[l]);   // one rounding to binary32
+            }
+        } else {
+            stage_tower<kThreads, kPow2, kDim>(lay, Rg, a.guide_bits, L, log2L);
         }
     }
     DevCounters *cnt = Rg.ctr;
@@ -205,15 +311,28 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     cl.sync();   // every CTA staged before any remote read
 
     const unsigned M = a.M;
-    const unsigned thr_last = S.thr[V - 1];
-    const int rows_per_pass = kThreads / L;
-    const int active = rows_per_pass * L;
-    const int ux = tid % L, uy0 = tid / L;
+    const unsigned thr_last = kPair ? S.thr[V - 1] : sm<unsigned>(lay.off_thr, V - 1);
+    LatConst K;
+    K.S = lay; K.cand = s_cand;
+    K.L = L; K.log2L = log2L; K.vbase = lat_guide_base(V); K.vlast = V - 1;
+    K.gshift = 32 - a.guide_bits;
+    K.warp = warp; K.lane = lane;
+    K.N = (unsigned)N; K.magic = magic; K.M = M; K.thr_last = thr_last;
+    K.key0 = key0; K.key1 = key1;
+    K.cut = lat_cut<sizeof(Real) == 8>(T, E, L); K.invTf = invTf; K.T = T;
+    // cubic update: base columns (x, y) < L/2, one per thread and plane
+    const int Lh3 = L >> 1;
+    const int rows_per_pass = kThreads / Lh3;
+    const int active = rows_per_pass * Lh3;
+    const int ux = tid % Lh3, uy0 = tid / Lh3;
     // square lattice update: base rows per pass and the threads that work
     const int qrpp = kThreads / (L >> 1);
     const int qactive = qrpp * (L >> 1);
 
-    if (tid == 0) s_zbase = ~0ull;
+    if (tid == 0) {
+        s_zbase = ~0ull;
+        s_best[0] = s_best[1] = 0xffffffffu;
+    }
     __syncthreads();
     for (unsigned long long h = 0; h < a.n_hops; ++h) {
         if (a.time_mode && warp == 0) {
@@ -255,6 +374,41 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                                     key0, key1);
             for (unsigned kb = 0; kb < M; kb += chunk) {
                 const unsigned base = kb + rank * sub;
+                unsigned best = 0xffffffffu;
+                if constexpr (!kPair) {
+                // single hops: the warps with labels take blocks of 64; one CTA
+                // barrier, then warp 0 sends the CTA's candidate to every CTA,
+                // a lane each
+                if (a.toy) {
+                    for (unsigned k = (unsigned)warp * 32u; k < sub; k += kThreads)
+                        if (lat_eval_toy<kPow2, kDim>(K, base + k, PP, V, a.toy_A0, &s_best[parity]))
+                            break;
+                } else if (sub >= 64u) {
+                    const unsigned k = (unsigned)warp * 64u;
+                    if (k < sub)
+                        cluster_eval<Real, kPow2, kDim, 2>(cl, K, eps, rows_local, rank, magicB,
+                                                           base + k, PP, &s_best[parity]);
+                }
+                __syncthreads();
+                best = s_best[parity];
+                if (warp == 0) {
+                    if (lane == 0) {
+                        s_c.late = rank == 0 && globaltimer_ns() - s_c.wall0 > a.hop_timeout_ns;
+                        s_c.evaluated += (M - kb < chunk) ? (M - kb) : chunk;
+                        s_best[parity ^ 1u] = 0xffffffffu;    // last read a chunk ago
+                    }
+                    __syncwarp();
+                    if ((unsigned)lane < C) {
+                        Slot sl;
+                        sl.label = best;
+                        sl.late = s_c.late;
+                        sl.cand = s_cand[best == 0xffffffffu ? 0 : (best - base) / 64u % 32u];
+                        if (a.toy && best != 0xffffffffu)
+                            sl.cand = s_cand[(best - base) / 32u % (kThreads / 32u)];
+                        *cl.map_shared_rank(&s_slot[parity][rank], (unsigned)lane) = sl;
+                    }
+                }
+                } else {
                 const bool mine = (unsigned)tid < half;
                 const unsigned k0 = base + (unsigned)tid, k1 = k0 + half;
                 Prop p0{}, p1{};
@@ -309,7 +463,6 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                 }
                 }
                 const int any = __syncthreads_or(acc0 || acc1);
-                unsigned best = 0xffffffffu;
                 if (any) {
                     const unsigned b0 = __ballot_sync(0xffffffffu, acc0);
                     const unsigned b1 = __ballot_sync(0xffffffffu, acc1);
@@ -374,6 +527,7 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                     }
                     s_c.evaluated += (M - kb < chunk) ? (M - kb) : chunk;
                 }
+                }
                 cl.sync();
                 unsigned gbest = 0xffffffffu, gwin = 0;
                 for (unsigned r = 0; r < C; ++r) {
@@ -408,8 +562,13 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
 
         // ---- commit (step 3a, 3c): every CTA flips its bitmask copy ----
         const unsigned ci = win.i, cj = win.j;
-        const int cdx = kDim == 3 ? (win.dxy << 22) >> 22 : (int)(short)(win.dxy & 0xffff);
-        const int cdy = kDim == 3 ? (win.dxy << 12) >> 22 : win.dxy >> 16;
+        int cdx, cdy, cdz;
+        if constexpr (kPair) {
+            cdx = kDim == 3 ? (win.dxy << 22) >> 22 : (int)(short)(win.dxy & 0xffff);
+            cdy = kDim == 3 ? (win.dxy << 12) >> 22 : win.dxy >> 16;
+        } else {
+            vec_fields<kPow2, kDim>((unsigned)win.dxy, L, log2L, cdx, cdy, cdz);
+        }
         const bool cpair = kPair && !a.toy && wpq.pair;
         const int cdx2 = !cpair ? 0 : kDim == 3 ? (wpq.dxy2 << 22) >> 22 : (int)(short)(wpq.dxy2 & 0xffff);
         const int cdy2 = !cpair ? 0 : kDim == 3 ? (wpq.dxy2 << 12) >> 22 : wpq.dxy2 >> 16;
@@ -451,49 +610,55 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
             }
         }
         rounds += 1;
+        __syncwarp();     // or warp 0 would run the update twice, once for this lane
 
         // ---- local-energy update of this CTA's rows (step 3b) ----
         if (kDim == 3 && !a.toy && tid < active) {
-            // thread -> column x = ux of the (z, y) rows uy0, uy0 + rows_per_pass,
-            // ... of this CTA's planes (row r = zl L + y, site r L + x); an
-            // executed pair applies the second electron's update after the
-            // first one's
+            // thread -> base column x = ux < L/2 of the base (z, y) rows uy0,
+            // uy0 + rows_per_pass, ... of this CTA's planes (row r = zl L/2 + y);
+            // a base site serves (x + a L/2, y + b L/2), a, b in {0, 1}, of its
+            // plane: on an even ring fold(d + L/2) = L/2 - fold(d).  An executed
+            // pair applies the second electron's update after the first one's.
+            const int Lh = Lh3;
+            const unsigned magicH = (unsigned)(4294967296ull / (unsigned)Lh + 1ull);
 #pragma unroll 1
             for (int pass = 0; pass < (cpair ? 2 : 1); ++pass) {
             const unsigned ui = pass ? wpq.k : ci, uj = pass ? wpq.l : cj;
             int xi, yi, zi, xj, yj, zj;
-            if (kPow2) {
-                const int m = L - 1;
-                xi = (int)ui & m; yi = (int)(ui >> log2L) & m; zi = (int)(ui >> (2 * log2L));
-                xj = (int)uj & m; yj = (int)(uj >> log2L) & m; zj = (int)(uj >> (2 * log2L));
-            } else {
-                const unsigned qi = __umulhi(ui, magic), qj = __umulhi(uj, magic);
-                xi = (int)(ui - qi * (unsigned)L); zi = (int)__umulhi(qi, magic);
-                yi = (int)qi - zi * L;
-                xj = (int)(uj - qj * (unsigned)L); zj = (int)__umulhi(qj, magic);
-                yj = (int)qj - zj * L;
-            }
+            site_xyz<kPow2>(ui, L, log2L, magic, xi, yi, zi);
+            site_xyz<kPow2>(uj, L, log2L, magic, xj, yj, zj);
             const int fxj = fold_axis(ux - xj, L), fxi = fold_axis(ux - xi, L);
-            if constexpr (kR2) {
-                const int qj = fxj * fxj, qi = fxi * fxi;
-                for (int r = uy0; r < rows_local * L; r += rows_per_pass) {
-                    const int zl = kPow2 ? (r >> log2L) : (int)__umulhi((unsigned)r, magic);
-                    const int y = r - zl * L, z = row0 + zl;
-                    const int fzj = fold_axis(z - zj, L), fyj = fold_axis(y - yj, L);
-                    const int fzi = fold_axis(z - zi, L), fyi = fold_axis(y - yi, L);
-                    Real *e = eps + r * L + ux;
-                    *e = Prec<Real>::add(*e, Prec<Real>::sub(tinv[qj + fyj * fyj + fzj * fzj],
-                                                             tinv[qi + fyi * fyi + fzi * fzi]));
+            const int gxj = Lh - fxj, gxi = Lh - fxi;
+            const int xqj = fxj * fxj, xqi = fxi * fxi, uqj = gxj * gxj, uqi = gxi * gxi;
+#pragma unroll 2
+            for (int r = uy0; r < rows_local * Lh; r += rows_per_pass) {
+                const int zl = (int)__umulhi((unsigned)r, magicH);
+                const int y = r - zl * Lh, z = row0 + zl;
+                const int fzj = fold_axis(z - zj, L), fyj = fold_axis(y - yj, L);
+                const int fzi = fold_axis(z - zi, L), fyi = fold_axis(y - yi, L);
+                Real *e = &sm<Real>(off_eps, (zl * L + y) * L + ux);
+                Real ta[4], tb[4];
+                if constexpr (kR2) {
+                    const int zqj = fzj * fzj, zqi = fzi * fzi;
+                    const int p0 = zqj + fyj * fyj, p1 = zqj + (Lh - fyj) * (Lh - fyj);
+                    const int q0 = zqi + fyi * fyi, q1 = zqi + (Lh - fyi) * (Lh - fyi);
+                    ta[0] = sm<Real>(off_tinv, p0 + xqj); tb[0] = sm<Real>(off_tinv, q0 + xqi);
+                    ta[1] = sm<Real>(off_tinv, p0 + uqj); tb[1] = sm<Real>(off_tinv, q0 + uqi);
+                    ta[2] = sm<Real>(off_tinv, p1 + xqj); tb[2] = sm<Real>(off_tinv, q1 + xqi);
+                    ta[3] = sm<Real>(off_tinv, p1 + uqj); tb[3] = sm<Real>(off_tinv, q1 + uqi);
+                } else {
+                    const int p0 = (fzj * H1 + fyj) * H1, p1 = (fzj * H1 + Lh - fyj) * H1;
+                    const int q0 = (fzi * H1 + fyi) * H1, q1 = (fzi * H1 + Lh - fyi) * H1;
+                    ta[0] = sm<Real>(off_tinv, p0 + fxj); tb[0] = sm<Real>(off_tinv, q0 + fxi);
+                    ta[1] = sm<Real>(off_tinv, p0 + gxj); tb[1] = sm<Real>(off_tinv, q0 + gxi);
+                    ta[2] = sm<Real>(off_tinv, p1 + fxj); tb[2] = sm<Real>(off_tinv, q1 + fxi);
+                    ta[3] = sm<Real>(off_tinv, p1 + gxj); tb[3] = sm<Real>(off_tinv, q1 + gxi);
                 }
-            } else {
-                for (int r = uy0; r < rows_local * L; r += rows_per_pass) {
-                    const int zl = kPow2 ? (r >> log2L) : (int)__umulhi((unsigned)r, magic);
-                    const int y = r - zl * L, z = row0 + zl;
-                    const int oj = (fold_axis(z - zj, L) * H1 + fold_axis(y - yj, L)) * H1 + fxj;
-                    const int oi = (fold_axis(z - zi, L) * H1 + fold_axis(y - yi, L)) * H1 + fxi;
-                    Real *e = eps + r * L + ux;
-                    *e = Prec<Real>::add(*e, Prec<Real>::sub(tinv[oj], tinv[oi]));
-                }
+                Real *e1 = e + Lh * L;
+                e[0] = Prec<Real>::add(e[0], Prec<Real>::sub(ta[0], tb[0]));
+                e[Lh] = Prec<Real>::add(e[Lh], Prec<Real>::sub(ta[1], tb[1]));
+                e1[0] = Prec<Real>::add(e1[0], Prec<Real>::sub(ta[2], tb[2]));
+                e1[Lh] = Prec<Real>::add(e1[Lh], Prec<Real>::sub(ta[3], tb[3]));
             }
             }
         } else if (kDim == 2 && !a.toy && tid < qactive) {

@@ -141,6 +141,60 @@ __device__ __forceinline__ unsigned hop_target(unsigned i, unsigned w, int L, in
 //   rec     per vector: 1/r_v + E dx_v (binary32 bits), displacement word
 //   vr64, edx64   1/r_v and E dx_v (binary64)
 
+// The tower's tables into shared memory.
+template <int kThreads, bool kPow2, int kDim>
+__device__ __forceinline__ void stage_tower(const LatLayout &lay, const DevReplica &Rg,
+                                            int guide_bits, int L, int log2L)
+{
+    const int tid = threadIdx.x, V = Rg.V;
+    // the device table has 2^kLatGuideBits entries; a coarser bucket
+    // holds its entries' common value, or 255
+    const int per = 1 << (kLatGuideBits - guide_bits);
+    for (int b = tid; b < (1 << guide_bits); b += kThreads) {
+        unsigned char g = Rg.guide8[b * per];
+        for (int e = 1; e < per; ++e)
+            if (Rg.guide8[b * per + e] != g) g = 255;
+        sm<unsigned char>(lay.off_guide, b) = g;
+    }
+    for (int l = tid; l < V; l += kThreads) {
+        const int dxy = Rg.disp[l];
+        // dx of the packed vector (10-bit fields on the cubic lattice)
+        const int dx = kDim == 3 ? (dxy << 22) >> 22 : (int)(short)(dxy & 0xffff);
+        const double edx = d_mul(Rg.E, (double)dx);   // E * dx, as in the serial chain
+        sm<unsigned>(lay.off_thr, l) = Rg.thr[l];
+        sm<double>(lay.off_vr64, l) = Rg.tinvd[l];
+        sm<double>(lay.off_edx64, l) = edx;
+        // one rounding to binary32
+        sm<uint2>(lay.off_rec, l) = make_uint2(
+            __float_as_uint((float)d_add(Rg.tinvd[l], edx)), vec_word<kPow2, kDim>(dxy, L, log2L));
+    }
+    // hint[b] = smallest v with thr[v] >= b 2^(32 - kLatHintBits)
+    for (int b = tid; b <= (1 << kLatHintBits); b += kThreads) {
+        int lo = 0, hi = V - 1;
+        const unsigned long long x = (unsigned long long)b << (32 - kLatHintBits);
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (x <= Rg.thr[mid])
+                hi = mid;
+            else
+                lo = mid + 1;
+        }
+        sm<unsigned short>(lay.off_hint, b) = (unsigned short)lo;
+    }
+}
+
+// dH above which no acceptance variate accepts, with a margin: binary32
+// variates are at least 2^-24 (ln: -16.64), binary64 ones 2^-33, and the
+// binary64 test calls e^y zero below y = -23.  The binary32 form decides
+// |dH| < 1e-5 apart.  The binary64 bound leaves room for the rounding of cv and
+// of fixed-point energies to binary32.
+template <bool kF64>
+__device__ __forceinline__ float lat_cut(double T, double E, int L)
+{
+    return kF64 ? (float)(23.1 * T + (8.0 + fabs(E) * (double)(L / 2)) * 0x1p-21)
+                : fmaxf((float)(17.0 * T), 1.1e-5f);
+}
+
 // The smallest vector v with x1 <= thr[v], by bisection between the bounds of
 // x1's top bits; false for a null proposal (x1 above the last threshold).
 __device__ __forceinline__ bool lat_search(const LatLayout &S, uint32_t x1, unsigned thr_last,
@@ -552,40 +606,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                                  : reinterpret_cast<const Real *>(Rg.tinv32);
         for (int l = tid; l < ntab; l += kThreads) sm<Real>(lay.off_tinv, l) = tab_g[l];
         for (int l = tid; l < words; l += kThreads) sm<unsigned>(lay.off_occ, l) = Rg.occ[l];
-        // the device table has 2^kLatGuideBits entries; a coarser bucket
-        // holds its entries' common value, or 255
-        const int per = 1 << (kLatGuideBits - a.guide_bits);
-        for (int b = tid; b < (1 << a.guide_bits); b += kThreads) {
-            unsigned char g = Rg.guide8[b * per];
-            for (int e = 1; e < per; ++e)
-                if (Rg.guide8[b * per + e] != g) g = 255;
-            sm<unsigned char>(lay.off_guide, b) = g;
-        }
-        for (int l = tid; l < V; l += kThreads) {
-            const int dxy = Rg.disp[l];
-            // dx of the packed vector (10-bit fields on the cubic lattice)
-            const int dx = kDim == 3 ? (dxy << 22) >> 22 : (int)(short)(dxy & 0xffff);
-            const double edx = d_mul(Rg.E, (double)dx);   // E * dx, as in the serial chain
-            sm<unsigned>(lay.off_thr, l) = Rg.thr[l];
-            sm<double>(lay.off_vr64, l) = Rg.tinvd[l];
-            sm<double>(lay.off_edx64, l) = edx;
-            // one rounding to binary32
-            sm<uint2>(lay.off_rec, l) = make_uint2(
-                __float_as_uint((float)d_add(Rg.tinvd[l], edx)), vec_word<kPow2, kDim>(dxy, L, log2L));
-        }
-        // hint[b] = smallest v with thr[v] >= b 2^(32 - kLatHintBits)
-        for (int b = tid; b <= (1 << kLatHintBits); b += kThreads) {
-            int lo = 0, hi = V - 1;
-            const unsigned long long x = (unsigned long long)b << (32 - kLatHintBits);
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (x <= Rg.thr[mid])
-                    hi = mid;
-                else
-                    lo = mid + 1;
-            }
-            sm<unsigned short>(lay.off_hint, b) = (unsigned short)lo;
-        }
+        stage_tower<kThreads, kPow2, kDim>(lay, Rg, a.guide_bits, L, log2L);
     }
     unsigned long long rounds = Rg.ctr->rounds;
     float m_ema = Rg.ctr->m_ema > 0.f ? Rg.ctr->m_ema : 64.0f;
@@ -611,12 +632,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
 
     const unsigned M = a.M;
     const unsigned thr_last = sm<unsigned>(lay.off_thr, V - 1);
-    // dH above which no acceptance variate accepts, with a margin: binary32
-    // variates are at least 2^-24 (ln: -16.64), binary64 ones 2^-33, and the
-    // binary64 test calls e^y zero below y = -23.  The binary32 form decides
-    // |dH| < 1e-5 apart.  The binary64 bound leaves room for cv's rounding.
-    const float cut = kF64 ? (float)(23.1 * T + (8.0 + fabs(Rg.E) * (double)(L / 2)) * 0x1p-21)
-                           : fmaxf((float)(17.0 * T), 1.1e-5f);
+    const float cut = lat_cut<kF64>(T, Rg.E, L);
 
     // binary64: the energies and the table in fixed point where that is exact
     // for every one of them (the configurations' W = 1 and 2 at half filling;
