@@ -87,7 +87,8 @@ struct alignas(16) DevReplica {
     // random-site geometry (CG_SITES_RANDOM; null otherwise)
     const double *G;          // N x N minimum-image 1/r, 0 on the diagonal
     const int *rguide;        // 16 ints per site: kRandomGuide layout
-    const uint2 *rrec;        // per pair: C mod 2^32, partner j | (C >> 32) << 31 (C <= 2^32)
+    const uint32_t *rw;       // per pair: C - 1 (random_weight_count entries)
+    const uint2 *rj;          // per pair: partner j, 1/r + E dx in binary32
     const double2 *rgx;       // per pair: 1/r, E dx (minimum-image dx, binary64)
     int rguide_small;         // 1: every partner list holds at most 255 pairs
 };
@@ -220,6 +221,9 @@ cudaError_t set_pr_random_smem_limit(int bytes);
 // The offsets are 16 bits: the library refuses lists of 2^16 or more pairs.
 constexpr int kRandomGuide = 16;
 constexpr int kRandomBuckets = 16;
+// The running weights are read in aligned groups of four, up to eleven past the
+// first of a window: the array is padded by that.
+inline size_t random_weight_count(size_t pairs) { return (pairs + 15) / 4 * 4; }
 // Sites whose eps a CTA of a C-CTA cluster owns: ceil(N / C) rounded up to a
 // multiple of 32 (CTA rank owns [rank Nc, min(N, (rank + 1) Nc))).
 __host__ __device__ inline int random_cluster_sites(int N, int C)

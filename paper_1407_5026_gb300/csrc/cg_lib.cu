@@ -280,7 +280,8 @@ struct Rep {
     double Zmax = 0.0;
     double *d_px = nullptr, *d_py = nullptr, *d_G = nullptr;
     int *d_guide = nullptr;           // kRandomGuide ints per site
-    uint2 *d_rec = nullptr;           // running weight and partner of each pair
+    uint32_t *d_rw = nullptr;         // running weight less 1 of each pair
+    uint2 *d_rj = nullptr;            // partner and binary32 1/r + E dx of each pair
     double2 *d_rgx = nullptr;         // 1/r and E dx of each pair
     bool pair = false;                // the handle proposes two-electron hops
     // random sites: every partner list holds at most 255 pairs, and on one
@@ -625,6 +626,9 @@ int choose_cluster(const cg_opts &o, const Rep &r, int optin)
 //   binary64: 384 below 2048 sites, where a hop is one chain of latencies
 //   (L = 16: 2.9 against 3.4 with 1024), 512 below 12,288 (L = 96: 3.6 against
 //   3.9), else 1024 (L = 128, T = 0.01: 15.1 against 15.6 with 512);
+//   clusters of a lattice: 512, which leave 128 registers and cost less per
+//   cluster barrier (L = 256 on 4 CTAs: 4.1 against 4.7 ms with 1024, 48^3 on 4
+//   CTAs: 1.63 and 1.82);
 //   two-electron hops: 256, and 512 from 12,288 sites on: a label holds more
 //   values than 64 registers (L = 64, 304 replicas: 3.7 against 4.6 with 512).
 int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
@@ -632,7 +636,9 @@ int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
     const int L = r.d.L, N = r.N;
     int t = o.block_threads;
     if (t == 0) {
-        if (r.random || cluster > 1)
+        if (cluster > 1 && !r.random)
+            t = 512;
+        else if (r.random)
             t = (o.precision == CG_FP64 || smem > 110 * 1024) ? 1024 : 512;
         else if (r.pair)
             t = N < 12288 ? 256 : 512;
@@ -670,27 +676,31 @@ void fill_dev(const Rep &r, const cg_opts &o, DevReplica &dr, cg_hop *log)
     dr.C0 = t.C0;
     dr.eps = r.d_eps; dr.occ = r.d_occ; dr.phi = r.d_phi; dr.ctr = r.d_ctr;
     dr.log = log;
-    dr.G = r.d_G; dr.rguide = r.d_guide; dr.rrec = r.d_rec; dr.rgx = r.d_rgx;
+    dr.G = r.d_G; dr.rguide = r.d_guide; dr.rw = r.d_rw; dr.rj = r.d_rj; dr.rgx = r.d_rgx;
     dr.rguide_small = r.guide_small ? 1 : 0;
 }
 
 // The device form of a random-site replica's partner lists: per site the
 // kRandomGuide record (list bounds, the pair each x1 bucket starts at, the
-// last running weight), per pair (C mod 2^32, j | (C >> 32) << 31) and
+// last running weight), per pair its running weight less 1 (C - 1: 32 bits,
+// 1 <= C <= 2^32; padded to whole loads), (j, 1/r + E dx in binary32) and
 // (1/r, E dx).
-void pack_random(const Rep &r, std::vector<int> &guide, std::vector<uint32_t> &rec,
-                 std::vector<double> &rgx)
+void pack_random(const Rep &r, std::vector<int> &guide, std::vector<uint32_t> &rw,
+                 std::vector<uint32_t> &rj, std::vector<double> &rgx)
 {
     const int N = r.N;
     const size_t m = r.rj.size();
     guide.assign((size_t)N * kRandomGuide, 0);
-    rec.assign(2 * m, 0u);
+    rw.assign(random_weight_count(m), 0xffffffffu);
+    rj.assign(2 * m, 0u);
     rgx.assign(2 * m, 0.0);
     for (size_t k = 0; k < m; ++k) {
-        // C_k <= 2^32 in 33 bits: the low word, and its top bit above the
-        // partner (partners < N < 2^31)
-        rec[2 * k] = (uint32_t)r.rC[k];
-        rec[2 * k + 1] = r.rj[k] | ((uint32_t)(r.rC[k] >> 32) << 31);
+        // C_k = 0 (weights below 2^-32 at the head of a list) selects no x1 and
+        // is never reached from a bucket's start; 0 keeps the order
+        rw[k] = r.rC[k] ? (uint32_t)(r.rC[k] - 1) : 0u;
+        rj[2 * k] = r.rj[k];
+        const float cv = (float)(r.rg[k] + r.redx[k]);
+        std::memcpy(&rj[2 * k + 1], &cv, 4);
         rgx[2 * k] = r.rg[k];
         rgx[2 * k + 1] = r.redx[k];
     }
@@ -980,7 +990,8 @@ size_t plan_bytes(int R, const cg_replica_desc *reps, const cg_opts &o)
             tmp.N = (int)N;
             const size_t cnt = build_random(tmp) == CG_OK ? tmp.rj.size() : 0;
             const size_t c1 = cnt ? cnt : 1;
-            total += 2 * up(N * 8) + up(N * N * 8) + up(N * kRandomGuide * 4) + up(c1 * 8) + up(c1 * 16);
+            total += 2 * up(N * 8) + up(N * N * 8) + up(N * kRandomGuide * 4) +
+                     up(random_weight_count(c1) * 4) + up(c1 * 8) + up(c1 * 16);
         }
         auto key = std::make_tuple(d.L, d.r_max, d.xi, dim_of(d));
         if (std::find(seen.begin(), seen.end(), key) == seen.end()) {
@@ -1178,19 +1189,21 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         if (dalloc(h.get(), (void **)&r.d_px, N * 8) || dalloc(h.get(), (void **)&r.d_py, N * 8) ||
             dalloc(h.get(), (void **)&r.d_G, N * N * 8) ||
             dalloc(h.get(), (void **)&r.d_guide, N * kRandomGuide * 4) ||
-            dalloc(h.get(), (void **)&r.d_rec, cnt * 8) ||
+            dalloc(h.get(), (void **)&r.d_rw, random_weight_count(cnt) * 4) ||
+            dalloc(h.get(), (void **)&r.d_rj, cnt * 8) ||
             dalloc(h.get(), (void **)&r.d_rgx, cnt * 16)) { destroy_partial(); return nullptr; }
         const size_t m = r.rj.size();
         std::vector<int> guide;
-        std::vector<uint32_t> rec;
+        std::vector<uint32_t> rw, rj;
         std::vector<double> rgx;
-        pack_random(r, guide, rec, rgx);
+        pack_random(r, guide, rw, rj, rgx);
         cudaMemcpyAsync(r.d_px, r.px.data(), N * 8, cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(r.d_py, r.py.data(), N * 8, cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(r.d_guide, guide.data(), N * kRandomGuide * 4, cudaMemcpyHostToDevice,
                         h->st);
         if (m) {
-            cudaMemcpyAsync(r.d_rec, rec.data(), m * 8, cudaMemcpyHostToDevice, h->st);
+            cudaMemcpyAsync(r.d_rw, rw.data(), rw.size() * 4, cudaMemcpyHostToDevice, h->st);
+            cudaMemcpyAsync(r.d_rj, rj.data(), m * 8, cudaMemcpyHostToDevice, h->st);
             cudaMemcpyAsync(r.d_rgx, rgx.data(), m * 16, cudaMemcpyHostToDevice, h->st);
         }
         if (launch_g_build(r.d_px, r.d_py, r.d.L, r.N, r.d_G, h->st) != cudaSuccess) {

@@ -50,6 +50,16 @@ __device__ __forceinline__ float approx_f32(double x)
     return __uint_as_float(bits);
 }
 
+// Binary32 value of the high word of a normal binary64 x: truncated to 20
+// mantissa bits.  ok is false unless 2^-126 <= |x| < 2^60 (0 included), where
+// the word shift does not give x's value.
+__device__ __forceinline__ float hi_to_f32(int hi, bool &ok)
+{
+    ok = ((unsigned)hi << 1) - (897u << 21) < ((1083u - 897u) << 21);
+    const unsigned sh = (unsigned)hi * 8u + 0x40000000u;
+    return __uint_as_float((sh & 0x7fffffffu) | ((unsigned)hi & 0x80000000u));
+}
+
 struct Shared {
     void *eps;
     void *tinv;

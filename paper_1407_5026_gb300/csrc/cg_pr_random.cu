@@ -12,8 +12,8 @@
 // the minimum-image fold maps d to -d exactly.
 //
 // pr_random: one CTA per replica, binary64; eps and the occupation bitmask in
-// shared memory, the partner lists (a 64-byte guide record per site, 8-byte
-// pair records) and G in global memory (read-only path).  The round and
+// shared memory, the partner lists (a 64-byte guide record per site; weights,
+// partners and couplings per pair) and G in global memory (read-only path).  The round and
 // lowest-accepting-label structure is that of the lattice's persistent
 // kernel (mixed PR algorithm, steps 1-3), with one label per thread in every
 // chunk, so the trajectory equals the serial chain's on the same random
@@ -128,6 +128,7 @@ pr_random(const DevReplica *__restrict__ reps, const int *__restrict__ index, Ru
     __syncthreads();
 
     const unsigned M = a.M;
+    const float cut = (float)(23.1 * T) + 0x1p-18f;
     // one label per thread in every chunk: a chunk costs the latency of one
     // chain of dependent global loads (list offsets, search probes, partner,
     // 1/r) however many labels it holds, so the widest chunk settles a hop in
@@ -149,10 +150,8 @@ pr_random(const DevReplica *__restrict__ reps, const int *__restrict__ index, Ru
                                                  gsm);
                 double dE0 = 0.0;
                 bool acc0 = false;
-                if (p0.theta) {
-                    dE0 = dE_random(Rg, eps, p0);
-                    acc0 = metropolis64(dE0, p0.x2, T, invTf);
-                }
+                if (p0.theta)
+                    acc0 = accept_random(Rg, eps[p0.i], eps[p0.j], p0, cut, T, invTf, dE0);
                 const int any = __syncthreads_or(acc0);
                 if (any) {
                     const unsigned b0 = __ballot_sync(0xffffffffu, acc0);
@@ -219,6 +218,7 @@ pr_random(const DevReplica *__restrict__ reps, const int *__restrict__ index, Ru
             occ[c.j >> 5] |= (1u << (c.j & 31));
         }
         rounds += 1;
+        __syncwarp();     // or warp 0 would run the update twice, once for this lane
 
         // ---- local-energy update (step 3b): rows j and i of G ----
         {

@@ -12,16 +12,9 @@ struct RCand {
     double dE;
 };
 
-// Running weight C_m <= 2^32 of a packed pair record {C_m mod 2^32,
-// partner | (C_m >> 32) << 31}.
-__device__ __forceinline__ unsigned long long pair_weight(uint2 r)
-{
-    return (unsigned long long)r.x | ((unsigned long long)(r.y >> 31) << 32);
-}
-
 struct RLabel {
-    unsigned i, j, m, x2;
-    double2 gx;               // 1/r_ij and E dx_ij of partner m
+    unsigned i, j, m, x2;     // m: the pair's index
+    float cv;                 // 1/r_ij + E dx_ij in binary32
     bool theta;
 };
 
@@ -29,11 +22,13 @@ struct RLabel {
 // its partner, so the partner is looked up for occupied sites only: the
 // smallest m of i's list with x1 < C_m.  One 64-byte load of i's guide record
 // gives the list's bounds, its last running weight (x1 at or above it: a null
-// proposal) and the bucket of pairs x1 >> 29 can select; a four-way search
-// (three independent probes per step) narrows the bucket to at most four
-// records, and the last scan reads whole records, so the partner comes with
-// its running weight; 1/r and E dx of each scanned record are loaded beside
-// it, so the chosen partner's come with no further dependent load.
+// proposal) and the bucket of pairs x1 >> 28 can select; a four-way search
+// (three independent probes per step) narrows a bucket of more than eight, and
+// the rest is counted from up to three aligned loads of four weights (C_m - 1,
+// 32 bits).  The chosen pair's partner and its binary32 1/r + E dx come with one
+// more load.  (Reading whole records with 1/r and E dx beside the weights took
+// seven sectors per label for these four; the L1's tag stage was the second
+// stall of the kernel, tex_throttle 3.5 per issue.)
 // gsm: the compacted guide records in shared memory (two uint4 per site:
 // {first, last lo, length | last hi << 16, 0} and the 16 bucket starts as
 // bytes), or null for the 64-byte records in global memory.
@@ -46,7 +41,7 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
     p.theta = false;
     p.i = p.j = p.m = 0;
     p.x2 = 0;
-    p.gx = make_double2(0.0, 0.0);
+    p.cv = 0.0f;
     if (!valid) return p;
     uint32_t x[4];
     philox_finish(k, PP, key0, key1, x);
@@ -54,6 +49,7 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
     p.x2 = x[2];
     if (!((occ[p.i >> 5] >> (p.i & 31)) & 1u)) return p;
     const unsigned long long x1 = x[1];
+    const uint32_t w1 = x[1];
     const unsigned b = x[1] >> 28, b1 = b + 1;
     int first, end, glo, ghi;
     unsigned long long last;
@@ -92,60 +88,63 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
                   : end;
     }
     int lo = glo, hi = min(ghi, end - 1) + 1;
-    const uint2 *rc = Rg.rrec;
-    // the answer lies in [lo, hi); record m holds C_m in 33 bits
-    while (hi - lo > 4) {
+    const uint32_t *rw = Rg.rw;
+    // the answer lies in [lo, hi); x1 < C_m iff x1 <= rw[m]
+    while (hi - lo > 8) {
         const int q = (hi - lo) >> 2;
         const int m1 = lo + q, m2 = m1 + q, m3 = m2 + q;
-        const unsigned long long c1 = pair_weight(__ldg(rc + m1)), c2 = pair_weight(__ldg(rc + m2)),
-                                 c3 = pair_weight(__ldg(rc + m3));
-        if (x1 < c1) {
+        const uint32_t c1 = __ldg(rw + m1), c2 = __ldg(rw + m2), c3 = __ldg(rw + m3);
+        if (w1 <= c1) {
             hi = m1 + 1;
-        } else if (x1 < c2) {
+        } else if (w1 <= c2) {
             lo = m1 + 1;
             hi = m2 + 1;
-        } else if (x1 < c3) {
+        } else if (w1 <= c3) {
             lo = m2 + 1;
             hi = m3 + 1;
         } else {
             lo = m3 + 1;
         }
     }
-    // the records with x1 < C_m form a suffix of [lo, hi): walking down, the
-    // last one that holds is the smallest
-    int m = hi - 1;
-    unsigned j = __ldg(rc + m).y & 0x7fffffffu;
-    double2 gx = __ldg(Rg.rgx + m);
+    // the pairs of [lo, hi - 1) with C_m <= x1 come before the answer (the
+    // weights rise along the list); a window of up to 11 from the group lo is in
+    const int base = lo & ~3;
+    const uint4 *r4 = reinterpret_cast<const uint4 *>(rw + base);
+    const uint4 wa = __ldg(r4);
+    uint4 wb = make_uint4(0u, 0u, 0u, 0u), wc = wb;
+    if (base + 4 < hi - 1) wb = __ldg(r4 + 1);
+    if (base + 8 < hi - 1) wc = __ldg(r4 + 2);
+    const uint32_t w[12] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w, wc.x, wc.y, wc.z, wc.w};
+    int m = lo;
 #pragma unroll
-    for (int t = 1; t <= 3; ++t) {
-        const int mt = hi - 1 - t;
-        if (mt >= lo) {
-            const uint2 r = __ldg(rc + mt);
-            const double2 gt = __ldg(Rg.rgx + mt);
-            if (x1 < pair_weight(r)) {
-                m = mt;
-                j = r.y & 0x7fffffffu;
-                gx = gt;
-            }
-        }
+    for (int t = 0; t < 12; ++t) {
+        const int e = base + t;
+        m += (e >= lo && e < hi - 1 && w[t] < w1) ? 1 : 0;
     }
+    const uint2 rc = __ldg(Rg.rj + m);
     p.m = (unsigned)m;
-    p.j = j;
-    p.gx = gx;
+    p.j = rc.x;
+    p.cv = __uint_as_float(rc.y);
     p.theta = !((occ[p.j >> 5] >> (p.j & 31)) & 1u);     // n_i = 1 here
     return p;
 }
 
-// dH = ((eps_j - eps_i) - 1/r_ij) - E dx_ij, each step rounded (binary64)
-__device__ __forceinline__ double dE_random_vals(double ei, double ej, const RLabel &p)
+// Step 2 for a label whose theta holds: its dH is bounded from the energies'
+// high words first (as in the lattice kernels), and the few labels below the cut
+// take the binary64 one, ((eps_j - eps_i) - 1/r_ij) - E dx_ij, each step rounded,
+// and the binary64 decision.  (Three binary64 adds per label on the slow pipe
+// were a quarter of a chunk.)
+__device__ __forceinline__ bool accept_random(const DevReplica &Rg, double ei, double ej,
+                                              const RLabel &p, float cut, double T, float invTf,
+                                              double &dE)
 {
-    return d_sub(d_sub(d_sub(ej, ei), p.gx.x), p.gx.y);
-}
-
-__device__ __forceinline__ double dE_random(const DevReplica &Rg, const double *eps,
-                                            const RLabel &p)
-{
-    return dE_random_vals(eps[p.i], eps[p.j], p);
+    bool oi, oj;
+    const float fi = hi_to_f32(__double2hiint(ei), oi), fj = hi_to_f32(__double2hiint(ej), oj);
+    const float d = (fj - fi) - p.cv, s = fabsf(fi) + fabsf(fj) + fabsf(p.cv);
+    if (!(fmaf(s, -0x1p-19f, d) < cut) && oi && oj) return false;
+    const double2 gx = __ldg(Rg.rgx + p.m);
+    dE = d_sub(d_sub(d_sub(ej, ei), gx.x), gx.y);
+    return metropolis64(dE, p.x2, T, invTf);
 }
 
 // Stage the compacted guide records of all N sites into shared memory (two

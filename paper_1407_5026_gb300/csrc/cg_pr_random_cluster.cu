@@ -105,6 +105,7 @@ pr_random_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ i
     cl.sync();   // every CTA staged before any remote read
 
     const unsigned M = a.M;
+    const float cut = (float)(23.1 * T) + 0x1p-18f;
     // one label per thread per chunk, as in pr_random: a chunk costs one
     // chain of dependent global loads however many labels it holds
     const unsigned chunk = (unsigned)kThreads * C;
@@ -130,8 +131,7 @@ pr_random_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ i
                 if (p0.theta) {
                     const double ei = cluster_eps_random(cl, eps, p0.i, Nc, magicW, rank);
                     const double ej = cluster_eps_random(cl, eps, p0.j, Nc, magicW, rank);
-                    dE0 = dE_random_vals(ei, ej, p0);
-                    acc0 = metropolis64(dE0, p0.x2, T, invTf);
+                    acc0 = accept_random(Rg, ei, ej, p0, cut, T, invTf, dE0);
                 }
                 const int any = __syncthreads_or(acc0);
                 unsigned best = 0xffffffffu;
@@ -215,6 +215,7 @@ pr_random_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ i
             occ[win.j >> 5] |= (1u << (win.j & 31));
         }
         rounds += 1;
+        __syncwarp();     // or warp 0 would run the update twice, once for this lane
 
         // ---- local-energy update of this CTA's sites (step 3b) ----
         {
