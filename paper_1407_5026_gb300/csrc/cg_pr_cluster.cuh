@@ -160,9 +160,10 @@ __device__ __forceinline__ void cluster_eval(coop::cluster_group &cl, const LatC
             bool oi, oj;
             const float fi = hi_to_f32(__double2hiint(ei[n]), oi);
             const float fj = hi_to_f32(__double2hiint(ej[n]), oj);
-            d[n] = (fj - fi) - cv[n];
-            cand[n] = cand[n] &&
-                      (fmaf(fabsf(fi) + fabsf(fj), -0x1p-19f, d[n]) < K.cut || !oi || !oj);
+            // at most dH (or nothing known: the test decides)
+            d[n] = fmaf(fabsf(fi) + fabsf(fj), -0x1p-19f, (fj - fi) - cv[n]) - K.slack;
+            if (!oi || !oj) d[n] = 0.0f;
+            cand[n] = cand[n] && d[n] < K.cut && !surely_rejected(d[n], x2[n], K.invTf);
         } else {
             d[n] = __fsub_rn(__fsub_rn(ej[n], ei[n]), cv[n]);
             cand[n] = cand[n] && d[n] < K.cut;
@@ -319,7 +320,7 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     K.warp = warp; K.lane = lane;
     K.N = (unsigned)N; K.magic = magic; K.M = M; K.thr_last = thr_last;
     K.key0 = key0; K.key1 = key1;
-    K.cut = lat_cut<sizeof(Real) == 8>(T, E, L); K.invTf = invTf; K.T = T;
+    K.cut = lat_cut<sizeof(Real) == 8>(T); K.slack = lat_slack(E, L); K.invTf = invTf; K.T = T;
     // cubic update: base columns (x, y) < L/2, one per thread and plane
     const int Lh3 = L >> 1;
     const int rows_per_pass = kThreads / Lh3;

@@ -207,6 +207,15 @@ __device__ __forceinline__ bool metropolis_f32(float dE, uint32_t x2, float invT
     return dE <= 0.0f || (float)(x2 >> 9) < metropolis_bound_f32(dE, invTf);
 }
 
+// Whether u rejects every dH >= lo, decided in binary32 with metropolis64's
+// margins: true only if the binary64 test rejects too.  It spares the binary64
+// pipe all but the labels that accept and a few in a thousand.
+__device__ __forceinline__ bool surely_rejected(float lo, uint32_t x2, float invTf)
+{
+    const float u = __uint2float_rn(x2) * 0x1p-32f;
+    return lo > 0.0f && u > __expf(-lo * invTf) * (1.0f + 2e-4f) + 0x1p-31f;
+}
+
 // Step 2 (accept test) of a label whose theta holds, from the two local
 // energies, 1/r_v and E dx_v (binary64) and their binary32 sum.
 template <typename Real>

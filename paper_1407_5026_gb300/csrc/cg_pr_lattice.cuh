@@ -186,13 +186,17 @@ __device__ __forceinline__ void stage_tower(const LatLayout &lay, const DevRepli
 // dH above which no acceptance variate accepts, with a margin: binary32
 // variates are at least 2^-24 (ln: -16.64), binary64 ones 2^-33, and the
 // binary64 test calls e^y zero below y = -23.  The binary32 form decides
-// |dH| < 1e-5 apart.  The binary64 bound leaves room for the rounding of cv and
-// of fixed-point energies to binary32.
+// |dH| < 1e-5 apart.
 template <bool kF64>
-__device__ __forceinline__ float lat_cut(double T, double E, int L)
+__device__ __forceinline__ float lat_cut(double T)
 {
-    return kF64 ? (float)(23.1 * T + (8.0 + fabs(E) * (double)(L / 2)) * 0x1p-21)
-                : fmaxf((float)(17.0 * T), 1.1e-5f);
+    return kF64 ? (float)(23.1 * T) : fmaxf((float)(17.0 * T), 1.1e-5f);
+}
+
+// Room for the rounding of cv and of fixed-point energies to binary32.
+__device__ __forceinline__ float lat_slack(double E, int L)
+{
+    return (float)((8.0 + fabs(E) * (double)(L / 2)) * 0x1p-21);
 }
 
 // The smallest vector v with x1 <= thr[v], by bisection between the bounds of
@@ -221,7 +225,7 @@ struct LatConst {
     int L, log2L, vbase, vlast, gshift, warp, lane;
     unsigned N, magic, M, thr_last;
     uint32_t key0, key1;
-    float cut, invTf;
+    float cut, slack, invTf;   // slack: binary64's bound on what binary32 loses of dH
     double T;
     // two-electron hops
     PairProp *pcand;           // per warp: the second electron of its candidate
@@ -380,15 +384,16 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
             // 2^-28 + 2^-22 each below 4; the cut's slack covers it
             const float fi = __int2float_rn(sm<int>(K.S.off_eps, 2 * si[n] + 1));
             const float fj = __int2float_rn(sm<int>(K.S.off_eps, 2 * sj[n] + 1));
-            d[n] = fmaf(fj - fi, 0x1p-28f, -cv[n]);
+            d[n] = fmaf(fj - fi, 0x1p-28f, -cv[n]) - K.slack;    // at most dH
             cand[n] = theta && !pair[n] && d[n] < K.cut;
         } else if constexpr (kF64) {
             bool oi, oj;
             const float fi = hi_to_f32(sm<int>(K.S.off_eps, 2 * si[n] + 1), oi);
             const float fj = hi_to_f32(sm<int>(K.S.off_eps, 2 * sj[n] + 1), oj);
-            d[n] = (fj - fi) - cv[n];
-            cand[n] = theta && !pair[n] &&
-                      (fmaf(fabsf(fi) + fabsf(fj), -0x1p-19f, d[n]) < K.cut || !oi || !oj);
+            // at most dH (or nothing known: the test decides)
+            d[n] = fmaf(fabsf(fi) + fabsf(fj), -0x1p-19f, (fj - fi) - cv[n]) - K.slack;
+            if (!oi || !oj) d[n] = 0.0f;
+            cand[n] = theta && !pair[n] && d[n] < K.cut;
         } else {
             d[n] = __fsub_rn(__fsub_rn(sm<float>(K.S.off_eps, sj[n]), sm<float>(K.S.off_eps, si[n])),
                              cv[n]);
@@ -425,6 +430,14 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
         }
     }
     if (!__any_sync(0xffffffffu, cand[0] || cand[NL - 1] || pacc)) return false;
+    // binary64: the bound on dH rejects most of them; what is left takes the
+    // slow pipe
+    if constexpr (kF64) {
+#pragma unroll
+        for (int n = 0; n < NL; ++n)
+            cand[n] = cand[n] && !surely_rejected(d[n], x2[n], K.invTf);
+        if (!__any_sync(0xffffffffu, cand[0] || cand[NL - 1] || pacc)) return false;
+    }
     // the accept test of the few labels near or below zero
     bool acc[NL];
     double dE[NL];
@@ -622,7 +635,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
 
     const unsigned M = a.M;
     const unsigned thr_last = sm<unsigned>(lay.off_thr, V - 1);
-    const float cut = lat_cut<kF64>(T, Rg.E, L);
+    const float cut = lat_cut<kF64>(T);
 
     // binary64: the energies and the table in fixed point where that is exact
     // for every one of them (the configurations' W = 1 and 2 at half filling;
@@ -652,7 +665,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     K.warp = warp; K.lane = lane;
     K.N = (unsigned)N; K.magic = magic; K.M = M; K.thr_last = thr_last;
     K.key0 = key0; K.key1 = key1;
-    K.cut = cut; K.invTf = invTf; K.T = T;
+    K.cut = cut; K.slack = lat_slack(Rg.E, L); K.invTf = invTf; K.T = T;
     K.pcand = s_pcand; K.pair_T = Rg.pair_T; K.pair_R = Rg.pair_R; K.tab64 = Rg.tinv64;
 
     unsigned par = 0;

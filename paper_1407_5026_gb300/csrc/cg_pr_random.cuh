@@ -140,8 +140,9 @@ __device__ __forceinline__ bool accept_random(const DevReplica &Rg, double ei, d
 {
     bool oi, oj;
     const float fi = hi_to_f32(__double2hiint(ei), oi), fj = hi_to_f32(__double2hiint(ej), oj);
-    const float d = (fj - fi) - p.cv, s = fabsf(fi) + fabsf(fj) + fabsf(p.cv);
-    if (!(fmaf(s, -0x1p-19f, d) < cut) && oi && oj) return false;
+    const float s = fabsf(fi) + fabsf(fj) + fabsf(p.cv);
+    const float lo = fmaf(s, -0x1p-19f, (fj - fi) - p.cv);      // at most dH
+    if (oi && oj && (!(lo < cut) || surely_rejected(lo, p.x2, invTf))) return false;
     const double2 gx = __ldg(Rg.rgx + p.m);
     dE = d_sub(d_sub(d_sub(ej, ei), gx.x), gx.y);
     return metropolis64(dE, p.x2, T, invTf);
