@@ -334,7 +334,10 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
                                int dim, const float *d_ghat, const float2 *d_tw, float2 *d_buf,
                                cudaStream_t st);
 size_t refresh_fft_buffer_bytes(int N, int R);
-bool refresh_fft_size_ok(int L);      // L = 2^m (4..1024) or 3 2^m (6..192)
+// L = 2^m (4..1024), 3 2^m (6..192), or a multiple of 8 (square 16..160, cubic
+// 16..64)
+bool refresh_fft_size_ok(int L, int dim);
+bool refresh_fft_clears(int L, int dim);
 int refresh_tc_ksplit(int N, int dim);
 int refresh_tc_max_replicas(int dim);   // replicas per launch
 size_t refresh_tc_scratch_bytes(int N, int dim, int R);

@@ -320,21 +320,44 @@ constexpr int kTcSmemLimit = 227 * 1024 - 1024;
 // memory.
 // In-place DFT (exponent -2 pi i j k / n) of n complex values at stride
 // `stride`, binary64, for the refresh's host-side table: radix 2 for n = 2^m,
-// the plain sum otherwise (n <= 192 there).
+// otherwise halved down to the odd part and the plain sum of that.
 void host_fft(std::complex<double> *x, int n, size_t stride)
 {
     if (n & (n - 1)) {
-        std::vector<std::complex<double>> in(n), w(n);
+        std::vector<std::complex<double>> w(n), out(n), t(n);
         for (int j = 0; j < n; ++j) {
-            in[j] = x[(size_t)j * stride];
             const double a = -2.0 * M_PI * (double)j / (double)n;
             w[j] = std::complex<double>(std::cos(a), std::sin(a));
         }
-        for (int k = 0; k < n; ++k) {
-            std::complex<double> acc = 0.0;
-            for (int j = 0; j < n; ++j) acc += in[j] * w[(size_t)j * k % n];
-            x[(size_t)k * stride] = acc;
+        // out[q m + k], k < m: the transform of x[q + u j], j < m, for q < u in
+        // bit-reversed order of q, u = n / m; m doubles from the odd part on
+        int m = n, u = 1;
+        while (m % 2 == 0) { m /= 2; u *= 2; }
+        for (int q = 0; q < u; ++q) {
+            int r = 0;
+            for (int b = 1; b < u; b *= 2) r = 2 * r + ((q / b) & 1);
+            for (int k = 0; k < m; ++k) {
+                std::complex<double> acc = 0.0;
+                int e = 0;
+                for (int j = 0; j < m; ++j) {
+                    acc += x[((size_t)r + (size_t)u * j) * stride] * w[(size_t)e * u];
+                    e += k;
+                    if (e >= m) e -= m;
+                }
+                out[(size_t)q * m + k] = acc;
+            }
         }
+        for (; m < n; m *= 2) {
+            const int step = n / (2 * m);
+            for (int q = 0; q < n; q += 2 * m)
+                for (int k = 0; k < m; ++k) {
+                    const std::complex<double> a = out[q + k], b = out[q + m + k] * w[k * step];
+                    t[q + k] = a + b;
+                    t[q + m + k] = a - b;
+                }
+            out.swap(t);
+        }
+        for (int k = 0; k < n; ++k) x[(size_t)k * stride] = out[k];
         return;
     }
     for (int i = 1, j = 0; i < n; ++i) {
@@ -391,7 +414,7 @@ void build_fft_tables(Tables &t)
 // L = 2^m or 3 2^m (CG_REFRESH_AUTO or CG_REFRESH_FFT).
 bool group_uses_fft(const cg_opts &o, int L, int dim)
 {
-    if (o.precision != CG_FP32 || !refresh_fft_size_ok(L)) return false;
+    if (o.precision != CG_FP32 || !refresh_fft_size_ok(L, dim)) return false;
     if (dim != 2 && dim != 3) return false;
     return o.refresh_kind == CG_REFRESH_AUTO || o.refresh_kind == CG_REFRESH_FFT;
 }
@@ -1376,7 +1399,8 @@ int refresh_group(cg_handle *h, const Group &g, cudaStream_t st)
         }
         return CG_OK;
     }
-    CG_CUDA(launch_reset_refresh_err(h->d_reps, h->d_index + g.first, g.count, st));
+    if (!(g.fft && refresh_fft_clears(g.L, g.dim)))
+        CG_CUDA(launch_reset_refresh_err(h->d_reps, h->d_index + g.first, g.count, st));
     if (g.fft) {
         const Tables &t = *h->reps[h->order[g.first]].tab;
         CG_CUDA(launch_refresh_fft(h->d_reps, h->d_index + g.first, g.count, g.L, g.dim, t.d_ghat,
@@ -1398,11 +1422,21 @@ int refresh_group(cg_handle *h, const Group &g, cudaStream_t st)
     return CG_OK;
 }
 
+// Every group's refresh; with several lattice sizes on the groups' own streams
+// between a fork and a join, as the runs are: each alone leaves most SMs idle.
 int refresh_all(cg_handle *h)
 {
+    const bool forked = h->groups.size() > 1;
+    if (forked) CG_CUDA(cudaEventRecord(h->fork, h->st));
     for (const Group &g : h->groups) {
-        const int rc = refresh_group(h, g, h->st);
+        cudaStream_t st = forked ? g.st : h->st;
+        if (forked) CG_CUDA(cudaStreamWaitEvent(st, h->fork, 0));
+        const int rc = refresh_group(h, g, st);
         if (rc) return rc;
+        if (forked) {
+            CG_CUDA(cudaEventRecord(g.done, st));
+            CG_CUDA(cudaStreamWaitEvent(h->st, g.done, 0));
+        }
     }
     return CG_OK;
 }

@@ -219,6 +219,16 @@ __device__ __forceinline__ void record_change(float ca, float cb, bool two, bool
     }
 }
 
+// The refresh's record of the largest change starts again (thread 0 of a CTA
+// that runs before every record_change of the pair).
+__device__ __forceinline__ void clear_change(bool two, DevCounters *da, DevCounters *db)
+{
+    if (threadIdx.x == 0) {
+        da->max_err_bits = 0ull;
+        if (two) db->max_err_bits = 0ull;
+    }
+}
+
 // One pass over W lines of one pair.  kMode: 0 forward x from the bitmasks;
 // 1 forward (buffer to buffer); 2 forward, product with DFT(g)/N, inverse
 // (the last axis); 3 inverse (buffer to buffer); 4 inverse x into eps.
@@ -330,10 +340,13 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
 }
 
 // ---------------------------------------------------------------------------
-// Square lattices of L = 16 to 128: the whole refresh of a replica pair in one
-// CTA.  Its L x L complex values stay in shared memory (132 KiB at L = 128)
-// through all the transforms, where the passes above write and read the pair's
-// values through L2 between launches and run a barrier per radix-2 stage.
+// Sides that are multiples of 8, square lattices of L = 16 to 160 and cubic ones
+// of 16 to 64.  On the square lattice one CTA does the whole refresh of a replica
+// pair: its L x L complex values stay in shared memory (132 KiB at L = 128)
+// through all the transforms, where the passes above write and read them through
+// L2 between launches and run a barrier per radix-2 stage (304 replicas of
+// L = 128: 0.225 -> 0.085 ms).  Cubic lattices take three launches over planes
+// instead of five passes.
 //
 // A line of L = R1 8 elements transforms in two steps, in place:
 //     X[c + R1 d] = sum_b W_8^(b d) W_L^(b c) sum_a W_R1^(a c) x[8 a + b]
@@ -472,64 +485,62 @@ __device__ __forceinline__ void dft(float2 (&v)[R])
     }
 }
 
+// CTA size of a plane's transforms: one item per thread in the 8-point steps of
+// up to 512 threads (128 registers; R1 > 12 holds 4 R1 of them), L = 128 on 1024.
 template <int L>
-constexpr int fft_cta_threads()
+constexpr int fft_plane_threads()
 {
-    return L == 128 ? 1024 : L == 96 ? 576 : L == 64 ? 512 : L == 48 ? 288 : L == 32 ? 128 : 64;
+    return L == 128 ? 1024 : L * L / 8 >= 512 ? 512 : (L * L / 8 + 31) / 32 * 32;
 }
 
-template <int L>
-__global__ void __launch_bounds__(fft_cta_threads<L>()) fft_cta_kernel(FftArgs a)
+// R-point transform of v for the R1 that dft has no steps for: the plain sum,
+// W_R^k = W_L^(8 k) from the shared twiddles (the same word for the whole warp).
+template <int L, bool kInv>
+__device__ __forceinline__ void dft_r1(float2 (&v)[L / 8], const float2 *tw)
 {
-    constexpr int R1 = L / 8, kT = fft_cta_threads<L>(), Ls = L + 1;
-    extern __shared__ float2 s[];
-    __shared__ unsigned s_err[2];
-    float2 *tw = s + L * Ls;                              // exp(-2 pi i k / L)
-    const int tid = threadIdx.x, p = blockIdx.x;
-    const DevReplica &Ra = a.reps[a.index[2 * p]];
-    const bool two = 2 * p + 1 < a.R;
-    const DevReplica &Rb = a.reps[a.index[two ? 2 * p + 1 : 2 * p]];
-    for (int k = tid; k < L; k += kT) tw[k] = a.tw[k];
-    if (tid < 2) s_err[tid] = 0u;
-    __syncthreads();
-    auto at = [&](int y, int x) -> float2 & {
-        return s[y * Ls + (x & ~7) + ((x ^ (x >> 3)) & 7)];
-    };
-    // rows r and r + 8 share a half-warp: their 8-element runs fall in
-    // opposite halves of the banks
-    auto row_of = [](int r) {
-        return L % 16 ? r : (r & ~15) | ((r & 1) << 3) | ((r >> 1) & 7);
-    };
-    // phi and eps, which the last sweep reads, on their way into L2 meanwhile
-    for (int r = 0; r < (two ? 2 : 1); ++r) {
-        const DevReplica &R = r ? Rb : Ra;
-        const char *f = reinterpret_cast<const char *>(R.phi), *e = reinterpret_cast<const char *>(R.eps);
-        for (int k = tid * 128; k < L * L * 8; k += kT * 128)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(f + k));
-        for (int k = tid * 128; k < L * L * 4; k += kT * 128)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(e + k));
-    }
-    // x, step 1, from the bitmasks
-    {
-        const float na = (float)Ra.nu, nb = (float)Rb.nu;
-        for (int it = tid; it < L * 8; it += kT) {
-            const int b = it & 7, y = row_of(it >> 3);
-            float2 v[R1];
+    constexpr int R = L / 8;
+    if constexpr (R == 2 || R == 3 || R == 4 || R == 6 || R == 8 || R == 12 || R == 16) {
+        dft<R, kInv>(v);
+    } else {
+        float2 o[R];
 #pragma unroll
-            for (int k = 0; k < R1; ++k) {
-                const unsigned site = (unsigned)(y * L + 8 * k + b);
-                const unsigned wa = __ldg(Ra.occ + (site >> 5)), wb = __ldg(Rb.occ + (site >> 5));
-                v[k] = make_float2((float)((wa >> (site & 31u)) & 1u) - na,
-                                   two ? (float)((wb >> (site & 31u)) & 1u) - nb : 0.0f);
+        for (int k = 0; k < R; ++k) o[k] = v[0];
+#pragma unroll
+        for (int n = 1; n < R; ++n) {
+            o[0] = cadd(o[0], v[n]);
+#pragma unroll
+            for (int k = 1; k < R; ++k) {
+                float2 w = tw[8 * ((n * k) % R)];
+                if (kInv) w.y = -w.y;
+                o[k].x = fmaf(v[n].x, w.x, fmaf(-v[n].y, w.y, o[k].x));
+                o[k].y = fmaf(v[n].x, w.y, fmaf(v[n].y, w.x, o[k].y));
             }
-            dft<R1, false>(v);
-#pragma unroll
-            for (int c = 0; c < R1; ++c) at(y, 8 * c + b) = c ? cmul(v[c], tw[b * c]) : v[c];
         }
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = o[k];
     }
-    __syncthreads();
+}
+
+// The sweeps of one L x L plane of a pair in shared memory (see above).
+template <int L>
+struct Plane {
+    static constexpr int R1 = L / 8, kT = fft_plane_threads<L>(), Ls = L + 1;
+    static constexpr int kSmem = (L * Ls + L) * (int)sizeof(float2);
+    float2 *s, *tw;
+
+    __device__ __forceinline__ float2 &at(int y, int x) const
+    {
+        return s[y * Ls + (x & ~7) + ((x ^ (x >> 3)) & 7)];
+    }
+    // rows r and r + 8 share a half-warp: their 8-element runs fall in opposite
+    // halves of the banks
+    static __device__ __forceinline__ int row_of(int r)
+    {
+        return L % 16 ? r : (r & ~15) | ((r & 1) << 3) | ((r >> 1) & 7);
+    }
     // item -> (row, c) of the 8-element groups of the rows
-    auto group_of = [](int it, int &y, int &c) {
+    static __device__ __forceinline__ void group_of(int it, int &y, int &c)
+    {
         if (R1 % 8 == 0) {
             const int rest = it >> 4;
             c = (it & 7) + 8 * (rest % (R1 / 8));
@@ -538,96 +549,158 @@ __global__ void __launch_bounds__(fft_cta_threads<L>()) fft_cta_kernel(FftArgs a
             c = it % R1;
             y = it / R1;
         }
-    };
-    // x, step 2
-    for (int it = tid; it < L * R1; it += kT) {
-        int y, c;
-        group_of(it, y, c);
-        float2 v[8];
-#pragma unroll
-        for (int b = 0; b < 8; ++b) v[b] = at(y, 8 * c + b);
-        dft<8, false>(v);
-#pragma unroll
-        for (int d = 0; d < 8; ++d) at(y, 8 * c + d) = v[d];
     }
-    __syncthreads();
-    // y, step 1
-    for (int it = tid; it < L * 8; it += kT) {
-        const int x = it % L, b = it / L;
-        float2 v[R1];
-#pragma unroll
-        for (int k = 0; k < R1; ++k) v[k] = at(8 * k + b, x);
-        dft<R1, false>(v);
-#pragma unroll
-        for (int c = 0; c < R1; ++c) at(8 * c + b, x) = c ? cmul(v[c], tw[b * c]) : v[c];
-    }
-    __syncthreads();
-    // y, step 2, the product with DFT(g)/N, and the inverse's first step
-    for (int it = tid; it < L * R1; it += kT) {
-        const int x = it % L, c = it / L, kx = (x >> 3) + R1 * (x & 7);
-        float2 v[8];
-#pragma unroll
-        for (int b = 0; b < 8; ++b) v[b] = at(8 * c + b, x);
-        dft<8, false>(v);
-#pragma unroll
-        for (int d = 0; d < 8; ++d) {
-            const float g = __ldg(a.ghat + (c + R1 * d) * L + kx);
-            v[d] = make_float2(v[d].x * g, v[d].y * g);
-        }
-        dft<8, true>(v);
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            float2 w = tw[b * c];
-            w.y = -w.y;
-            at(8 * c + b, x) = cmul(v[b], w);
-        }
-    }
-    __syncthreads();
-    // y, the inverse's second step
-    for (int it = tid; it < L * 8; it += kT) {
-        const int x = it % L, b = it / L;
-        float2 v[R1];
-#pragma unroll
-        for (int c = 0; c < R1; ++c) v[c] = at(8 * c + b, x);
-        dft<R1, true>(v);
-#pragma unroll
-        for (int k = 0; k < R1; ++k) at(8 * k + b, x) = v[k];
-    }
-    __syncthreads();
-    // x, the inverse's first step
-    for (int it = tid; it < L * R1; it += kT) {
-        int y, c;
-        group_of(it, y, c);
-        float2 v[8];
-#pragma unroll
-        for (int d = 0; d < 8; ++d) v[d] = at(y, 8 * c + d);
-        dft<8, true>(v);
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            float2 w = tw[b * c];
-            w.y = -w.y;
-            at(y, 8 * c + b) = cmul(v[b], w);
-        }
-    }
-    __syncthreads();
-    // x, the inverse's second step, into eps
-    float err_a = 0.0f, err_b = 0.0f;
+    __device__ __forceinline__ void twiddles(const float2 *g) const
     {
-        const double *__restrict__ pa = Ra.phi, *__restrict__ pb = Rb.phi;
-        float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps);
-        float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps);
+        for (int k = threadIdx.x; k < L; k += kT) tw[k] = g[k];
+    }
+    __device__ __forceinline__ float2 conj_tw(int e) const
+    {
+        return make_float2(tw[e].x, -tw[e].y);
+    }
+    // x, both forward steps, from the bitmasks of the plane at site0
+    __device__ __forceinline__ void x_from_bits(const DevReplica &Ra, const DevReplica &Rb, bool two,
+                                                unsigned site0) const
+    {
+        const float na = (float)Ra.nu, nb = (float)Rb.nu;
+        for (int it = threadIdx.x; it < L * 8; it += kT) {
+            const int b = it & 7, y = row_of(it >> 3);
+            float2 v[R1];
+#pragma unroll
+            for (int k = 0; k < R1; ++k) {
+                const unsigned site = site0 + (unsigned)(y * L + 8 * k + b);
+                const unsigned wa = __ldg(Ra.occ + (site >> 5)), wb = __ldg(Rb.occ + (site >> 5));
+                v[k] = make_float2((float)((wa >> (site & 31u)) & 1u) - na,
+                                   two ? (float)((wb >> (site & 31u)) & 1u) - nb : 0.0f);
+            }
+            dft_r1<L, false>(v, tw);
+#pragma unroll
+            for (int c = 0; c < R1; ++c) at(y, 8 * c + b) = c ? cmul(v[c], tw[b * c]) : v[c];
+        }
+        __syncthreads();
+        for (int it = threadIdx.x; it < L * R1; it += kT) {
+            int y, c;
+            group_of(it, y, c);
+            float2 v[8];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) v[b] = at(y, 8 * c + b);
+            dft<8, false>(v);
+#pragma unroll
+            for (int d = 0; d < 8; ++d) at(y, 8 * c + d) = v[d];
+        }
+    }
+    // columns, step 1 (kGlobal: read from rows of the buffer, `row` values apart)
+    template <bool kGlobal>
+    __device__ __forceinline__ void col_step1(const float2 *g, size_t row) const
+    {
+        for (int it = threadIdx.x; it < L * 8; it += kT) {
+            const int x = it % L, b = it / L;
+            float2 v[R1];
+#pragma unroll
+            for (int k = 0; k < R1; ++k) v[k] = kGlobal ? g[(8 * k + b) * row + x] : at(8 * k + b, x);
+            dft_r1<L, false>(v, tw);
+#pragma unroll
+            for (int c = 0; c < R1; ++c) at(8 * c + b, x) = c ? cmul(v[c], tw[b * c]) : v[c];
+        }
+    }
+    // columns, step 2, the product with DFT(g)/N and the inverse's first step;
+    // wave numbers of slot x and c + R1 d: gh[(c + R1 d) gstride + kx]
+    __device__ __forceinline__ void col_product(const float *gh, size_t gstride) const
+    {
+        for (int it = threadIdx.x; it < L * R1; it += kT) {
+            const int x = it % L, c = it / L, kx = (x >> 3) + R1 * (x & 7);
+            float2 v[8];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) v[b] = at(8 * c + b, x);
+            dft<8, false>(v);
+#pragma unroll
+            for (int d = 0; d < 8; ++d) {
+                const float g = __ldg(gh + (c + R1 * d) * gstride + kx);
+                v[d] = make_float2(v[d].x * g, v[d].y * g);
+            }
+            dft<8, true>(v);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) at(8 * c + b, x) = cmul(v[b], conj_tw(b * c));
+        }
+    }
+    // columns, the inverse's second step (kGlobal: into rows of the buffer)
+    template <bool kGlobal>
+    __device__ __forceinline__ void col_inverse2(float2 *g, size_t row) const
+    {
+        for (int it = threadIdx.x; it < L * 8; it += kT) {
+            const int x = it % L, b = it / L;
+            float2 v[R1];
+#pragma unroll
+            for (int c = 0; c < R1; ++c) v[c] = at(8 * c + b, x);
+            dft_r1<L, true>(v, tw);
+#pragma unroll
+            for (int k = 0; k < R1; ++k) {
+                if (kGlobal)
+                    g[(8 * k + b) * row + x] = v[k];
+                else
+                    at(8 * k + b, x) = v[k];
+            }
+        }
+    }
+    // columns, step 2 forward into the buffer, and back from it
+    __device__ __forceinline__ void col_step2_store(float2 *g) const
+    {
+        for (int it = threadIdx.x; it < L * R1; it += kT) {
+            const int x = it % L, c = it / L;
+            float2 v[8];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) v[b] = at(8 * c + b, x);
+            dft<8, false>(v);
+#pragma unroll
+            for (int d = 0; d < 8; ++d) g[(8 * c + d) * L + x] = v[d];
+        }
+    }
+    __device__ __forceinline__ void col_inverse1_load(const float2 *g) const
+    {
+        for (int it = threadIdx.x; it < L * R1; it += kT) {
+            const int x = it % L, c = it / L;
+            float2 v[8];
+#pragma unroll
+            for (int d = 0; d < 8; ++d) v[d] = g[(8 * c + d) * L + x];
+            dft<8, true>(v);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) at(8 * c + b, x) = cmul(v[b], conj_tw(b * c));
+        }
+    }
+    // x, the inverse's first step
+    __device__ __forceinline__ void x_inverse1() const
+    {
+        for (int it = threadIdx.x; it < L * R1; it += kT) {
+            int y, c;
+            group_of(it, y, c);
+            float2 v[8];
+#pragma unroll
+            for (int d = 0; d < 8; ++d) v[d] = at(y, 8 * c + d);
+            dft<8, true>(v);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) at(y, 8 * c + b) = cmul(v[b], conj_tw(b * c));
+        }
+    }
+    // x, the inverse's second step, into eps of the plane at site0; the largest
+    // changes of the thread's sites
+    __device__ __forceinline__ void x_into_eps(const DevReplica &Ra, const DevReplica &Rb, bool two,
+                                               unsigned site0, float &err_a, float &err_b) const
+    {
+        const double *__restrict__ pa = Ra.phi + site0, *__restrict__ pb = Rb.phi + site0;
+        float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps) + site0;
+        float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps) + site0;
         // the transforms took n - nu with nu rounded to binary32; sum_t g(s-t)
         // = C0 for every s, so (nu_f - nu) C0 restores the exact nu
         const float ca = (float)d_mul(d_sub((double)(float)Ra.nu, Ra.nu), Ra.C0);
         const float cb = (float)d_mul(d_sub((double)(float)Rb.nu, Rb.nu), Rb.C0);
-        for (int it = tid; it < L * 8; it += kT) {
+        for (int it = threadIdx.x; it < L * 8; it += kT) {
             const int b = it & 7, y = row_of(it >> 3), site = y * L + b;
             float2 v[R1];
 #pragma unroll
             for (int c = 0; c < R1; ++c) v[c] = at(y, 8 * c + b);
-            dft<R1, true>(v);
-            // four elements' loads in flight at a time
-            constexpr int kBatch = R1 % 4 == 0 ? 4 : R1 % 3 == 0 ? 3 : 2;
+            dft_r1<L, true>(v, tw);
+            // a few elements' loads in flight at a time
+            constexpr int kBatch = R1 % 4 == 0 ? 4 : R1 % 3 == 0 ? 3 : R1 % 5 == 0 ? 5 : R1 % 2 == 0 ? 2 : 1;
 #pragma unroll
             for (int k0 = 0; k0 < R1; k0 += kBatch) {
                 double fa[kBatch], fb[kBatch];
@@ -654,17 +727,118 @@ __global__ void __launch_bounds__(fft_cta_threads<L>()) fft_cta_kernel(FftArgs a
             }
         }
     }
+    // phi and eps of the plane, which the last sweep reads, on their way into L2
+    __device__ __forceinline__ void prefetch(const DevReplica &R, unsigned site0) const
+    {
+        const char *f = reinterpret_cast<const char *>(R.phi + site0);
+        const char *e = reinterpret_cast<const char *>(reinterpret_cast<const float *>(R.eps) + site0);
+        for (int k = threadIdx.x * 128; k < L * L * 8; k += kT * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(f + k));
+        for (int k = threadIdx.x * 128; k < L * L * 4; k += kT * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(e + k));
+    }
+};
+
+// The square lattice: the whole refresh of a pair.
+template <int L>
+__global__ void __launch_bounds__(fft_plane_threads<L>()) fft_square_kernel(FftArgs a)
+{
+    extern __shared__ float2 s[];
+    __shared__ unsigned s_err[2];
+    const Plane<L> P{s, s + L * Plane<L>::Ls};
+    const int p = blockIdx.x;
+    const DevReplica &Ra = a.reps[a.index[2 * p]];
+    const bool two = 2 * p + 1 < a.R;
+    const DevReplica &Rb = a.reps[a.index[two ? 2 * p + 1 : 2 * p]];
+    P.twiddles(a.tw);
+    if (threadIdx.x < 2) s_err[threadIdx.x] = 0u;
+    clear_change(two, Ra.ctr, Rb.ctr);
+    __syncthreads();
+    P.prefetch(Ra, 0u);
+    if (two) P.prefetch(Rb, 0u);
+    P.x_from_bits(Ra, Rb, two, 0u);
+    __syncthreads();
+    P.template col_step1<false>(nullptr, 0);
+    __syncthreads();
+    P.col_product(a.ghat, L);
+    __syncthreads();
+    P.template col_inverse2<false>(nullptr, 0);
+    __syncthreads();
+    P.x_inverse1();
+    __syncthreads();
+    float err_a = 0.0f, err_b = 0.0f;
+    P.x_into_eps(Ra, Rb, two, 0u, err_a, err_b);
     record_change(err_a, err_b, two, true, Ra.ctr, Rb.ctr, s_err);
 }
 
-template <int L>
-cudaError_t launch_cta(const FftArgs &a, int pairs, cudaStream_t st)
+// The cubic lattice in three launches over L x L planes: x and y of a z-plane
+// from the bitmasks into the buffer (kStep 0); z of a (z, x) plane, the product
+// and back (1); y and x back into eps (2).  The buffer holds the slots as the
+// transforms leave them; only the product looks the wave numbers up.
+template <int L, int kStep>
+__global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftArgs a)
 {
-    const int smem = (L * (L + 1) + L) * (int)sizeof(float2);
-    const cudaError_t e = cudaFuncSetAttribute(fft_cta_kernel<L>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    extern __shared__ float2 s[];
+    __shared__ unsigned s_err[2];
+    constexpr int R1 = L / 8;
+    const Plane<L> P{s, s + L * Plane<L>::Ls};
+    const int p = blockIdx.x / L, o = blockIdx.x - p * L;
+    const DevReplica &Ra = a.reps[a.index[2 * p]];
+    const bool two = 2 * p + 1 < a.R;
+    const DevReplica &Rb = a.reps[a.index[two ? 2 * p + 1 : 2 * p]];
+    float2 *buf = a.buf + (size_t)p * L * L * L;
+    const unsigned site0 = (unsigned)(o * L * L);
+    P.twiddles(a.tw);
+    if (kStep == 2 && threadIdx.x < 2) s_err[threadIdx.x] = 0u;
+    __syncthreads();
+    if (kStep == 0) {
+        if (o == 0) clear_change(two, Ra.ctr, Rb.ctr);
+        P.x_from_bits(Ra, Rb, two, site0);
+        __syncthreads();
+        P.template col_step1<false>(nullptr, 0);
+        __syncthreads();
+        P.col_step2_store(buf + site0);
+    } else if (kStep == 1) {
+        // slot o of y holds wave number o / 8 + R1 (o mod 8)
+        const int ky = (o >> 3) + R1 * (o & 7);
+        float2 *g = buf + o * L;
+        P.template col_step1<true>(g, (size_t)L * L);
+        __syncthreads();
+        P.col_product(a.ghat + ky * L, (size_t)L * L);
+        __syncthreads();
+        P.template col_inverse2<true>(g, (size_t)L * L);
+    } else {
+        P.prefetch(Ra, site0);
+        if (two) P.prefetch(Rb, site0);
+        P.col_inverse1_load(buf + site0);
+        __syncthreads();
+        P.template col_inverse2<false>(nullptr, 0);
+        __syncthreads();
+        P.x_inverse1();
+        __syncthreads();
+        float err_a = 0.0f, err_b = 0.0f;
+        P.x_into_eps(Ra, Rb, two, site0, err_a, err_b);
+        record_change(err_a, err_b, two, o == 0, Ra.ctr, Rb.ctr, s_err);
+    }
+}
+
+template <int L>
+cudaError_t launch_square(const FftArgs &a, int pairs, cudaStream_t st)
+{
+    const cudaError_t e = cudaFuncSetAttribute(
+        fft_square_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, Plane<L>::kSmem);
     if (e) return e;
-    fft_cta_kernel<L><<<pairs, fft_cta_threads<L>(), smem, st>>>(a);
+    fft_square_kernel<L><<<pairs, Plane<L>::kT, Plane<L>::kSmem, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int L>
+cudaError_t launch_cubic(const FftArgs &a, int pairs, cudaStream_t st)
+{
+    // planes of up to 64 x 64 values: 33 KiB
+    fft_cubic_kernel<L, 0><<<pairs * L, Plane<L>::kT, Plane<L>::kSmem, st>>>(a);
+    fft_cubic_kernel<L, 1><<<pairs * L, Plane<L>::kT, Plane<L>::kSmem, st>>>(a);
+    fft_cubic_kernel<L, 2><<<pairs * L, Plane<L>::kT, Plane<L>::kSmem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -691,10 +865,16 @@ static int refresh_fft_lines(int L)
     return W;
 }
 
-// The sides the FFT refresh takes: 2^m (4 <= L <= 1024) or 3 2^m (6 <= L <= 192).
-bool refresh_fft_size_ok(int L)
+// Whether the transforms of this side clear the replicas' error records
+// themselves (else launch_reset_refresh_err comes first).
+bool refresh_fft_clears(int L, int dim) { return L % 8 == 0 && L >= 16 && L <= (dim == 3 ? 64 : 160); }
+
+// The sides the FFT refresh takes: 2^m (4 <= L <= 1024), 3 2^m (6 <= L <= 192)
+// and multiples of 8 (square 16 to 160, cubic 16 to 64).
+bool refresh_fft_size_ok(int L, int dim)
 {
     if (L >= 4 && L <= 1024 && (L & (L - 1)) == 0) return true;
+    if (refresh_fft_clears(L, dim)) return true;
     const int M = L / 3;
     return L % 3 == 0 && L >= 6 && L <= 192 && (M & (M - 1)) == 0;
 }
@@ -703,7 +883,7 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
                                int dim, const float *d_ghat, const float2 *d_tw, float2 *d_buf,
                                cudaStream_t st)
 {
-    if (R < 1 || !refresh_fft_size_ok(L) || (dim != 2 && dim != 3)) return cudaErrorInvalidValue;
+    if (R < 1 || !refresh_fft_size_ok(L, dim) || (dim != 2 && dim != 3)) return cudaErrorInvalidValue;
     FftArgs a;
     a.reps = d_reps;
     a.index = d_index;
@@ -711,7 +891,7 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
     a.L = L;
     const bool pow2 = (L & (L - 1)) == 0;
     a.log2L = pow2 ? __builtin_ctz((unsigned)L) : 0;
-    a.M3 = pow2 ? 0 : L / 3;
+    a.M3 = pow2 ? 0 : L / 3;              // (read by the passes alone)
     a.log2M = pow2 ? 0 : __builtin_ctz((unsigned)(L / 3));
     a.W = refresh_fft_lines(L);
     a.buf = d_buf;
@@ -722,19 +902,22 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
     const int groups = lines / a.W;
     cudaError_t e;
     if (dim == 2) {
-        // a pair per CTA where its values fit shared memory
+        // a pair per CTA where its values fit shared memory (206 KiB at L = 160)
         switch (L) {
-        case 16: return launch_cta<16>(a, pairs, st);
-        case 24: return launch_cta<24>(a, pairs, st);
-        case 32: return launch_cta<32>(a, pairs, st);
-        case 48: return launch_cta<48>(a, pairs, st);
-        case 64: return launch_cta<64>(a, pairs, st);
-        case 96: return launch_cta<96>(a, pairs, st);
-        case 128: return launch_cta<128>(a, pairs, st);
+#define CG_SIDE(n) case n: return launch_square<n>(a, pairs, st);
+        CG_SIDE(16) CG_SIDE(24) CG_SIDE(32) CG_SIDE(40) CG_SIDE(48) CG_SIDE(56) CG_SIDE(64)
+        CG_SIDE(72) CG_SIDE(80) CG_SIDE(88) CG_SIDE(96) CG_SIDE(104) CG_SIDE(112) CG_SIDE(120)
+        CG_SIDE(128) CG_SIDE(136) CG_SIDE(144) CG_SIDE(152) CG_SIDE(160)
+#undef CG_SIDE
         }
         if ((e = launch_pass<0>(a, 0, pairs, groups, st))) return e;
         if ((e = launch_pass<2>(a, 1, pairs, groups, st))) return e;
         return launch_pass<4>(a, 0, pairs, groups, st);
+    }
+    switch (L) {
+#define CG_SIDE(n) case n: return launch_cubic<n>(a, pairs, st);
+    CG_SIDE(16) CG_SIDE(24) CG_SIDE(32) CG_SIDE(40) CG_SIDE(48) CG_SIDE(56) CG_SIDE(64)
+#undef CG_SIDE
     }
     if ((e = launch_pass<0>(a, 0, pairs, groups, st))) return e;
     if ((e = launch_pass<1>(a, 1, pairs, groups, st))) return e;
