@@ -381,7 +381,7 @@ __device__ __forceinline__ bool lat_eval(const LatConst &K, unsigned kb, const P
         const bool theta = on[n] && !((wj >> (sj[n] & 31u)) & 1u);
         if constexpr (kFix) {
             // the high words: units of 2^-28, cut and rounded by at most
-            // 2^-28 + 2^-22 each below 4; the cut's slack covers it
+            // 2^-28 + 2^-22 each below 8; the cut's slack covers it
             const float fi = __int2float_rn(sm<int>(K.S.off_eps, 2 * si[n] + 1));
             const float fj = __int2float_rn(sm<int>(K.S.off_eps, 2 * sj[n] + 1));
             d[n] = fmaf(fj - fi, 0x1p-28f, -cv[n]) - K.slack;    // at most dH
@@ -815,10 +815,10 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
             }
         }
         if (kF64 && fixed) {
-            // an energy has reached 4 in size: back to binary64 before the
+            // an energy has reached 6 in size: back to binary64 before the
             // next hop could leave the integers' range of 8 (a hop moves it by
             // at most 1 per electron)
-            if (__syncthreads_or((int)(big >> 30) & 1)) {
+            if (__syncthreads_or(big >= kFixMost)) {
                 for (int l = tid; l < N; l += kThreads)
                     sm<double>(lay.off_eps, l) = fix_to_double(sm<long long>(lay.off_eps, l));
                 for (int l = tid; l < ntab; l += kThreads)

@@ -21,11 +21,13 @@ __device__ __forceinline__ T &sm(int off, int i = 0)
 // ---- binary64 energies in fixed point ----
 // GB300 adds binary64 numbers at 1/64 of its binary32 rate, and the update's
 // two adds per site were 63% of a hop of the L = 128 batch.  An energy that is
-// a multiple of 2^-60 below 4 in size, and the table's 1/r (a multiple of 2^-60
-// for r <= 256), are exact in a 64-bit integer of that unit, so the two
+// a multiple of 2^-60 below 6 in size, and the table's 1/r (a multiple of 2^-60
+// for r <= 256), are exact in a 64-bit integer of that unit (below 8: a hop moves
+// an energy by at most 1 per electron), so the two
 // roundings of eps + (1/r_lj - 1/r_li) become integer shifts and adds with the
 // same bits: an integer sum, rounded to 53 significant bits, ties to even.
 constexpr int kFixBits = 60;
+constexpr unsigned kFixMost = 6u << (kFixBits - 32);   // high word of the bound 6
 
 // Both conversions in integer arithmetic (the binary64 pipe is the slow one).
 __device__ __forceinline__ double fix_to_double(long long e)
@@ -40,32 +42,33 @@ __device__ __forceinline__ double fix_to_double(long long e)
 }
 
 // x as an integer of 2^-60; ok is cleared unless that is exact, sign of zero
-// included, and |x| < 4.
+// included, and |x| < 6.
 __device__ __forceinline__ long long fix_from_double(double x, bool &ok)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     if (b == 0) return 0;
     const int ex = (int)((b >> 52) & 0x7ffull), sh = ex - (1023 - kFixBits + 52);
     const unsigned long long m = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-    // ex <= 1024: below 4 (inf and NaN fail here); sh > -53: not below 2^-60
+    // ex <= 1025: below 8 (inf and NaN fail here); sh > -53: not below 2^-60
     // (subnormals and -0 fail here); no bit below 2^-60
-    if (ex > 1024 || sh <= -53 || (sh < 0 && (m & ((1ull << -sh) - 1ull)))) {
+    if (ex > 1025 || sh <= -53 || (sh < 0 && (m & ((1ull << -sh) - 1ull)))) {
         ok = false;
         return 0;
     }
     const long long e = (long long)(sh >= 0 ? m << sh : m >> -sh);
+    if ((unsigned)((unsigned long long)e >> 32) >= kFixMost) ok = false;
     return (b >> 63) ? -e : e;
 }
 
-// s rounded to 53 significant bits, ties to even; big gathers the high words
-// (bit 30 set: |s| >= 2^62).  The position of the leading bit is taken from
+// s rounded to 53 significant bits, ties to even; big takes the largest high word
+// (kFixMost or more: |s| may be 6 or more).  The position of the leading bit is taken from
 // the one's complement of a negative s: it differs from |s|'s for s = -2^k
 // alone, which either rounding keeps.
 __device__ __forceinline__ long long fix_round53(long long s, unsigned &big)
 {
     const unsigned lo = (unsigned)s, hi = (unsigned)((unsigned long long)s >> 32);
     const unsigned h = hi ^ (unsigned)((int)hi >> 31);
-    big |= h;
+    big = max(big, h);
     unsigned msb;
     asm("bfind.u32 %0, %1;" : "=r"(msb) : "r"(h));    // 0xffffffff for h = 0
     const int sh = max((int)msb - 20, 0);             // bits below the 53 kept (at most 10)

@@ -3,7 +3,7 @@
 * hop lists longer than the byte guide holds (more than 255 vectors), guide
   tables of every size, and steep towers whose buckets need the search;
 * binary64 energies in fixed point, back in binary64 in the middle of a run
-  (an energy of 4 or more), and never in it (a W that is no binary fraction);
+  (an energy of 6 or more), and never in it (a W that is no binary fraction);
 * batches of more replicas than SMs, where CTAs choose their replica;
 * the per-pair transforms of every side they are built for, and the binary64
   refresh of a group in one launch.
@@ -77,11 +77,13 @@ def test_chain_equals_the_oracle(B, case, threads):
 
 
 @pytest.mark.parametrize("L,dim", [(32, 2), (48, 2), (12, 3)])
-@pytest.mark.parametrize("W,shift", [(1.0, 0.0), (2.0, 3.0), (0.7, 0.0), (1.0, 5.0)],
-                         ids=["fixed", "to_binary64", "fine_phi", "never_fixed"])
+@pytest.mark.parametrize("W,shift", [(1.0, 0.0), (2.0, 3.0), (0.7, 0.0), (1.0, 5.0), (2.0, 3.6), (2.0, 3.95)],
+                         ids=["fixed", "fixed_past_4", "fine_phi", "never_fixed", "past_6_L48",
+                              "past_6_L32"])
 def test_fixed_point_energies(B, L, dim, W, shift):
-    # shift: a pattern of site energies that brings some eps near or past 4;
-    # with 3.0 the run starts below it and hops push single sites over
+    # shift: a pattern of site energies that brings some eps near or past 6, the
+    # fixed form's bound; with 3.6 (L = 48) and 3.95 (L = 32) the run starts
+    # below it and hops push single sites over
     p = dict(BASE, L=L, r_max=3, W=W, T=0.5)
     s = B.System([dict(p, dim=dim)], precision=B.CG_FP64)
     try:
