@@ -1810,6 +1810,32 @@ int cg_read_group_state(cg_handle *h, int group, uint32_t *occ_words_host, void 
     return CG_OK;
 }
 
+// Ones in `words` words, eight at a time through byte-wise sums that the compiler
+// turns into vector code (a count per word does not vectorise): a byte takes 8 from
+// each word, so a lane is folded after 31 of them at the latest.
+static long long count_ones(const uint32_t *w, int words)
+{
+    long long n = 0;
+    int q = 0;
+    while (q + 8 <= words) {
+        const int blocks = std::min((words - q) / 8, 31);
+        uint32_t sum[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        for (int b = 0; b < blocks; ++b, q += 8)
+            for (int j = 0; j < 8; ++j) {
+                uint32_t x = w[q + j];
+                x -= (x >> 1) & 0x55555555u;
+                x = (x & 0x33333333u) + ((x >> 2) & 0x33333333u);
+                sum[j] += (x + (x >> 4)) & 0x0f0f0f0fu;
+            }
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t s = (sum[j] & 0x00ff00ffu) + ((sum[j] >> 8) & 0x00ff00ffu);
+            n += (s & 0xffffu) + (s >> 16);
+        }
+    }
+    for (; q < words; ++q) n += __builtin_popcount(w[q]);
+    return n;
+}
+
 int cg_write_group_state(cg_handle *h, int group, const uint32_t *occ_words_host,
                          const void *eps_host, const cg_counters *c_host)
 {
@@ -1823,8 +1849,7 @@ int cg_write_group_state(cg_handle *h, int group, const uint32_t *occ_words_host
         for (size_t k = 0; k < cnt; ++k) {
             const Rep &r = h->reps[h->order[g.first + (int)k]];
             const uint32_t *w = occ_words_host + k * r0.words;
-            long long n = 0;
-            for (int q = 0; q < r0.words; ++q) n += __builtin_popcount(w[q]);
+            const long long n = count_ones(w, r0.words);
             if ((r0.N & 31) && (w[r0.words - 1] >> (r0.N & 31)))
                 return fail(CG_ESTATE, "occupation bits beyond the last site");
             if (n != (long long)std::floor(r.d.nu * r.N + 0.5))
