@@ -314,10 +314,6 @@ struct Group {
 // of sm_100-class GPUs less 1 KiB for its static barriers
 constexpr int kTcSmemLimit = 227 * 1024 - 1024;
 
-// Whether a group of `count` binary32 replicas of side L and dimension dim
-// refreshes on the tensor cores: the site count must be a multiple of 128 and
-// the contraction's stages plus the folded table must fit one CTA's shared
-// memory.
 // In-place DFT (exponent -2 pi i j k / n) of n complex values at stride
 // `stride`, binary64, for the refresh's host-side table: radix 2 for n = 2^m,
 // otherwise halved down to the odd part and the plain sum of that.
@@ -410,23 +406,37 @@ void build_fft_tables(Tables &t)
     }
 }
 
-// Whether a group of binary32 replicas of side L refreshes by the FFT:
-// L = 2^m or 3 2^m (CG_REFRESH_AUTO or CG_REFRESH_FFT).
-bool group_uses_fft(const cg_opts &o, int L, int dim)
-{
-    if (o.precision != CG_FP32 || !refresh_fft_size_ok(L, dim)) return false;
-    if (dim != 2 && dim != 3) return false;
-    return o.refresh_kind == CG_REFRESH_AUTO || o.refresh_kind == CG_REFRESH_FFT;
-}
-
-bool group_uses_tc(const cg_opts &o, int L, int count, int dim)
+// Whether the tensor cores can refresh a group of `count` binary32 replicas of
+// side L and dimension dim: the site count must be a multiple of 128 and the
+// contraction's stages plus the folded table must fit one CTA's shared memory.
+bool tc_fits(int L, int count, int dim)
 {
     const long long N = dim == 3 ? (long long)L * L * L : (long long)L * L;
     const int H1 = L / 2 + 1, tab = dim == 3 ? H1 * H1 * H1 : H1 * H1;
     const int R_pad = (std::min(count, refresh_tc_max_replicas(dim)) + 15) / 16 * 16;
-    if (o.precision != CG_FP32 || N % 128 != 0) return false;
-    if (refresh_tc_smem_bytes(R_pad, tab) > kTcSmemLimit) return false;
-    if (group_uses_fft(o, L, dim)) return false;
+    return N % 128 == 0 && refresh_tc_smem_bytes(R_pad, tab) <= kTcSmemLimit;
+}
+
+// Whether a group of `count` binary32 replicas of side L refreshes by the FFT:
+// sides 2^m and 3 2^m (CG_REFRESH_AUTO or CG_REFRESH_FFT), and the other
+// sides of the per-plane transforms where the automatic choice would be the
+// contraction, whose error is twenty times as large (rms at L = 112: 7e-6; 128
+// replicas: 329 us a resume with the contraction, 135 with the transforms).
+// Where it would be the binary64 sum it stays that, the more exact one (L = 40:
+// 4e-8).
+bool group_uses_fft(const cg_opts &o, int L, int count, int dim)
+{
+    if (o.precision != CG_FP32 || (dim != 2 && dim != 3)) return false;
+    if (o.refresh_kind != CG_REFRESH_AUTO && o.refresh_kind != CG_REFRESH_FFT) return false;
+    if (refresh_fft_size_ok(L)) return true;
+    return o.refresh_kind == CG_REFRESH_AUTO && refresh_fft_plane(L, dim) && count >= 8 &&
+           tc_fits(L, count, dim);
+}
+
+bool group_uses_tc(const cg_opts &o, int L, int count, int dim)
+{
+    if (o.precision != CG_FP32 || !tc_fits(L, count, dim)) return false;
+    if (group_uses_fft(o, L, count, dim)) return false;
     if (o.refresh_kind == CG_REFRESH_BF16X2) return true;
     if (o.refresh_kind == CG_REFRESH_AUTO) return count >= 8;
     return false;
@@ -988,7 +998,7 @@ size_t plan_bytes(int R, const cg_replica_desc *reps, const cg_opts &o)
     size_t tc_total = 0;
     for (auto &g : groups) tc_total += up(sched_bytes(std::get<2>(g)));
     for (auto &g : groups)
-        if (group_uses_fft(o, std::get<0>(g), std::get<1>(g))) {
+        if (group_uses_fft(o, std::get<0>(g), std::get<2>(g), std::get<1>(g))) {
             const size_t L = (size_t)std::get<0>(g);
             const size_t N = std::get<1>(g) == 3 ? L * L * L : L * L;
             tc_total += up(refresh_fft_buffer_bytes((int)N, std::get<2>(g))) + up(N * 4) +
@@ -1161,7 +1171,11 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
                 destroy_partial();
                 return nullptr;
             }
-            if (!r.random && group_uses_fft(o, r.d.L, dim_of(r.d))) build_fft_tables(*t);
+            int count = 0;                    // lattice replicas of this L and dim
+            for (int m = 0; m < R; ++m)
+                count += reps[m].sites != CG_SITES_RANDOM && reps[m].L == r.d.L &&
+                         dim_of(reps[m]) == dim_of(r.d);
+            if (!r.random && group_uses_fft(o, r.d.L, count, dim_of(r.d))) build_fft_tables(*t);
             r.tab = t.get();
             h->tables.push_back(std::move(t));
         }
@@ -1310,7 +1324,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
             destroy_partial();
             return nullptr;
         }
-        g.fft = !g.random && group_uses_fft(o, g.L, g.dim);
+        g.fft = !g.random && group_uses_fft(o, g.L, g.count, g.dim);
         if (g.fft && dalloc(h.get(), (void **)&g.d_fft,
                             refresh_fft_buffer_bytes(dim_of(h->reps[order[g.first]].d) == 3
                                                          ? g.L * g.L * g.L : g.L * g.L,
@@ -1399,7 +1413,7 @@ int refresh_group(cg_handle *h, const Group &g, cudaStream_t st)
         }
         return CG_OK;
     }
-    if (!(g.fft && refresh_fft_clears(g.L, g.dim)))
+    if (!(g.fft && refresh_fft_plane(g.L, g.dim)))
         CG_CUDA(launch_reset_refresh_err(h->d_reps, h->d_index + g.first, g.count, st));
     if (g.fft) {
         const Tables &t = *h->reps[h->order[g.first]].tab;

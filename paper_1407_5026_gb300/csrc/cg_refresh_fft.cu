@@ -6,7 +6,10 @@
 // two replicas share one complex transform: z = a + i b (a, b = n - nu of the
 // two) gives IDFT(DFT(z) . DFT(g)) = (a * g) + i (b * g).
 //
-// L = 2^m or 3 2^m.  Transforms in binary32 along one axis per pass, W lines
+// Two forms.  The sides of refresh_fft_plane keep a whole plane in one CTA (below,
+// "Planes in one CTA").  The other
+// sides 2^m and 3 2^m (the smallest ones and those past that range) run in
+// passes: transforms in binary32 along one axis per pass, W lines
 // per CTA in shared memory.  L = 2^m: a forward pass loads in bit-reversed
 // order and runs radix-2 decimation-in-time butterflies (natural-order
 // output); an inverse pass runs decimation-in-frequency butterflies on
@@ -340,13 +343,16 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
 }
 
 // ---------------------------------------------------------------------------
-// Sides that are multiples of 8, square lattices of L = 16 to 160 and cubic ones
-// of 16 to 64.  On the square lattice one CTA does the whole refresh of a replica
+// Planes in one CTA: refresh_fft_plane's sides.  On the square lattice one CTA does the whole refresh of a replica
 // pair: its L x L complex values stay in shared memory (132 KiB at L = 128)
 // through all the transforms, where the passes above write and read them through
 // L2 between launches and run a barrier per radix-2 stage (304 replicas of
 // L = 128: 0.225 -> 0.085 ms).  Cubic lattices take three launches over planes
-// instead of five passes.
+// instead of five passes (152 of 32^3: 0.243 -> 0.067 ms; 16 of 48^3: 0.104 ->
+// 0.050).  Sides that are neither 2^m nor 3 2^m take the place of
+// the tensor-core contraction (128 of L = 112, a resume with its copies: 329 ->
+// 135 us).  What bounds it: latency of the seven sweeps and their barriers at one
+// or two CTAs per SM, then the 18 N bytes of phi, eps and table from memory.
 //
 // A line of L = R1 8 elements transforms in two steps, in place:
 //     X[c + R1 d] = sum_b W_8^(b d) W_L^(b c) sum_a W_R1^(a c) x[8 a + b]
@@ -375,6 +381,18 @@ template <bool kInv>
 __device__ __forceinline__ float2 ctw(float2 v, float wr, float wi)
 {
     return cmul(v, make_float2(wr, kInv ? wi : -wi));
+}
+
+// v times exp(-i pi / 4) (inverse: exp(i pi / 4)): the sums first (exact for the
+// first axis' n - nu), then 1/sqrt 2 in two parts, one rounding each.
+template <bool kInv>
+__device__ __forceinline__ float2 rot45(float2 v)
+{
+    constexpr float kS = 0.7071067811865476f;
+    constexpr float kSlo = (float)(0.70710678118654752440 - (double)kS);
+    const float a = v.x + v.y, b = kInv ? v.x - v.y : v.y - v.x;
+    const float sa = fmaf(a, kS, a * kSlo), sb = fmaf(b, kS, b * kSlo);
+    return kInv ? make_float2(sb, sa) : make_float2(sa, sb);
 }
 
 template <bool kInv>
@@ -434,9 +452,9 @@ __device__ __forceinline__ void dft(float2 (&v)[R])
     } else if constexpr (R == 8) {
         dft4<kInv>(v[0], v[2], v[4], v[6]);
         dft4<kInv>(v[1], v[3], v[5], v[7]);
-        v[3] = ctw<kInv>(v[3], kS, kS);
+        v[3] = rot45<kInv>(v[3]);
         v[5] = rot90<kInv>(v[5]);
-        v[7] = ctw<kInv>(v[7], -kS, kS);
+        v[7] = rot45<kInv>(rot90<kInv>(v[7]));
         float2 o[8];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -865,25 +883,31 @@ static int refresh_fft_lines(int L)
     return W;
 }
 
-// Whether the transforms of this side clear the replicas' error records
-// themselves (else launch_reset_refresh_err comes first).
-bool refresh_fft_clears(int L, int dim) { return L % 8 == 0 && L >= 16 && L <= (dim == 3 ? 64 : 160); }
-
-// The sides the FFT refresh takes: 2^m (4 <= L <= 1024), 3 2^m (6 <= L <= 192)
-// and multiples of 8 (square 16 to 160, cubic 16 to 64).
-bool refresh_fft_size_ok(int L, int dim)
+// The sides 2^m (4 <= L <= 1024) and 3 2^m (6 <= L <= 192).
+bool refresh_fft_size_ok(int L)
 {
     if (L >= 4 && L <= 1024 && (L & (L - 1)) == 0) return true;
-    if (refresh_fft_clears(L, dim)) return true;
     const int M = L / 3;
     return L % 3 == 0 && L >= 6 && L <= 192 && (M & (M - 1)) == 0;
+}
+
+// Sides of the per-plane transforms: multiples of 16 to 160 and 24 (square), and
+// 16, 24, 32, 48, 64 (cubic: at 40 and 56 the contraction's binary16 split is the
+// more exact).  They clear the replicas' error records themselves (else
+// launch_reset_refresh_err comes first).
+bool refresh_fft_plane(int L, int dim)
+{
+    if (L == 24 && dim == 2) return true;
+    if (dim == 3) return refresh_fft_size_ok(L) && L >= 16 && L <= 64;
+    return L % 16 == 0 && L >= 16 && L <= 160;
 }
 
 cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int R, int L,
                                int dim, const float *d_ghat, const float2 *d_tw, float2 *d_buf,
                                cudaStream_t st)
 {
-    if (R < 1 || !refresh_fft_size_ok(L, dim) || (dim != 2 && dim != 3)) return cudaErrorInvalidValue;
+    if (!d_ghat || !d_tw || !d_buf) return cudaErrorInvalidValue;
+    if (R < 1 || !(refresh_fft_size_ok(L) || refresh_fft_plane(L, dim)) || (dim != 2 && dim != 3)) return cudaErrorInvalidValue;
     FftArgs a;
     a.reps = d_reps;
     a.index = d_index;
@@ -905,9 +929,8 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
         // a pair per CTA where its values fit shared memory (206 KiB at L = 160)
         switch (L) {
 #define CG_SIDE(n) case n: return launch_square<n>(a, pairs, st);
-        CG_SIDE(16) CG_SIDE(24) CG_SIDE(32) CG_SIDE(40) CG_SIDE(48) CG_SIDE(56) CG_SIDE(64)
-        CG_SIDE(72) CG_SIDE(80) CG_SIDE(88) CG_SIDE(96) CG_SIDE(104) CG_SIDE(112) CG_SIDE(120)
-        CG_SIDE(128) CG_SIDE(136) CG_SIDE(144) CG_SIDE(152) CG_SIDE(160)
+        CG_SIDE(16) CG_SIDE(24) CG_SIDE(32) CG_SIDE(48) CG_SIDE(64) CG_SIDE(80) CG_SIDE(96)
+        CG_SIDE(112) CG_SIDE(128) CG_SIDE(144) CG_SIDE(160)
 #undef CG_SIDE
         }
         if ((e = launch_pass<0>(a, 0, pairs, groups, st))) return e;
@@ -916,7 +939,7 @@ cudaError_t launch_refresh_fft(const DevReplica *d_reps, const int *d_index, int
     }
     switch (L) {
 #define CG_SIDE(n) case n: return launch_cubic<n>(a, pairs, st);
-    CG_SIDE(16) CG_SIDE(24) CG_SIDE(32) CG_SIDE(40) CG_SIDE(48) CG_SIDE(56) CG_SIDE(64)
+    CG_SIDE(16) CG_SIDE(24) CG_SIDE(32) CG_SIDE(48) CG_SIDE(64)
 #undef CG_SIDE
     }
     if ((e = launch_pass<0>(a, 0, pairs, groups, st))) return e;

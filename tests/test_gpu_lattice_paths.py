@@ -128,14 +128,18 @@ def test_batches_past_one_replica_per_sm(B, R):
         s.close()
 
 
-@pytest.mark.parametrize("L,dim", [(L, 2) for L in range(16, 161, 8)] +
-                         [(L, 3) for L in range(16, 65, 8)])
-@pytest.mark.parametrize("R", [1, 4])
+@pytest.mark.parametrize("L,dim", [(L, 2) for L in [24] + list(range(16, 161, 16))] +
+                         [(L, 3) for L in (16, 24, 32, 48, 64)])
+@pytest.mark.parametrize("R", [1, 4, 9])
 def test_transform_refresh_of_a_pair(B, L, dim, R):
-    if dim == 3 and L > 32 and R > 1:
+    # sides that are neither 2^m nor 3 2^m go by the transforms from 8 replicas on
+    fast = L in (16, 24, 32, 48, 64, 96, 128)
+    if fast == (R == 9):
+        pytest.skip("not by the transforms" if R < 9 else "covered by 1 and 4")
+    if fast and dim == 3 and L > 32 and R > 1:
         R = 2
     reps = [dict(BASE, L=L, r_max=3, seed=s, replica=s, nu=0.25, dim=dim) for s in range(R)]
-    s = B.System(reps, precision=B.CG_FP32, refresh_kind=B.CG_REFRESH_FFT)
+    s = B.System(reps, precision=B.CG_FP32, refresh_kind=B.CG_REFRESH_AUTO)
     try:
         assert s.run(60, 512) == B.CG_OK
         before = [s.state(k)[1] for k in range(R)]
