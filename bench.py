@@ -50,7 +50,8 @@ TRAFFIC_CAPTURE = {"sources_sha256_16": "651cca43504ee42b", "bytes_per_launch": 
 def kernel_sources_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("cg_pr_kernel.cu", "cg_pr_persistent.cuh", "cg_pr_common.cuh", "cg_device.cuh"):
+    for f in ("cg_pr_kernel.cu", "cg_pr_lattice.cuh", "cg_pr_update.cuh", "cg_pr_common.cuh",
+              "cg_device.cuh"):
         with open(os.path.join(ROOT, "paper_1407_5026_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -151,7 +152,7 @@ def workload_config(args, R):
                   else "autotuned from {1024, 4096, 16384, 65536} (relaxing with "
                        f"{args.M})"),
             "refresh": "every 1024 hops: eps from its definition by the convolution "
-                       "theorem (binary32 radix-2 FFTs, two replicas per complex "
+                       "theorem (binary32 FFTs, two replicas per complex "
                        "transform, times DFT(1/r); phi added in binary64)",
             "l2": "256 MB buffer zeroed between steps (outside the timed events)",
             "state": f"chains relaxed {args.relax_steps * HOPS_PER_STEP} hops from "
@@ -463,7 +464,7 @@ def run_ours(args):
                                              for k in ("threads", "cluster")))
                                  else None),
                      "traffic_unit": "DRAM bytes per launch (ncu capture)",
-                     "kernel": "pr_persistent<float>",
+                     "kernel": "pr_lattice<float>",
                      "bytes_per_hop": bytes_per_hop,
                      # the strict lower bound: the eps read-modify-write alone
                      # (2 s N bytes per hop, the two table reads counted as free)
@@ -488,16 +489,16 @@ def run_ours(args):
         # over the share of the CTAs' cycles spent in label rounds
         "rejection_roofline": rejection_roofline(evaluated, sum(run_ms) * 1e-3, cyc_rej,
                                                  cyc_upd, philox_peak),
-        # the refresh as a whole (error reset and the three FFT passes)
+        # the refresh as a whole (one launch)
         # against the measured HBM copy rate
         "refresh_roofline": refresh_roofline(N, R, statistics.mean(ref_ms)),
         "phase_split": {"refresh_ms_per_step": statistics.mean(ref_ms),
                         "run_ms_per_step": statistics.mean(run_ms),
                         "update_cycles_frac": cyc_upd / max(1, cyc_upd + cyc_rej),
                         "max_eps_err_last_refresh": max_err},
-        # per step: one persistent launch per L, then the refresh: error reset
-        # and three FFT passes
-        "gpu_launches": args.steps * (1 + 4),
+        # per step: the launch that orders the replicas by expected work, the
+        # persistent launch and the refresh
+        "gpu_launches": args.steps * 3,
         "clocks": clk,
         "peaks_measured": {"barrier_us_by_ctas": {str(c): v for c, v in barrier_us.items()},
                            "smem_rmw32_GBps": smem_peak / 1e9, "dadd_per_s": dadd_peak,
@@ -685,15 +686,14 @@ def rejection_roofline(evaluated, run_s, cyc_rej, cyc_upd, philox_peak):
             "rejection_cycle_share": share,
             "peak_source": "measured: Philox-4x32-10 blocks/s of the PR kernels' label "
                            "generator on all SMs (cg_microbench kind 3)",
-            "kernel": "pr_persistent<float>"}
+            "kernel": "pr_lattice<float>"}
 
 
 def refresh_roofline(N, R, ms):
     """The FFT refresh's bytes per replica and refresh: the occupation bits
-    (N/8), four sweeps of its half of the complex transform buffer (4 x 4 N:
-    written by the first pass, read and written by the second, read by the
-    third), half of DFT(g)/N (2 N, one read per replica pair), phi (8 N) and
-    eps read and written (8 N), against the measured HBM copy rate."""
+    (N/8), half of DFT(g)/N (2 N, one read per replica pair), phi (8 N) and
+    eps read and written (8 N), against the measured HBM copy rate (a pair's
+    transform stays in its CTA's shared memory)."""
     peaks = {}
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -704,11 +704,11 @@ def refresh_roofline(N, R, ms):
         peak, src = float(peaks["hbm_gbs"]), "of measured (MEASURED_PEAKS.json hbm_gbs)"
     else:
         peak, src = 6800.0, "of fallback (6.8 TB/s)"
-    per_replica = N / 8.0 + 16.0 * N + 2.0 * N + 8.0 * N + 8.0 * N
+    per_replica = N / 8.0 + 2.0 * N + 8.0 * N + 8.0 * N
     achieved = per_replica * R / (ms * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_source": src,
-            "kernel": "fft_pass_kernel x 3 (+ error reset)",
+            "kernel": "fft_square_kernel",
             "bytes_per_refresh": per_replica * R}
 
 

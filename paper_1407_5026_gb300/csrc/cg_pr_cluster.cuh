@@ -2,7 +2,15 @@
 // whose local energies do not fit one CTA's shared memory (e.g. L = 256 in
 // binary32, 256 KiB of eps): one replica per thread-block cluster of C CTAs.
 //
-// Same chain as cg_pr_kernel.cu (mixed PR algorithm, steps 1-3); the work of
+// What bounds it: the two cluster barriers of a hop and the short chains of
+// shared and distributed loads between them; the issue slots are 38% busy.  512
+// threads leave a label 128 registers and cost less per barrier than 1024 (L =
+// 256 on 4 CTAs 4.1 against 4.7 ms; 256 threads 4.7: too few warps to hide the
+// update's loads).  With the label code of the one-CTA kernel, one CTA barrier
+// per chunk and candidates sent by a lane each, ms per run call before and
+// after: 16 replicas of L = 256 5.68 -> 4.24; 48^3 2.47 -> 1.64.
+//
+// Same chain as cg_pr_lattice.cuh (mixed PR algorithm, steps 1-3); the work of
 // a replica is spread over the cluster:
 //   * on the square lattice CTA `rank` owns the base rows
 //     [rank B, (rank+1) B), B = L/(2C), and their partner rows y + L/2 of eps
@@ -15,8 +23,8 @@
 //   * a chunk of labels is split into C contiguous sub-ranges, CTA rank
 //     evaluating sub-range rank; eps_i and eps_j of a proposal are read from
 //     the owning CTA's shared memory through distributed shared memory;
-//   * each CTA finds its lowest accepting label (OR barrier, ballot, warp
-//     minimum), then thread 0 writes it and its payload into every CTA's
+//   * each CTA finds its lowest accepting label (ballot, shared minimum), then
+//     lane r of a warp writes it and its payload into CTA r's
 //     exchange slot (double-buffered by chunk parity); one cluster barrier
 //     later every CTA holds all C candidates and takes the minimum, so the
 //     executed hop is the lowest accepting label of the whole chunk;

