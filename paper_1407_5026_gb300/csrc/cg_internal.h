@@ -87,8 +87,8 @@ struct alignas(16) DevReplica {
     // random-site geometry (CG_SITES_RANDOM; null otherwise)
     const double *G;          // N x N minimum-image 1/r, 0 on the diagonal
     const int *rguide;        // 16 ints per site: kRandomGuide layout
-    const uint32_t *rw;       // per pair: C - 1 (random_weight_count entries)
-    const uint2 *rj;          // per pair: partner j, 1/r + E dx in binary32
+    const uint32_t *rw;       // per pair: C - 1
+    const uint32_t *rj;       // per pair: random_partner_word
     const double2 *rgx;       // per pair: 1/r, E dx (minimum-image dx, binary64)
     int rguide_small;         // 1: every partner list holds at most 255 pairs
 };
@@ -221,9 +221,15 @@ cudaError_t set_pr_random_smem_limit(int bytes);
 // The offsets are 16 bits: the library refuses lists of 2^16 or more pairs.
 constexpr int kRandomGuide = 16;
 constexpr int kRandomBuckets = 16;
-// The running weights are read in aligned groups of four, up to eleven past the
-// first of a window: the array is padded by that.
-inline size_t random_weight_count(size_t pairs) { return (pairs + 15) / 4 * 4; }
+// A pair's partner (17 bits: N <= 131072) and, in the upper 15 bits, sign, exponent
+// and six bits of 1/r + E dx, rounded up: the chain's first look at a label needs a
+// bound on dH from below only.  Weight and this word take 8 bytes per pair.
+constexpr uint32_t kPartnerMask = (1u << 17) - 1;
+inline uint32_t random_partner_word(unsigned j, uint32_t cv_bits)
+{
+    const uint32_t up = cv_bits >> 31 ? cv_bits : cv_bits + kPartnerMask;
+    return (up & ~kPartnerMask) | j;
+}
 // Sites whose eps a CTA of a C-CTA cluster owns: ceil(N / C) rounded up to a
 // multiple of 32 (CTA rank owns [rank Nc, min(N, (rank + 1) Nc))).
 __host__ __device__ inline int random_cluster_sites(int N, int C)

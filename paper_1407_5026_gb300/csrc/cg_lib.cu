@@ -280,8 +280,8 @@ struct Rep {
     double Zmax = 0.0;
     double *d_px = nullptr, *d_py = nullptr, *d_G = nullptr;
     int *d_guide = nullptr;           // kRandomGuide ints per site
-    uint32_t *d_rw = nullptr;         // running weight less 1 of each pair
-    uint2 *d_rj = nullptr;            // partner and binary32 1/r + E dx of each pair
+    uint32_t *d_rw = nullptr;         // running weight less 1 of each pair, then the
+                                      // pairs' random_partner_words
     double2 *d_rgx = nullptr;         // 1/r and E dx of each pair
     bool pair = false;                // the handle proposes two-electron hops
     // random sites: every partner list holds at most 255 pairs, and on one
@@ -709,31 +709,31 @@ void fill_dev(const Rep &r, const cg_opts &o, DevReplica &dr, cg_hop *log)
     dr.C0 = t.C0;
     dr.eps = r.d_eps; dr.occ = r.d_occ; dr.phi = r.d_phi; dr.ctr = r.d_ctr;
     dr.log = log;
-    dr.G = r.d_G; dr.rguide = r.d_guide; dr.rw = r.d_rw; dr.rj = r.d_rj; dr.rgx = r.d_rgx;
+    dr.G = r.d_G; dr.rguide = r.d_guide; dr.rw = r.d_rw; dr.rj = r.d_rw + r.rj.size();
+    dr.rgx = r.d_rgx;
     dr.rguide_small = r.guide_small ? 1 : 0;
 }
 
 // The device form of a random-site replica's partner lists: per site the
 // kRandomGuide record (list bounds, the pair each x1 bucket starts at, the
 // last running weight), per pair its running weight less 1 (C - 1: 32 bits,
-// 1 <= C <= 2^32; padded to whole loads), (j, 1/r + E dx in binary32) and
-// (1/r, E dx).
+// 1 <= C <= 2^32), after them all its partner word, and (1/r, E dx).
 void pack_random(const Rep &r, std::vector<int> &guide, std::vector<uint32_t> &rw,
-                 std::vector<uint32_t> &rj, std::vector<double> &rgx)
+                 std::vector<double> &rgx)
 {
     const int N = r.N;
     const size_t m = r.rj.size();
     guide.assign((size_t)N * kRandomGuide, 0);
-    rw.assign(random_weight_count(m), 0xffffffffu);
-    rj.assign(2 * m, 0u);
+    rw.assign(2 * m, 0u);
     rgx.assign(2 * m, 0.0);
     for (size_t k = 0; k < m; ++k) {
         // C_k = 0 (weights below 2^-32 at the head of a list) selects no x1 and
         // is never reached from a bucket's start; 0 keeps the order
         rw[k] = r.rC[k] ? (uint32_t)(r.rC[k] - 1) : 0u;
-        rj[2 * k] = r.rj[k];
         const float cv = (float)(r.rg[k] + r.redx[k]);
-        std::memcpy(&rj[2 * k + 1], &cv, 4);
+        uint32_t bits;
+        std::memcpy(&bits, &cv, 4);
+        rw[m + k] = random_partner_word(r.rj[k], bits);
         rgx[2 * k] = r.rg[k];
         rgx[2 * k + 1] = r.redx[k];
     }
@@ -1024,7 +1024,7 @@ size_t plan_bytes(int R, const cg_replica_desc *reps, const cg_opts &o)
             const size_t cnt = build_random(tmp) == CG_OK ? tmp.rj.size() : 0;
             const size_t c1 = cnt ? cnt : 1;
             total += 2 * up(N * 8) + up(N * N * 8) + up(N * kRandomGuide * 4) +
-                     up(random_weight_count(c1) * 4) + up(c1 * 8) + up(c1 * 16);
+                     up(c1 * 8) + up(c1 * 16);
         }
         auto key = std::make_tuple(d.L, d.r_max, d.xi, dim_of(d));
         if (std::find(seen.begin(), seen.end(), key) == seen.end()) {
@@ -1226,21 +1226,19 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         if (dalloc(h.get(), (void **)&r.d_px, N * 8) || dalloc(h.get(), (void **)&r.d_py, N * 8) ||
             dalloc(h.get(), (void **)&r.d_G, N * N * 8) ||
             dalloc(h.get(), (void **)&r.d_guide, N * kRandomGuide * 4) ||
-            dalloc(h.get(), (void **)&r.d_rw, random_weight_count(cnt) * 4) ||
-            dalloc(h.get(), (void **)&r.d_rj, cnt * 8) ||
+            dalloc(h.get(), (void **)&r.d_rw, cnt * 8) ||   // (a multiple of 256 bytes)
             dalloc(h.get(), (void **)&r.d_rgx, cnt * 16)) { destroy_partial(); return nullptr; }
         const size_t m = r.rj.size();
         std::vector<int> guide;
-        std::vector<uint32_t> rw, rj;
+        std::vector<uint32_t> rw;
         std::vector<double> rgx;
-        pack_random(r, guide, rw, rj, rgx);
+        pack_random(r, guide, rw, rgx);
         cudaMemcpyAsync(r.d_px, r.px.data(), N * 8, cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(r.d_py, r.py.data(), N * 8, cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(r.d_guide, guide.data(), N * kRandomGuide * 4, cudaMemcpyHostToDevice,
                         h->st);
         if (m) {
             cudaMemcpyAsync(r.d_rw, rw.data(), rw.size() * 4, cudaMemcpyHostToDevice, h->st);
-            cudaMemcpyAsync(r.d_rj, rj.data(), m * 8, cudaMemcpyHostToDevice, h->st);
             cudaMemcpyAsync(r.d_rgx, rgx.data(), m * 16, cudaMemcpyHostToDevice, h->st);
         }
         if (launch_g_build(r.d_px, r.d_py, r.d.L, r.N, r.d_G, h->st) != cudaSuccess) {

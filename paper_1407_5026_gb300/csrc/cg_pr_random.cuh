@@ -14,7 +14,7 @@ struct RCand {
 
 struct RLabel {
     unsigned i, j, m, x2;     // m: the pair's index
-    float cv;                 // 1/r_ij + E dx_ij in binary32
+    float cv;                 // 1/r_ij + E dx_ij or up to 1/64 of it above
     bool theta;
 };
 
@@ -25,8 +25,8 @@ struct RLabel {
 // proposal) and the bucket of pairs x1 >> 28 can select; a four-way search
 // (three independent probes per step) narrows a bucket of more than eight, and
 // the rest is counted from up to three aligned loads of four weights (C_m - 1,
-// 32 bits).  The chosen pair's partner and its binary32 1/r + E dx come with one
-// more load.  (Reading whole records with 1/r and E dx beside the weights took
+// 32 bits).  The chosen pair's partner and a bound on its 1/r + E dx come with one
+// more load of 4 bytes.  (Reading whole records with 1/r and E dx beside the weights took
 // seven sectors per label for these four; the L1's tag stage was the second
 // stall of the kernel, tex_throttle 3.5 per issue.)
 // gsm: the compacted guide records in shared memory (two uint4 per site:
@@ -108,6 +108,8 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
     }
     // the pairs of [lo, hi - 1) with C_m <= x1 come before the answer (the
     // weights rise along the list); a window of up to 11 from the group lo is in
+    // (the last group may read up to three words past the weights, where the
+    // partners' lie; they do not count)
     const int base = lo & ~3;
     const uint4 *r4 = reinterpret_cast<const uint4 *>(rw + base);
     const uint4 wa = __ldg(r4);
@@ -121,10 +123,10 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
         const int e = base + t;
         m += (e >= lo && e < hi - 1 && w[t] < w1) ? 1 : 0;
     }
-    const uint2 rc = __ldg(Rg.rj + m);
+    const uint32_t rc = __ldg(Rg.rj + m);
     p.m = (unsigned)m;
-    p.j = rc.x;
-    p.cv = __uint_as_float(rc.y);
+    p.j = rc & kPartnerMask;
+    p.cv = __uint_as_float(rc & ~kPartnerMask);
     p.theta = !((occ[p.j >> 5] >> (p.j & 31)) & 1u);     // n_i = 1 here
     return p;
 }
