@@ -14,7 +14,8 @@
 // What bounds it: the dependent loads of a label (guide record, weights,
 // partner) from L2 and HBM.  Weights of 32 bits apart from the partners cost a
 // label four sectors where whole pair records cost seven; with the rejection
-// decided in binary32 (24 replicas of L = 64, ms per run call): 4.40 -> 3.95.
+// decided in binary32 (24 replicas of L = 64, ms per run call): 4.40 -> 3.95; with
+// weight and partner in 8 bytes, the partner's word bounding dH: 3.93.
 //
 // pr_random: one CTA per replica, binary64; eps and the occupation bitmask in
 // shared memory, the partner lists (a 64-byte guide record per site; weights,
