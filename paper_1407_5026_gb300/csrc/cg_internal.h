@@ -184,14 +184,18 @@ __host__ __device__ inline LatLayout lat_layout(int N, int tab_entries, int V, i
     return s;
 }
 
+// Shared memory a kernel may not take dynamically: its static part (the
+// cluster kernel's exchange slots take it past 2 KiB with two-electron hops).
+inline int lat_static_bytes(bool pair) { return pair ? 3072 : 2048; }
+
 // Guide bits of that kernel: a finer table sends fewer labels to the search
 // (about 0.5% of x1's range at 14 bits, 1% at 13 for r_max = 8), so the
 // largest of 14, 13 and 12 that costs no CTA per SM (228 KiB of shared memory,
-// at most four CTAs of 256 threads by registers) and fits the 227 KiB of one
-// CTA with room for the static part.  12 bits take less than the two-electron
-// kernel's layout, so a lattice that fits that one fits this.
-constexpr int kLatSmemMost = 227 * 1024 - 2048;
-inline int lat_guide_bits(int N, int tab_entries, int V, int words, int real_bytes)
+// at most four CTAs of 256 threads by registers) and fits `most` bytes, the
+// room the lattice is admitted by.  12 bits take less than smem_layout, so a
+// lattice that fits that layout fits this one.
+constexpr int kSmemPerCta = 227 * 1024;
+inline int lat_guide_bits(int N, int tab_entries, int V, int words, int real_bytes, int most)
 {
     auto total = [&](int b) { return lat_layout(N, tab_entries, V, words, real_bytes, b).total; };
     auto ctas = [&](int b) {
@@ -199,7 +203,7 @@ inline int lat_guide_bits(int N, int tab_entries, int V, int words, int real_byt
         return c < 4 ? c : 4;
     };
     for (int b = kLatGuideBits; b > 12; --b)
-        if (total(b) <= kLatSmemMost && ctas(b) == ctas(12)) return b;
+        if (total(b) <= most && ctas(b) == ctas(12)) return b;
     return 12;
 }
 

@@ -580,8 +580,9 @@ struct LatTables {
 LatTables lat_tables(const Rep &r, int precision, int cluster)
 {
     const int rb = precision == CG_FP64 ? 8 : 4, folded = (int)r.tab->t64.size(), V = r.tab->V;
+    const int most = kSmemPerCta - lat_static_bytes(r.pair);
     if (cluster == 1) {
-        const int b = lat_guide_bits(r.N, folded, V, r.words, rb);
+        const int b = lat_guide_bits(r.N, folded, V, r.words, rb, most);
         return {b, false, lat_layout(r.N, folded, V, r.words, rb, b).total};
     }
     const bool cubic = dim_of(r.d) == 3;
@@ -589,7 +590,7 @@ LatTables lat_tables(const Rep &r, int precision, int cluster)
         for (int b = kLatGuideBits; b >= 12; --b) {
             const int total = lat_layout(r.N / cluster, r2 ? (int)r.tab->r2_64.size() : folded, V,
                                          r.words, rb, b).total;
-            if (total <= kLatSmemMost || (b == 12 && r2 == (cubic ? 1 : 0)))
+            if (total <= most || (b == 12 && r2 == (cubic ? 1 : 0)))
                 return {b, r2 == 1, total};
         }
     return {12, cubic, 0};      // not reached
@@ -632,9 +633,7 @@ int cluster_rows_unit(const cg_replica_desc &d, int c)
 // fits.  0 when nothing fits.
 int choose_cluster(const cg_opts &o, const Rep &r, int optin)
 {
-    // room for the kernels' static shared memory (the pair-hop cluster
-    // kernel's exchange slots take it past 2 KiB)
-    const int budget = optin - (o.pair_frac > 0.0 ? 3072 : 2048);
+    const int budget = optin - lat_static_bytes(o.pair_frac > 0.0);
     if (o.cluster_size > 1) {
         const int c = o.cluster_size;
         if ((c == 2 || c == 4 || c == 8) && r.d.L % cluster_rows_unit(r.d, c) == 0 &&
@@ -1988,7 +1987,7 @@ static std::vector<std::pair<int, int>> cluster_candidates(const cg_handle *h, c
     }
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    const int budget = optin - (h->opts.pair_frac > 0.0 ? 3072 : 2048);
+    const int budget = optin - lat_static_bytes(h->opts.pair_frac > 0.0);
     for (int c = 1; c <= 8; c *= 2) {
         if (c > 1 && !g.random && (g.L % (g.dim == 3 ? c : 2 * c) != 0 || g.L < 16)) continue;
         int sm = 0;
