@@ -1174,7 +1174,14 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
             for (int m = 0; m < R; ++m)
                 count += reps[m].sites != CG_SITES_RANDOM && reps[m].L == r.d.L &&
                          dim_of(reps[m]) == dim_of(r.d);
-            if (!r.random && group_uses_fft(o, r.d.L, count, dim_of(r.d))) build_fft_tables(*t);
+            // DFT(1/r) and the twiddles depend on L and dim alone: with several
+            // r_max or xi the first replica's table has them, which is the one
+            // refresh_group reads
+            bool have = false;
+            for (const auto &q : h->tables)
+                have = have || (q->L == r.d.L && q->dim == dim_of(r.d) && !q->ghat.empty());
+            if (!have && !r.random && group_uses_fft(o, r.d.L, count, dim_of(r.d)))
+                build_fft_tables(*t);
             r.tab = t.get();
             h->tables.push_back(std::move(t));
         }
