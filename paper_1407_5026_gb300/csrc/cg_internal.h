@@ -275,7 +275,7 @@ cudaError_t launch_pr_persistent(int precision, const DevReplica *d_reps,
 cudaError_t launch_pr_persistent3(int precision, const DevReplica *d_reps, const int *d_index,
                                   int n_ctas, int threads, int smem_bytes, const RunArgs &args,
                                   cudaStream_t st, int L);
-cudaError_t set_pr3_smem_limit(int precision, int bytes);
+cudaError_t set_pr3_smem_limit(int precision, int bytes, bool pair);
 // The cubic lattice with two-electron hops (cg_pr_kernel3d_pair.cu).
 cudaError_t launch_pr_persistent3_pair(int precision, const DevReplica *d_reps,
                                        const int *d_index, int n_ctas, int threads,
@@ -316,7 +316,7 @@ cudaError_t launch_debug_gauss(const uint64_t *seed, const uint32_t *rep, const 
                                double *z, int n, cudaStream_t st);
 cudaError_t launch_debug_tower(const unsigned short *guide, const unsigned *thr, int V,
                                const uint32_t *x1, int *out, int n, cudaStream_t st);
-cudaError_t set_pr_smem_limit(int precision, int bytes);
+cudaError_t set_pr_smem_limit(int precision, int bytes, bool pair);
 int microbench(int kind, int device, double *result);
 // Histogram of eps (binary64 or binary32 by precision) of `count` replicas
 // starting at d_reps, added to the nbins counters at out.

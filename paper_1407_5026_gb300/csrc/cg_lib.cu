@@ -661,8 +661,10 @@ int choose_cluster(const cg_opts &o, const Rep &r, int optin)
 //   clusters of a lattice: 512, which leave 128 registers and cost less per
 //   cluster barrier (L = 256 on 4 CTAs: 4.1 against 4.7 ms with 1024, 48^3 on 4
 //   CTAs: 1.63 and 1.82);
-//   two-electron hops: 256, and 512 from 12,288 sites on: a label holds more
-//   values than 64 registers (L = 64, 304 replicas: 3.7 against 4.6 with 512).
+//   two-electron hops: 256, in binary32 384 from 20,480 sites on: a label holds
+//   more values than the 64 registers of 512 threads, which spill (152 replicas
+//   of L = 112: 15.2 against 15.7 with 512; L = 150: 18.4 with 384, 20.8 with
+//   256, 19.8 with 512).
 int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
 {
     const int L = r.d.L, N = r.N;
@@ -673,7 +675,7 @@ int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
         else if (r.random)
             t = (o.precision == CG_FP64 || smem > 110 * 1024) ? 1024 : 512;
         else if (r.pair)
-            t = N < 12288 ? 256 : 512;
+            t = o.precision == CG_FP64 || N < 20480 ? 256 : 384;
         else if (o.precision == CG_FP64)
             t = N < 2048 ? 384 : N < 12288 ? 512 : 1024;
         else
@@ -1370,7 +1372,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         destroy_partial();
         return nullptr;
     }
-    if (set_pr_smem_limit(o.precision, optin - 2048) != cudaSuccess ||
+    if (set_pr_smem_limit(o.precision, optin - 2048, o.pair_frac > 0.0) != cudaSuccess ||
         set_pr_random_smem_limit(optin - 2048) != cudaSuccess) {
         fail(CG_ECUDA, "cudaFuncSetAttribute(max dynamic shared memory) failed");
         destroy_partial();

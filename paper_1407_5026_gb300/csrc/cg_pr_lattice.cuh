@@ -894,4 +894,82 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
     }
 }
 
+// ---------------------------------------------------------------------------
+// Instances.  The sides of the configurations and of their mixed batch (square
+// 32, 48, 64, 96, 128; cubic 32 in binary32, the largest power of two whose eps
+// fits one CTA) are fixed at compile time: the update's offsets and loop counts
+// and the label's wraps become constants.  Single and two-electron hops, both
+// clocks alike.  ms per run call with L at run time and fixed, 152 replicas, a
+// fifth pair labels, 96 hops: L = 32 0.91 -> 0.77, 48 0.99 -> 0.84, 64 1.01 ->
+// 0.85, 96 1.27 -> 1.05, 128 1.50 -> 1.20 (binary64, 64: 1.97 -> 1.82).  Any
+// other L is read at run time, as a power of two or not.
+// ---------------------------------------------------------------------------
+
+using LatKernel = void (*)(const DevReplica *, const int *, RunArgs);
+
+template <typename Real, int kThreads, bool kTime, int kDim, bool kPair>
+LatKernel lattice_side(int L)
+{
+    if constexpr (kDim == 2) {
+        switch (L) {
+        case 32: return pr_lattice<Real, kThreads, 5, kTime, kDim, kPair>;
+        case 48: return pr_lattice<Real, kThreads, -48, kTime, kDim, kPair>;
+        case 64: return pr_lattice<Real, kThreads, 6, kTime, kDim, kPair>;
+        case 96: return pr_lattice<Real, kThreads, -96, kTime, kDim, kPair>;
+        case 128: return pr_lattice<Real, kThreads, 7, kTime, kDim, kPair>;
+        }
+    } else if constexpr (sizeof(Real) == 4) {
+        if (L == 32) return pr_lattice<Real, kThreads, 5, kTime, kDim, kPair>;
+    }
+    return (L & (L - 1)) == 0 ? pr_lattice<Real, kThreads, 0, kTime, kDim, kPair>
+                              : pr_lattice<Real, kThreads, -1, kTime, kDim, kPair>;
+}
+
+// Null for a CTA size that is not built.
+template <bool kTime, int kDim, bool kPair>
+LatKernel lattice_kernel(int precision, int threads, int L)
+{
+    if (precision == CG_FP64) {
+        switch (threads) {
+        case 1024: return lattice_side<double, 1024, kTime, kDim, kPair>(L);
+        case 512: return lattice_side<double, 512, kTime, kDim, kPair>(L);
+        case 384: return lattice_side<double, 384, kTime, kDim, kPair>(L);
+        case 256: return lattice_side<double, 256, kTime, kDim, kPair>(L);
+        }
+    } else {
+        switch (threads) {
+        case 1024: return lattice_side<float, 1024, kTime, kDim, kPair>(L);
+        case 512: return lattice_side<float, 512, kTime, kDim, kPair>(L);
+        case 384: return lattice_side<float, 384, kTime, kDim, kPair>(L);
+        case 256: return lattice_side<float, 256, kTime, kDim, kPair>(L);
+        }
+    }
+    return nullptr;
+}
+
+template <bool kTime, int kDim, bool kPair>
+cudaError_t launch_lattice(int precision, const DevReplica *d_reps, const int *d_index, int n_ctas,
+                           int threads, int smem_bytes, const RunArgs &args, cudaStream_t st,
+                           int L)
+{
+    const LatKernel k = lattice_kernel<kTime, kDim, kPair>(precision, threads, L);
+    if (!k) return cudaErrorInvalidValue;
+    k<<<n_ctas, threads, smem_bytes, st>>>(d_reps, d_index, args);
+    return cudaGetLastError();
+}
+
+// Room for `bytes` of dynamic shared memory in every instance of one precision.
+template <bool kTime, int kDim, bool kPair>
+cudaError_t set_lattice_limit(int precision, int bytes)
+{
+    for (int threads : {256, 384, 512, 1024})
+        for (int L : {4, 6, 32, 48, 64, 96, 128}) {
+            const LatKernel k = lattice_kernel<kTime, kDim, kPair>(precision, threads, L);
+            const cudaError_t e =
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (e) return e;
+        }
+    return cudaSuccess;
+}
+
 }  // namespace cg
