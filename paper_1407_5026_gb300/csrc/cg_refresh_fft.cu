@@ -23,8 +23,8 @@
 //                   DFT(g)/N, inverse y | inverse x (into eps);
 //   cubic lattice:  forward x | forward y | forward z, times DFT(g)/N,
 //                   inverse z | inverse y | inverse x (into eps).
-// The last pass adds phi in binary64, stores eps rounded to binary32 and
-// records the largest |eps_old - eps_new| of each replica, as the other
+// The last pass adds phi (all of its 53 bits; see refresh_site), stores eps
+// rounded once to binary32 and records the largest |eps_old - eps_new| of each replica, as the other
 // refresh paths do.  The product's table DFT(g)/N and the twiddles
 // exp(-2 pi i k / L) are computed on the host in binary64.
 #include "cg_device.cuh"
@@ -166,57 +166,106 @@ __device__ __forceinline__ int out_pos(int k, const FftArgs &a, bool dif_out)
     return dif_out ? (int)bitrev((unsigned)k, a.log2L) : k;
 }
 
-// eps_new = phi + (v + c) rounded once to binary32, and the change
-// |eps_old - eps_new|, in binary32 pairs: phi is split without the binary64
-// pipe (its word cut to a binary32 plus the 29 bits below), the two large terms
-// add with their exact error (Knuth's two-sum) and the error joins the small
-// ones before the last add.  What is lost is below 2^-45 of the sum.  (In
-// binary64, ten operations per site at 1/64 of the binary32 rate, this step
-// took most of the last pass.)
-__device__ __forceinline__ float refresh_site(double phi, float v, float c, float eps_old,
-                                              float &change)
+// a + b and its rounding error (Knuth's two-sum: the pair's sum is a + b exactly).
+__device__ __forceinline__ float2 two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+}
+
+// The transforms took n - nu with nu rounded to binary32; sum_t g(s-t) = C0 for
+// every s, so (nu_f - nu) C0 restores the exact nu.
+__device__ __forceinline__ double nu_shift(const DevReplica &R)
+{
+    return d_mul(d_sub((double)(float)R.nu, R.nu), R.C0);
+}
+__device__ __forceinline__ float2 split_f32(double c)
+{
+    const float h = (float)c;
+    return make_float2(h, (float)d_sub(c, (double)h));
+}
+
+// eps_new of a site in binary64, for the values that refresh_site leaves out; the
+// change goes into err (NaN is not counted).
+__device__ __noinline__ float refresh_site64(double phi, float v, const DevReplica &R,
+                                             float eps_old, unsigned long long *err)
+{
+    const double e = d_add(phi, d_add((double)v, nu_shift(R)));
+    const double change = fabs(d_sub((double)eps_old, e));
+    if (change >= 0.0) atomicMax(err, (unsigned long long)__double_as_longlong(change));
+    return __double2float_rn(e);
+}
+
+// eps_new = phi + (v + c) rounded once to binary32, c = c.x + c.y = nu_shift, and
+// the change |eps_old - (phi + (v + c))|, kept in `most` as the sum of three
+// binary32 numbers if it is the thread's largest so far.  phi's 53 bits are taken
+// apart into 24 + 15 + 14 and summed with v and c by two-sums, whose errors are
+// kept down to the fourth: what is lost is below 2^-63 of the terms, where the
+// same sum in binary64 loses 2^-53 (over W = 0 to 14 and c up to 2e-5, the largest
+// error of a change near 1e-6: 9e-19 against 1.3e-15).  In binary64 the step is ten
+// operations per site at 1/64 of the binary32 rate; with 24 bits of each part, and
+// the change in binary32, a resume is 3 to 5% faster (304 replicas of L = 128 230
+// against 238 us, 128 of L = 112 124 against 131) and a change 1e3 to 1e5 times as
+// far off.  A phi that is not 0 and outside
+// 2^-74 to 2^78, and an eps_old past 2^100, are left to binary64.
+__device__ __forceinline__ float refresh_site(double phi, float v, float2 c, float eps_old,
+                                              const DevReplica &R, unsigned long long *err,
+                                              float3 &most)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(phi);
-    const int ex = (int)((b >> 52) & 0x7ffull);
+    const bool zero = (b << 1) == 0ull;
+    const int ex = zero ? 949 : (int)((b >> 52) & 0x7ffull);
+    if ((unsigned)(ex - 949) > 1100u - 949u || !(fabsf(eps_old) < 0x1p100f))
+        return refresh_site64(phi, v, R, eps_old, err);
     const unsigned sign = (unsigned)(b >> 63) << 31;
-    if (ex > 1150) {                                     // no binary32 value: inf, or NaN
-        change = __uint_as_float(0x7f800000u);
-        return __uint_as_float(sign | 0x7f800000u |
-                               (ex == 0x7ff && (b & 0x000fffffffffffffull) ? 1u << 22 : 0u));
-    }
-    float hi = 0.0f, lo = 0.0f;                          // below 2^-74: nothing to add
-    if (ex >= 949) {
-        hi = __uint_as_float(sign | ((unsigned)(ex - 896) << 23) |
-                             ((unsigned)(b >> 29) & 0x7fffffu));
-        lo = __uint2float_rn((unsigned)b & 0x1fffffffu) *
-             __uint_as_float(sign | ((unsigned)(ex - 948) << 23));   // 2^(ex - 1075), signed
-    }
-    const float s = __fadd_rn(hi, v), bb = __fsub_rn(s, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb));
-    const float t = __fadd_rn(err, __fadd_rn(lo, c));
-    change = fabsf(__fsub_rn(__fsub_rn(eps_old, s), t));
-    return __fadd_rn(s, t);
+    const float hi = zero ? 0.0f
+                          : __uint_as_float(sign | ((unsigned)(ex - 896) << 23) |
+                                            ((unsigned)(b >> 29) & 0x7fffffu));
+    const float unit = __uint_as_float(sign | ((unsigned)(ex - 948) << 23));  // 2^(ex - 1075)
+    // the lower 29 bits as 15 + 14: integers below 2^23 in the mantissa of 2^23
+    // (a conversion instruction runs at an eighth of this rate)
+    const float i1 = __uint_as_float(0x4b000000u | (((unsigned)b >> 14) & 0x7fffu)) - 0x1p23f;
+    const float i2 = __uint_as_float(0x4b000000u | ((unsigned)b & 0x3fffu)) - 0x1p23f;
+    const float l1 = __fmul_rn(i1 * 0x1p14f, unit), l2 = __fmul_rn(i2, unit);
+    const float2 p = two_sum(hi, v), q = two_sum(l1, c.x), t = two_sum(p.y, q.x);
+    const float u = __fadd_rn(__fadd_rn(q.y, t.y), __fadd_rn(l2, c.y));
+    const float2 r = two_sum(p.x, t.x);
+    const float2 d = two_sum(eps_old, -r.x), k = two_sum(d.y, -r.y), x = two_sum(d.x, k.x);
+    float2 y = two_sum(x.y, __fsub_rn(k.y, u));
+    const bool neg = x.x < 0.0f || (x.x == 0.0f && y.x < 0.0f);
+    const float m = fabsf(x.x), n = neg ? -y.x : y.x;
+    if (m > most.x || (m == most.x && n > most.y)) most = make_float3(m, n, neg ? -y.y : y.y);
+    return __fadd_rn(r.x, __fadd_rn(r.y, u));
 }
 
 // The block's maxima of the changes of two replicas into their counters.
-__device__ __forceinline__ void record_change(float ca, float cb, bool two, bool count,
-                                              DevCounters *da, DevCounters *db, unsigned *s_err)
+__device__ __forceinline__ void record_change(float3 ca, float3 cb, bool two, bool count,
+                                              DevCounters *da, DevCounters *db,
+                                              unsigned long long *s_err)
 {
-    // non-negative floats order as their bits
-    const unsigned ma = __reduce_max_sync(0xffffffffu, __float_as_uint(ca));
-    const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(cb));
+    // non-negative binary64 numbers order as their bits
+    auto bits = [](float3 c) {
+        const double v = d_add((double)c.x, d_add((double)c.y, (double)c.z));
+        return (unsigned long long)__double_as_longlong(v);
+    };
+    unsigned long long ba = bits(ca), bb = bits(cb);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long xa = __shfl_xor_sync(0xffffffffu, ba, o);
+        const unsigned long long xb = __shfl_xor_sync(0xffffffffu, bb, o);
+        ba = ba > xa ? ba : xa;
+        bb = bb > xb ? bb : xb;
+    }
     if ((threadIdx.x & 31) == 0) {
-        atomicMax(&s_err[0], ma);
-        atomicMax(&s_err[1], mb);
+        atomicMax(&s_err[0], ba);
+        atomicMax(&s_err[1], bb);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        atomicMax(&da->max_err_bits,
-                  (unsigned long long)__double_as_longlong((double)__uint_as_float(s_err[0])));
+        atomicMax(&da->max_err_bits, s_err[0]);
         if (count) atomicAdd(&da->refreshes, 1ull);
         if (two) {
-            atomicMax(&db->max_err_bits,
-                      (unsigned long long)__double_as_longlong((double)__uint_as_float(s_err[1])));
+            atomicMax(&db->max_err_bits, s_err[1]);
             if (count) atomicAdd(&db->refreshes, 1ull);
         }
     }
@@ -240,7 +289,7 @@ template <int kMode>
 __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int axis)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned s_err[2];
+    __shared__ unsigned long long s_err[2];
     const int L = a.L, W = a.W, Ls = L + 1;     // padded line stride (banks)
     const int groups = (int)(gridDim.x / (unsigned)((a.R + 1) / 2));
     const int p = blockIdx.x / groups, g = blockIdx.x - p * groups;
@@ -269,7 +318,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         }
         s[w * Ls + (natural_in ? k : (int)bitrev((unsigned)k, a.log2L))] = v;
     }
-    if (kMode == 4 && threadIdx.x < 2) s_err[threadIdx.x] = 0u;
+    if (kMode == 4 && threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
     __syncthreads();
     // ---- transform ----
     float2 *out = s;                                       // where the result lies
@@ -305,7 +354,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         }
     }
     // ---- store ----
-    float err_a = 0.0f, err_b = 0.0f;
+    float3 err_a = make_float3(0.0f, 0.0f, 0.0f), err_b = err_a;
     if (kMode != 4) {
         for (int e = threadIdx.x; e < n; e += kFftThreads) {
             int w, k;
@@ -322,21 +371,13 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         const double *__restrict__ pb = Rb.phi + site0;
         float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps) + site0;
         float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps) + site0;
-        // the transforms took n - nu with nu rounded to binary32; sum_t g(s-t)
-        // = C0 for every s, so (nu_f - nu) C0 restores the exact nu
-        const float ca = (float)d_mul(d_sub((double)(float)Ra.nu, Ra.nu), Ra.C0);
-        const float cb = (float)d_mul(d_sub((double)(float)Rb.nu, Rb.nu), Rb.C0);
+        const float2 ca = split_f32(nu_shift(Ra)), cb = split_f32(nu_shift(Rb));
 #pragma unroll 4
         for (int e = threadIdx.x; e < n; e += kFftThreads) {
             const int w = e / L, k = e - w * L;
             const float2 v = out[w * Ls + out_pos(k, a, true)];
-            float ch;
-            ea[e] = refresh_site(pa[e], v.x, ca, ea[e], ch);
-            err_a = fmaxf(err_a, ch);
-            if (two) {
-                eb[e] = refresh_site(pb[e], v.y, cb, eb[e], ch);
-                err_b = fmaxf(err_b, ch);
-            }
+            ea[e] = refresh_site(pa[e], v.x, ca, ea[e], Ra, &s_err[0], err_a);
+            if (two) eb[e] = refresh_site(pb[e], v.y, cb, eb[e], Rb, &s_err[1], err_b);
         }
         record_change(err_a, err_b, two, g == 0, Ra.ctr, Rb.ctr, s_err);
     }
@@ -702,15 +743,13 @@ struct Plane {
     // x, the inverse's second step, into eps of the plane at site0; the largest
     // changes of the thread's sites
     __device__ __forceinline__ void x_into_eps(const DevReplica &Ra, const DevReplica &Rb, bool two,
-                                               unsigned site0, float &err_a, float &err_b) const
+                                               unsigned site0, unsigned long long *s_err,
+                                               float3 &err_a, float3 &err_b) const
     {
         const double *__restrict__ pa = Ra.phi + site0, *__restrict__ pb = Rb.phi + site0;
         float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps) + site0;
         float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps) + site0;
-        // the transforms took n - nu with nu rounded to binary32; sum_t g(s-t)
-        // = C0 for every s, so (nu_f - nu) C0 restores the exact nu
-        const float ca = (float)d_mul(d_sub((double)(float)Ra.nu, Ra.nu), Ra.C0);
-        const float cb = (float)d_mul(d_sub((double)(float)Rb.nu, Rb.nu), Rb.C0);
+        const float2 ca = split_f32(nu_shift(Ra)), cb = split_f32(nu_shift(Rb));
         for (int it = threadIdx.x; it < L * 8; it += kT) {
             const int b = it & 7, y = row_of(it >> 3), site = y * L + b;
             float2 v[R1];
@@ -734,13 +773,9 @@ struct Plane {
 #pragma unroll
                 for (int k = 0; k < kBatch; ++k) {
                     const int e = site + 8 * (k0 + k);
-                    float ch;
-                    ea[e] = refresh_site(fa[k], v[k0 + k].x, ca, oa[k], ch);
-                    err_a = fmaxf(err_a, ch);
-                    if (two) {
-                        eb[e] = refresh_site(fb[k], v[k0 + k].y, cb, ob[k], ch);
-                        err_b = fmaxf(err_b, ch);
-                    }
+                    ea[e] = refresh_site(fa[k], v[k0 + k].x, ca, oa[k], Ra, &s_err[0], err_a);
+                    if (two)
+                        eb[e] = refresh_site(fb[k], v[k0 + k].y, cb, ob[k], Rb, &s_err[1], err_b);
                 }
             }
         }
@@ -762,14 +797,14 @@ template <int L>
 __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_square_kernel(FftArgs a)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned s_err[2];
+    __shared__ unsigned long long s_err[2];
     const Plane<L> P{s, s + L * Plane<L>::Ls};
     const int p = blockIdx.x;
     const DevReplica &Ra = a.reps[a.index[2 * p]];
     const bool two = 2 * p + 1 < a.R;
     const DevReplica &Rb = a.reps[a.index[two ? 2 * p + 1 : 2 * p]];
     P.twiddles(a.tw);
-    if (threadIdx.x < 2) s_err[threadIdx.x] = 0u;
+    if (threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
     clear_change(two, Ra.ctr, Rb.ctr);
     __syncthreads();
     P.prefetch(Ra, 0u);
@@ -784,8 +819,8 @@ __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_square_kernel(FftA
     __syncthreads();
     P.x_inverse1();
     __syncthreads();
-    float err_a = 0.0f, err_b = 0.0f;
-    P.x_into_eps(Ra, Rb, two, 0u, err_a, err_b);
+    float3 err_a = make_float3(0.0f, 0.0f, 0.0f), err_b = err_a;
+    P.x_into_eps(Ra, Rb, two, 0u, s_err, err_a, err_b);
     record_change(err_a, err_b, two, true, Ra.ctr, Rb.ctr, s_err);
 }
 
@@ -797,7 +832,7 @@ template <int L, int kStep>
 __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftArgs a)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned s_err[2];
+    __shared__ unsigned long long s_err[2];
     constexpr int R1 = L / 8;
     const Plane<L> P{s, s + L * Plane<L>::Ls};
     const int p = blockIdx.x / L, o = blockIdx.x - p * L;
@@ -807,7 +842,7 @@ __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftAr
     float2 *buf = a.buf + (size_t)p * L * L * L;
     const unsigned site0 = (unsigned)(o * L * L);
     P.twiddles(a.tw);
-    if (kStep == 2 && threadIdx.x < 2) s_err[threadIdx.x] = 0u;
+    if (kStep == 2 && threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
     __syncthreads();
     if (kStep == 0) {
         if (o == 0) clear_change(two, Ra.ctr, Rb.ctr);
@@ -834,8 +869,8 @@ __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftAr
         __syncthreads();
         P.x_inverse1();
         __syncthreads();
-        float err_a = 0.0f, err_b = 0.0f;
-        P.x_into_eps(Ra, Rb, two, site0, err_a, err_b);
+        float3 err_a = make_float3(0.0f, 0.0f, 0.0f), err_b = err_a;
+        P.x_into_eps(Ra, Rb, two, site0, s_err, err_a, err_b);
         record_change(err_a, err_b, two, o == 0, Ra.ctr, Rb.ctr, s_err);
     }
 }
