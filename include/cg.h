@@ -481,6 +481,15 @@ int cg_debug_gauss(const uint64_t *seed_host, const uint32_t *replica_host,
  * allocates and frees device memory internally. */
 int cg_debug_tower(cg_handle *h, int replica, const uint32_t *x1_host, int32_t *v_host, int n);
 
+/* Test-only: the order in which a launch of `group` now would deal its replicas
+ * to CTAs, heaviest first, as positions within the group (order_host: one per
+ * replica).  A group of more replicas than SMs, and at most four times as many,
+ * on one CTA each pairs heavy ones with light ones on an SM by their attempts
+ * per hop: of the last launch, or, where the state was written since or none has
+ * run, of the counters as they stand.  CG_EINVAL for any other group (its
+ * launches take the replicas in order), CG_ECUDA on a CUDA error. */
+int cg_debug_schedule(cg_handle *h, int group, int32_t *order_host);
+
 /* Density of states of the local energies: the histogram g(eps) whose
  * Coulomb gap the paper discusses (section "Results for the lattice model in
  * two dimensions", single-particle density of states).  For the sites s of

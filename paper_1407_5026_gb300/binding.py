@@ -31,7 +31,8 @@ EXPORTED = [
     "cg_destroy", "cg_last_error", "cg_num_replicas", "cg_num_sites", "cg_run",
     "cg_run_async", "cg_sync", "cg_run_logged", "cg_read_state", "cg_write_state",
     "cg_observables", "cg_refresh", "cg_refresh_async", "cg_microbench",
-    "cg_set_toy_acceptance", "cg_debug_philox", "cg_debug_exp", "cg_debug_tower", "cg_version",
+    "cg_set_toy_acceptance", "cg_debug_philox", "cg_debug_exp", "cg_debug_tower", "cg_debug_schedule",
+    "cg_version",
     "cg_group_replicas", "cg_read_group_state", "cg_write_group_state", "cg_debug_gauss",
     "cg_refresh_tc_noalloc", "cg_autotune", "cg_num_groups", "cg_group_shape",
     "cg_set_trace", "cg_read_trace", "cg_eps_histogram", "cg_site_positions",
@@ -158,6 +159,8 @@ def load(path: str | None = None):
                                               ctypes.c_int]),
             "cg_read_group_state": (ctypes.c_int, [vp, ctypes.c_int, u32p, vp, vp]),
             "cg_write_group_state": (ctypes.c_int, [vp, ctypes.c_int, u32p, vp, vp]),
+            "cg_debug_schedule": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int,
+                                                 P(ctypes.c_int32)]),
             "cg_debug_tower": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, u32p,
                                               ctypes.POINTER(ctypes.c_int32), ctypes.c_int]),
             "cg_version": (ctypes.c_char_p, []),
@@ -471,6 +474,13 @@ def cg_debug_tower(h, replica, x1):
     out = np.zeros(len(x1), dtype=np.int32)
     _check(load().cg_debug_tower(h, replica, _ptr(x1, ctypes.c_uint32),
                                  _ptr(out, ctypes.c_int32), len(x1)))
+    return out
+
+
+def cg_debug_schedule(h, group):
+    """Positions within the group in the order a launch would deal them, heaviest first."""
+    out = np.zeros(len(group_dims(h, group)[0]), dtype=np.int32)
+    _check(load().cg_debug_schedule(h, group, _ptr(out, ctypes.c_int32)))
     return out
 
 

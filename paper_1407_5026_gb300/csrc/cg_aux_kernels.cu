@@ -211,8 +211,9 @@ __global__ void __launch_bounds__(1024) pr_schedule_kernel(const DevReplica *__r
 {
     extern __shared__ float cost[];
     for (int k = threadIdx.x; k < count; k += blockDim.x) {
+        // before a launch of this state: the chain's own counters (0: none yet)
         const DevCounters *c = reps[index[k]].ctr;
-        cost[k] = c->rate > 0.f ? c->rate : c->m_ema;
+        cost[k] = c->rate > 0.f ? c->rate : c->hops ? (float)c->attempts / (float)c->hops : 0.f;
     }
     for (int k = threadIdx.x; k < count + kSchedSms; k += blockDim.x) sched[count + k] = 0;
     __syncthreads();

@@ -295,6 +295,7 @@ struct Group {
     bool random = false;             // random-site replicas (pr_random)
     bool sguide = false;             // their guide records in shared memory
     int *d_sched = nullptr;          // claim table of launches with several CTAs per SM
+    bool stale_rate = false;         // attempts per hop of a state written over since
     int gbits = kLatGuideBits;       // lat_tables of the group's cluster size
     bool r2 = false;
     int cluster = 1;                 // CTAs per replica
@@ -1461,6 +1462,30 @@ int refresh_all(cg_handle *h)
     return CG_OK;
 }
 
+// Whether a launch of the group pairs heavy replicas with light ones on an SM: more
+// CTAs than SMs, all resident at once (the rank count is quadratic, and past one
+// wave the hardware deals the CTAs out as SMs come free).
+bool pairs_by_work(const cg_handle *h, const Group &g)
+{
+    return !g.random && g.cluster == 1 && g.d_sched && g.count > h->n_sms &&
+           g.count <= 4 * h->n_sms;
+}
+
+// Before launches, and outside a graph of this library's own: attempts per hop
+// measured on a state that cg_write_group_state has replaced since do not order
+// the replicas (queued here, not by the write, which a resume without a run would
+// pay for: 246 against 238 us at 304 replicas of L = 128).
+int clear_stale_rates(cg_handle *h)
+{
+    for (Group &g : h->groups) {
+        if (!g.stale_rate || !pairs_by_work(h, g)) continue;
+        CG_CUDA(cudaMemset2DAsync(&h->reps[h->order[g.first]].d_ctr->rate, sizeof(DevCounters), 0,
+                                  sizeof(float), (size_t)g.count, h->st));
+        g.stale_rate = false;
+    }
+    return CG_OK;
+}
+
 int launch_group(cg_handle *h, const Group &g, unsigned long long hops, unsigned M,
                  unsigned long long log_off, cudaStream_t st)
 {
@@ -1481,11 +1506,7 @@ int launch_group(cg_handle *h, const Group &g, unsigned long long hops, unsigned
     a.guide_bits = g.gbits;
     a.cluster_r2 = g.r2 ? 1 : 0;
     a.n_sms = h->n_sms;
-    // more CTAs than SMs, all resident at once: pair heavy replicas with light
-    // ones (the rank count is quadratic, and past one wave the hardware deals
-    // the CTAs out as SMs come free)
-    if (!g.random && g.cluster == 1 && g.d_sched && g.count > h->n_sms &&
-        g.count <= 4 * h->n_sms) {
+    if (pairs_by_work(h, g)) {
         a.sched = g.d_sched;
         CG_CUDA(launch_pr_schedule(h->d_reps, h->d_index + g.first, g.count, g.d_sched, st));
     }
@@ -1514,6 +1535,7 @@ int enqueue_run(cg_handle *h, unsigned long long n_hops, unsigned M, bool logged
     if (!h) return fail(CG_EINVAL, "null handle");
     if (M > (1u << 24)) return fail(CG_EINVAL, "M must be in [1, 2^24] (0: per-group M)");
     if (cudaSetDevice(h->device) != cudaSuccess) return fail(CG_ECUDA, "cudaSetDevice failed");
+    if (const int rc = clear_stale_rates(h)) return rc;
     const bool refresh = h->opts.precision == CG_FP32 && h->opts.refresh_every > 0;
     const bool forked = h->groups.size() > 1;
     unsigned long long done = 0;
@@ -1546,6 +1568,7 @@ int enqueue_run_graph(cg_handle *h, unsigned long long n_hops, unsigned M)
 {
     if (M > (1u << 24)) return fail(CG_EINVAL, "M must be in [1, 2^24] (0: per-group M)");
     if (cudaSetDevice(h->device) != cudaSuccess) return fail(CG_ECUDA, "cudaSetDevice failed");
+    if (const int rc = clear_stale_rates(h)) return rc;
     for (const auto &e : h->graphs)
         if (e.n_hops == n_hops && e.M == M && e.hsr_before == h->hops_since_refresh) {
             CG_CUDA(cudaGraphLaunch(e.exec, h->st));
@@ -1886,7 +1909,8 @@ int cg_write_group_state(cg_handle *h, int group, const uint32_t *occ_words_host
                                 h->st));
     if (c_host) {
         // the public counters are replaced; the library's own fields (chunk
-        // statistics, refresh record, trace state, phase clocks) are kept
+        // statistics, refresh record, trace state, phase clocks) are kept, but
+        // for the replaced state's attempts per hop
         DevCounters *dc = h->h_ctr + g.first;  // pinned, group order
         CG_CUDA(cudaMemcpyAsync(dc, r0.d_ctr, cnt * sizeof(DevCounters),
                                 cudaMemcpyDeviceToHost, h->st));
@@ -1896,9 +1920,12 @@ int cg_write_group_state(cg_handle *h, int group, const uint32_t *occ_words_host
             dc[k].attempts = c_host[k].attempts; dc[k].evaluated = c_host[k].evaluated;
             dc[k].P = c_host[k].P; dc[k].energy = c_host[k].energy;
             dc[k].time = c_host[k].time;
+            dc[k].rate = 0.0f;
         }
         CG_CUDA(cudaMemcpyAsync(r0.d_ctr, dc, cnt * sizeof(DevCounters),
                                 cudaMemcpyHostToDevice, h->st));
+    } else if (occ_words_host || eps_host) {
+        h->groups[group].stale_rate = true;
     }
     CG_CUDA(cudaStreamSynchronize(h->st));
     return CG_OK;
@@ -2341,6 +2368,22 @@ int cg_eps_histogram(cg_handle *h, int first, int count, int nbins, double lo, d
     const double scale = (double)nbins / (hi - lo);
     CG_CUDA(launch_eps_histogram(h->d_reps + first, count, max_N, h->opts.precision, nbins, lo,
                                  scale, reinterpret_cast<unsigned long long *>(counts_dev), h->st));
+    return CG_OK;
+}
+
+int cg_debug_schedule(cg_handle *h, int group, int32_t *order_host)
+{
+    if (!h || !order_host || group < 0 || group >= (int)h->groups.size())
+        return fail(CG_EINVAL, "bad group or null output");
+    const Group &g = h->groups[group];
+    if (!pairs_by_work(h, g))
+        return fail(CG_EINVAL, "the group's launches take its replicas in order");
+    if (cudaSetDevice(h->device) != cudaSuccess) return fail(CG_ECUDA, "cudaSetDevice failed");
+    if (const int rc = clear_stale_rates(h)) return rc;
+    CG_CUDA(launch_pr_schedule(h->d_reps, h->d_index + g.first, g.count, g.d_sched, h->st));
+    CG_CUDA(cudaMemcpyAsync(order_host, g.d_sched, sizeof(int) * (size_t)g.count,
+                            cudaMemcpyDeviceToHost, h->st));
+    CG_CUDA(cudaStreamSynchronize(h->st));
     return CG_OK;
 }
 
