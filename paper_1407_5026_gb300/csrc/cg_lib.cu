@@ -666,7 +666,10 @@ int choose_cluster(const cg_opts &o, const Rep &r, int optin)
 //   more values than the 64 registers of 512 threads, which spill (152 replicas
 //   of L = 112: 15.2 against 15.7 with 512; L = 150: 18.4 with 384, 20.8 with
 //   256, 19.8 with 512).
-int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
+//   random sites: 1024, and 512 below 512 sites, where a hop takes few labels and
+//   a chunk of 1024 costs more than a second one (24 replicas of L = 16, 128 hops,
+//   T = 0.3: 1.43 against 2.09 ms; T = 0.05: 1.46 and 1.73; T = 0.02: 3.5 and 3.2).
+int choose_threads(const cg_opts &o, const Rep &r, int cluster)
 {
     const int L = r.d.L, N = r.N;
     int t = o.block_threads;
@@ -674,7 +677,7 @@ int choose_threads(const cg_opts &o, const Rep &r, int smem, int cluster)
         if (cluster > 1 && !r.random)
             t = 512;
         else if (r.random)
-            t = (o.precision == CG_FP64 || smem > 110 * 1024) ? 1024 : 512;
+            t = N < 512 ? 512 : 1024;
         else if (r.pair)
             t = o.precision == CG_FP64 || N < 20480 ? 256 : 384;
         else if (o.precision == CG_FP64)
@@ -1318,7 +1321,7 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
         g.smem = smem;
         g.cluster = cluster;
         set_lat_tables(h.get(), g);
-        g.threads = choose_threads(o, h->reps[order[g.first]], smem, cluster);
+        g.threads = choose_threads(o, h->reps[order[g.first]], cluster);
         if (cluster > 1 && g.random) {
             // the random-site cluster kernel takes 256, 512 or 1024 threads
             if (g.threads == 384) g.threads = 512;

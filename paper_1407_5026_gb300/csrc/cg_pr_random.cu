@@ -12,10 +12,10 @@
 // the minimum-image fold maps d to -d exactly.
 //
 // What bounds it: the dependent loads of a label (guide record, weights,
-// partner) from L2 and HBM.  Weights of 32 bits apart from the partners cost a
-// label four sectors where whole pair records cost seven; with the rejection
-// decided in binary32 (24 replicas of L = 64, ms per run call): 4.40 -> 3.95; with
-// weight and partner in 8 bytes, the partner's word bounding dH: 3.93.
+// partner and couplings) from L2 and HBM.  Weights of 32 bits apart from the
+// partners cost a label five sectors where whole pair records cost seven, and most
+// rejections are decided in binary32 from the partner's word, which bounds dH (24
+// replicas of L = 64, ms per run call of 128 hops at T = 0.05): 4.39 -> 4.12.
 //
 // pr_random: one CTA per replica, binary64; eps and the occupation bitmask in
 // shared memory, the partner lists (a 64-byte guide record per site; weights,
@@ -157,7 +157,7 @@ pr_random(const DevReplica *__restrict__ reps, const int *__restrict__ index, Ru
                 double dE0 = 0.0;
                 bool acc0 = false;
                 if (p0.theta)
-                    acc0 = accept_random(Rg, eps[p0.i], eps[p0.j], p0, cut, T, invTf, dE0);
+                    acc0 = accept_random(eps[p0.i], eps[p0.j], p0, cut, T, invTf, dE0);
                 const int any = __syncthreads_or(acc0);
                 if (any) {
                     const unsigned b0 = __ballot_sync(0xffffffffu, acc0);

@@ -13,7 +13,8 @@ struct RCand {
 };
 
 struct RLabel {
-    unsigned i, j, m, x2;     // m: the pair's index
+    unsigned i, j, x2;
+    double2 gx;               // 1/r_ij and E dx_ij
     float cv;                 // 1/r_ij + E dx_ij or up to 1/64 of it above
     bool theta;
 };
@@ -25,10 +26,13 @@ struct RLabel {
 // proposal) and the bucket of pairs x1 >> 28 can select; a four-way search
 // (three independent probes per step) narrows a bucket of more than eight, and
 // the rest is counted from up to three aligned loads of four weights (C_m - 1,
-// 32 bits).  The chosen pair's partner and a bound on its 1/r + E dx come with one
-// more load of 4 bytes.  (Reading whole records with 1/r and E dx beside the weights took
-// seven sectors per label for these four; the L1's tag stage was the second
-// stall of the kernel, tex_throttle 3.5 per issue.)
+// 32 bits).  The chosen pair's partner with a bound on its 1/r + E dx, and 1/r
+// and E dx themselves, are two more loads side by side: five sectors per label
+// where whole records, read with their 1/r and E dx in the scan, took seven.
+// (1/r and E dx loaded for the few labels that need them would save one sector
+// but put one more load into the chain of a hop: 24 replicas of L = 64 4.20
+// against 4.11 ms per 128 hops at T = 0.05, 4.35 against 4.20 at T = 0.3; one
+// of L = 32 at T = 0.3 2.53 against 2.43.)
 // gsm: the compacted guide records in shared memory (two uint4 per site:
 // {first, last lo, length | last hi << 16, 0} and the 16 bucket starts as
 // bytes), or null for the 64-byte records in global memory.
@@ -39,8 +43,9 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
 {
     RLabel p;
     p.theta = false;
-    p.i = p.j = p.m = 0;
+    p.i = p.j = 0;
     p.x2 = 0;
+    p.gx = make_double2(0.0, 0.0);
     p.cv = 0.0f;
     if (!valid) return p;
     uint32_t x[4];
@@ -124,7 +129,7 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
         m += (e >= lo && e < hi - 1 && w[t] < w1) ? 1 : 0;
     }
     const uint32_t rc = __ldg(Rg.rj + m);
-    p.m = (unsigned)m;
+    p.gx = __ldg(Rg.rgx + m);
     p.j = rc & kPartnerMask;
     p.cv = __uint_as_float(rc & ~kPartnerMask);
     p.theta = !((occ[p.j >> 5] >> (p.j & 31)) & 1u);     // n_i = 1 here
@@ -136,17 +141,15 @@ __device__ __forceinline__ RLabel propose_random(const DevReplica &Rg, const uns
 // take the binary64 one, ((eps_j - eps_i) - 1/r_ij) - E dx_ij, each step rounded,
 // and the binary64 decision.  (Three binary64 adds per label on the slow pipe
 // were a quarter of a chunk.)
-__device__ __forceinline__ bool accept_random(const DevReplica &Rg, double ei, double ej,
-                                              const RLabel &p, float cut, double T, float invTf,
-                                              double &dE)
+__device__ __forceinline__ bool accept_random(double ei, double ej, const RLabel &p, float cut,
+                                              double T, float invTf, double &dE)
 {
     bool oi, oj;
     const float fi = hi_to_f32(__double2hiint(ei), oi), fj = hi_to_f32(__double2hiint(ej), oj);
     const float s = fabsf(fi) + fabsf(fj) + fabsf(p.cv);
     const float lo = fmaf(s, -0x1p-19f, (fj - fi) - p.cv);      // at most dH
     if (oi && oj && (!(lo < cut) || surely_rejected(lo, p.x2, invTf))) return false;
-    const double2 gx = __ldg(Rg.rgx + p.m);
-    dE = d_sub(d_sub(d_sub(ej, ei), gx.x), gx.y);
+    dE = d_sub(d_sub(d_sub(ej, ei), p.gx.x), p.gx.y);
     return metropolis64(dE, p.x2, T, invTf);
 }
 

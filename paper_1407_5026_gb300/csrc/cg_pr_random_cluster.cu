@@ -131,7 +131,7 @@ pr_random_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ i
                 if (p0.theta) {
                     const double ei = cluster_eps_random(cl, eps, p0.i, Nc, magicW, rank);
                     const double ej = cluster_eps_random(cl, eps, p0.j, Nc, magicW, rank);
-                    acc0 = accept_random(Rg, ei, ej, p0, cut, T, invTf, dE0);
+                    acc0 = accept_random(ei, ej, p0, cut, T, invTf, dE0);
                 }
                 const int any = __syncthreads_or(acc0);
                 unsigned best = 0xffffffffu;
