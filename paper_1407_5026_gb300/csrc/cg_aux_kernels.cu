@@ -111,7 +111,9 @@ __global__ void __launch_bounds__(256) refresh_fp64_kernel(const DevReplica *__r
 {
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ unsigned long long s_max;
-    const DevReplica &R = reps[index[blockIdx.y]];
+    // a copy: the loop below reads its extents each time round, and through a
+    // reference from memory (one replica of L = 144: 1.07 against 0.89 ms)
+    const DevReplica R = reps[index[blockIdx.y]];
     const int L = R.L, N = R.N, H1 = R.H1, words = R.words, ntab = tab_entries(R);
     const int Lz = R.dim == 3 ? L : 1;
     double *tab_s = reinterpret_cast<double *>(sm);
