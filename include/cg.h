@@ -471,12 +471,13 @@ int cg_debug_exp(const double *x_host, double *out_host, int n);
 int cg_debug_gauss(const uint64_t *seed_host, const uint32_t *replica_host,
                    const uint64_t *hops_host, double *z_host, int n);
 
-/* Test-only: the PR kernels' tower sampler (guide table + thresholds of
+/* Test-only: the PR kernels' tower samplers (guide tables + thresholds of
  * replica `replica`, section "Hopping conduction in the Coulomb glass": hop
  * vector by tower sampling) on the GPU for n 32-bit words x1 (host arrays).
  * v_host[k] = the smallest vector index v with x1 < C_v, C the integer
  * cumulative weights in the table's order, or -1 for a null proposal
- * (x1 >= C_{V-1}).  Returns CG_EINVAL for bad arguments or a random-site
+ * (x1 >= C_{V-1}); -2 where the samplers (two-electron hops on clusters; all
+ * other lattice kernels, with each size of their guide) differ.  Returns CG_EINVAL for bad arguments or a random-site
  * replica (it draws from its partner lists), CG_ECUDA on a CUDA error;
  * allocates and frees device memory internally. */
 int cg_debug_tower(cg_handle *h, int replica, const uint32_t *x1_host, int32_t *v_host, int n);

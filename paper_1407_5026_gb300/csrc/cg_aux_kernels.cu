@@ -12,7 +12,7 @@
 //                 for tests.
 #include "cg_device.cuh"
 #include "cg_internal.h"
-#include "cg_pr_common.cuh"
+#include "cg_pr_lattice.cuh"
 
 namespace cg {
 
@@ -260,9 +260,27 @@ __global__ void debug_tower_kernel(const unsigned short *guide, const unsigned *
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
-    // the PR kernels' sampler (on the global copies of the tables); -1 marks a
-    // null proposal
+    // two-electron hops on clusters (on the global copies of the tables); -1
+    // marks a null proposal
     out[t] = x1[t] > thr[V - 1] ? -1 : tower_lookup(guide, thr, x1[t]);
+}
+
+// The sampler of the other lattice kernels, with a guide of 2^bits bytes staged as
+// they stage it; a word on which the two differ becomes -2.
+__global__ void __launch_bounds__(256) debug_lat_tower_kernel(const DevReplica *__restrict__ rep,
+                                                              int bits, const uint32_t *x1,
+                                                              int *out, int n)
+{
+    const int V = rep->V;
+    const LatLayout lay = lat_layout(0, 0, V, 0, 8, bits);
+    stage_tower<256, false, 2>(lay, *rep, bits, rep->L, 0);
+    __syncthreads();
+    const unsigned last = sm<unsigned>(lay.off_thr, V - 1);
+    for (int t = blockIdx.x * 256 + threadIdx.x; t < n; t += gridDim.x * 256) {
+        int v;
+        if (!lat_draw(lay, x1[t], 32 - bits, lat_guide_base(V), V - 1, last, v)) v = -1;
+        if (out[t] != v) out[t] = -2;
+    }
 }
 
 // g(eps): one CTA per (chunk of sites, replica) builds a shared-memory
@@ -301,10 +319,20 @@ cudaError_t launch_eps_histogram(const DevReplica *d_reps, int count, int max_N,
     return cudaGetLastError();
 }
 
-cudaError_t launch_debug_tower(const unsigned short *guide, const unsigned *thr, int V,
-                               const uint32_t *x1, int *out, int n, cudaStream_t st)
+cudaError_t launch_debug_tower(const DevReplica *d_rep, const unsigned short *guide,
+                               const unsigned *thr, int V, const uint32_t *x1, int *out, int n,
+                               cudaStream_t st)
 {
     debug_tower_kernel<<<(n + 127) / 128, 128, 0, st>>>(guide, thr, V, x1, out, n);
+    for (int bits = 12; bits <= kLatGuideBits; ++bits) {
+        const int smem = lat_layout(0, 0, V, 0, 8, bits).total;
+        if (smem > kSmemPerCta - lat_static_bytes(false)) break;      // no kernel takes it either
+        const cudaError_t e = cudaFuncSetAttribute(
+            debug_lat_tower_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e) return e;
+        const int ctas = (n + 255) / 256;
+        debug_lat_tower_kernel<<<ctas < 304 ? ctas : 304, 256, smem, st>>>(d_rep, bits, x1, out, n);
+    }
     return cudaGetLastError();
 }
 

@@ -314,8 +314,9 @@ cudaError_t launch_debug_philox(const uint32_t *ctr, const uint32_t *key,
 cudaError_t launch_debug_exp(const double *x, double *out, int n, cudaStream_t st);
 cudaError_t launch_debug_gauss(const uint64_t *seed, const uint32_t *rep, const uint64_t *hop,
                                double *z, int n, cudaStream_t st);
-cudaError_t launch_debug_tower(const unsigned short *guide, const unsigned *thr, int V,
-                               const uint32_t *x1, int *out, int n, cudaStream_t st);
+cudaError_t launch_debug_tower(const DevReplica *d_rep, const unsigned short *guide,
+                               const unsigned *thr, int V, const uint32_t *x1, int *out, int n,
+                               cudaStream_t st);
 cudaError_t set_pr_smem_limit(int precision, int bytes, bool pair);
 int microbench(int kind, int device, double *result);
 // Histogram of eps (binary64 or binary32 by precision) of `count` replicas

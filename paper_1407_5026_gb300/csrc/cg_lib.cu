@@ -2403,7 +2403,7 @@ int cg_debug_tower(cg_handle *h, int replica, const uint32_t *x1_host, int32_t *
     uint32_t *dx = (uint32_t *)d;
     int *dv = (int *)(d + 4 * (size_t)n);
     cudaError_t e = cudaMemcpy(dx, x1_host, 4 * (size_t)n, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = launch_debug_tower(t.d_guide, t.d_thr, t.V, dx, dv, n, 0);
+    if (e == cudaSuccess) e = launch_debug_tower(h->d_reps + replica, t.d_guide, t.d_thr, t.V, dx, dv, n, 0);
     if (e == cudaSuccess) e = cudaMemcpy(v_host, dv, 4 * (size_t)n, cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return fail(CG_ECUDA, cudaGetErrorString(e));

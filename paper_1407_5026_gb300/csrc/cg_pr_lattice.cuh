@@ -221,6 +221,18 @@ __device__ __forceinline__ bool lat_search(const LatLayout &S, uint32_t x1, unsi
     return true;
 }
 
+// The vector of a word x1: the guide's, or the search's where it has none; false
+// for a null proposal (v is then some vector's index).
+__device__ __forceinline__ bool lat_draw(const LatLayout &S, uint32_t x1, int gshift, int vbase,
+                                         int vlast, unsigned thr_last, int &v)
+{
+    const int g = (int)sm<unsigned char>(S.off_guide, x1 >> gshift);
+    v = g + vbase;
+    if (g != 255) return true;
+    v = vlast;
+    return lat_search(S, x1, thr_last, v);
+}
+
 // What a label's evaluation reads that stays fixed over a launch.
 struct LatConst {
     LatLayout S;
@@ -263,13 +275,7 @@ __device__ __forceinline__ LatPair lat_pair(const LatConst &K, unsigned label,
     const unsigned W = (unsigned)(2 * R + 1);
     const int ex = (int)__umulhi(y[0], W) - R, ey = (int)__umulhi(y[2], W) - R;
     const int ez = kDim == 3 ? (int)__umulhi(y[3], W) - R : 0;
-    const int g = (int)sm<unsigned char>(K.S.off_guide, y[1] >> K.gshift);
-    q.v2 = g + K.vbase;
-    bool live = true;
-    if (g == 255) {
-        q.v2 = K.vlast;
-        live = lat_search(K.S, y[1], K.thr_last, q.v2);
-    }
+    const bool live = lat_draw(K.S, y[1], K.gshift, K.vbase, K.vlast, K.thr_last, q.v2);
     const uint2 rc = sm<uint2>(K.S.off_rec, q.v2);
     q.cv2 = __uint_as_float(rc.x);
     q.w2 = rc.y;
