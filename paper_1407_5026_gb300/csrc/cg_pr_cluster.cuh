@@ -392,7 +392,7 @@ pr_cluster(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
                     for (unsigned k = (unsigned)warp * 32u; k < sub; k += kThreads)
                         if (lat_eval_toy<kPow2, kDim>(K, base + k, PP, V, a.toy_A0, &s_best[parity]))
                             break;
-                } else if (sub >= 64u) {
+                } else {
                     const unsigned k = (unsigned)warp * 64u;
                     if (k < sub)
                         cluster_eval<Real, kPow2, kDim, 2>(cl, K, eps, rows_local, rank, magicB,

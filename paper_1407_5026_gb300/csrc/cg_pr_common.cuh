@@ -457,17 +457,6 @@ __device__ __forceinline__ bool accept_pair_vals(Real ei, Real ej, Real ek, Real
     return (float)(p.x2 >> 9) < __fmaf_rn(__expf(-dEf * invTf), 0x1p23f, -0.5f);
 }
 
-template <typename Real, bool kPow2, int kDim = 2>
-__device__ __forceinline__ bool accept_pair(const Shared &S, const DevReplica &Rg, const Prop &p,
-                                            const PairProp &q, double T, float invTf,
-                                            double &dE_out, int L, int log2L, unsigned magic,
-                                            int H1)
-{
-    const Real *eps = reinterpret_cast<const Real *>(S.eps);
-    return accept_pair_vals<Real, kPow2, kDim>(eps[p.i], eps[p.j], eps[q.k], eps[q.l], S, Rg, p, q, T,
-                                         invTf, dE_out, L, log2L, magic, H1);
-}
-
 // dH of an executed pair in binary64 (binary32 form: from the widened
 // energies and the binary64 table, once per hop).
 template <typename Real, bool kPow2, int kDim = 2>
@@ -481,24 +470,6 @@ __device__ __forceinline__ double pair_hop_dE_vals(Real ei, Real ej, Real ek, Re
                                   q, L, log2L, magic, H1);
 }
 
-template <typename Real, bool kPow2, int kDim = 2>
-__device__ __forceinline__ double pair_hop_dE(const Shared &S, const DevReplica &Rg,
-                                              const Prop &p, const PairProp &q, double dE,
-                                              int L, int log2L, unsigned magic, int H1)
-{
-    const Real *eps = reinterpret_cast<const Real *>(S.eps);
-    return pair_hop_dE_vals<Real, kPow2, kDim>(eps[p.i], eps[p.j], eps[q.k], eps[q.l], S, Rg, p, q,
-                                         dE, L, log2L, magic, H1);
-}
-
-template <typename Real>
-__device__ __forceinline__ bool accept(const Shared &S, const Prop &p, double T, float invTf,
-                                       double &dE_out)
-{
-    const Real *eps = reinterpret_cast<const Real *>(S.eps);
-    return accept_vals<Real>(eps[p.i], eps[p.j], S, p, T, invTf, dE_out);
-}
-
 // dH of the executed hop in binary64 (the binary32 form widens it here, once
 // per hop, instead of on every label).
 template <typename Real>
@@ -508,13 +479,6 @@ __device__ __forceinline__ double hop_dE_vals(Real ei, Real ej, const Shared &S,
     if (sizeof(Real) == 8 || dE != 0.0) return dE;
     const float dEf = __fsub_rn(__fsub_rn((float)ej, (float)ei), S.cv32[p.v]);
     return (double)dEf;
-}
-
-template <typename Real>
-__device__ __forceinline__ double hop_dE(const Shared &S, const Prop &p, double dE)
-{
-    const Real *eps = reinterpret_cast<const Real *>(S.eps);
-    return hop_dE_vals<Real>(eps[p.i], eps[p.j], S, p, dE);
 }
 
 }  // namespace cg
