@@ -179,10 +179,30 @@ __device__ __forceinline__ double nu_shift(const DevReplica &R)
 {
     return d_mul(d_sub((double)(float)R.nu, R.nu), R.C0);
 }
-__device__ __forceinline__ float2 split_f32(double c)
+
+// What a CTA keeps of its pair in shared memory.  Values and maxima that take
+// binary64 are formed once per CTA: 28 conversions and sums in every thread
+// filled a third of the kernel's time with that pipe (304 replicas of L = 128:
+// 50 us).
+struct PairShared {
+    float2 shift[2];               // nu_shift as the sum of two binary32 numbers
+    float nu[2];
+    unsigned long long err[2];     // largest change of refresh_site64, binary64 bits
+    float3 most[2][32];            // the warps' largest other changes
+};
+
+// By the first two threads of a CTA; a barrier before the first use.
+__device__ __forceinline__ void pair_consts(PairShared &k, const DevReplica &Ra,
+                                            const DevReplica &Rb)
 {
-    const float h = (float)c;
-    return make_float2(h, (float)d_sub(c, (double)h));
+    if (threadIdx.x < 2) {
+        const DevReplica &R = threadIdx.x ? Rb : Ra;
+        const double c = nu_shift(R);
+        const float h = (float)c;
+        k.shift[threadIdx.x] = make_float2(h, (float)d_sub(c, (double)h));
+        k.nu[threadIdx.x] = (float)R.nu;
+        k.err[threadIdx.x] = 0ull;
+    }
 }
 
 // eps_new of a site in binary64, for the values that refresh_site leaves out; the
@@ -204,8 +224,8 @@ __device__ __noinline__ float refresh_site64(double phi, float v, const DevRepli
 // same sum in binary64 loses 2^-53 (over W = 0 to 14 and c up to 2e-5, the largest
 // error of a change near 1e-6: 9e-19 against 1.3e-15).  In binary64 the step is ten
 // operations per site at 1/64 of the binary32 rate; with 24 bits of each part, and
-// the change in binary32, a resume is 3 to 5% faster (304 replicas of L = 128 230
-// against 238 us, 128 of L = 112 124 against 131) and a change 1e3 to 1e5 times as
+// the change in binary32, a resume is 1 to 5% faster (304 replicas of L = 128 230
+// against 234 us, 128 of L = 112 124 against 130) and a change 1e3 to 1e5 times as
 // far off.  A phi that is not 0 and outside
 // 2^-74 to 2^78, and an eps_old past 2^100, are left to binary64.
 __device__ __forceinline__ float refresh_site(double phi, float v, float2 c, float eps_old,
@@ -238,36 +258,43 @@ __device__ __forceinline__ float refresh_site(double phi, float v, float2 c, flo
     return __fadd_rn(r.x, __fadd_rn(r.y, u));
 }
 
+// The larger of two changes (sums of three binary32 numbers, largest first).
+__device__ __forceinline__ float3 larger(float3 a, float3 b)
+{
+    return b.x > a.x || (b.x == a.x && b.y > a.y) ? b : a;
+}
+__device__ __forceinline__ float3 warp_most(float3 c)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        c = larger(c, make_float3(__shfl_xor_sync(0xffffffffu, c.x, o),
+                                  __shfl_xor_sync(0xffffffffu, c.y, o),
+                                  __shfl_xor_sync(0xffffffffu, c.z, o)));
+    return c;
+}
+
 // The block's maxima of the changes of two replicas into their counters.
 __device__ __forceinline__ void record_change(float3 ca, float3 cb, bool two, bool count,
-                                              DevCounters *da, DevCounters *db,
-                                              unsigned long long *s_err)
+                                              DevCounters *da, DevCounters *db, PairShared &ps)
 {
-    // non-negative binary64 numbers order as their bits
-    auto bits = [](float3 c) {
-        const double v = d_add((double)c.x, d_add((double)c.y, (double)c.z));
-        return (unsigned long long)__double_as_longlong(v);
-    };
-    unsigned long long ba = bits(ca), bb = bits(cb);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        const unsigned long long xa = __shfl_xor_sync(0xffffffffu, ba, o);
-        const unsigned long long xb = __shfl_xor_sync(0xffffffffu, bb, o);
-        ba = ba > xa ? ba : xa;
-        bb = bb > xb ? bb : xb;
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&s_err[0], ba);
-        atomicMax(&s_err[1], bb);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    ca = warp_most(ca);
+    cb = warp_most(cb);
+    if (lane == 0) {
+        ps.most[0][warp] = ca;
+        ps.most[1][warp] = cb;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        atomicMax(&da->max_err_bits, s_err[0]);
-        if (count) atomicAdd(&da->refreshes, 1ull);
-        if (two) {
-            atomicMax(&db->max_err_bits, s_err[1]);
-            if (count) atomicAdd(&db->refreshes, 1ull);
-        }
+    if (warp) return;
+    for (int r = 0; r < (two ? 2 : 1); ++r) {
+        const float3 c = warp_most(ps.most[r][lane < (int)(blockDim.x >> 5) ? lane : 0]);
+        if (lane) continue;
+        DevCounters *d = r ? db : da;
+        // non-negative binary64 numbers order as their bits
+        const double v = d_add((double)c.x, d_add((double)c.y, (double)c.z));
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+        atomicMax(&d->max_err_bits, b > ps.err[r] ? b : ps.err[r]);
+        if (count) atomicAdd(&d->refreshes, 1ull);
     }
 }
 
@@ -289,7 +316,7 @@ template <int kMode>
 __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int axis)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned long long s_err[2];
+    __shared__ PairShared ps;
     const int L = a.L, W = a.W, Ls = L + 1;     // padded line stride (banks)
     const int groups = (int)(gridDim.x / (unsigned)((a.R + 1) / 2));
     const int p = blockIdx.x / groups, g = blockIdx.x - p * groups;
@@ -318,7 +345,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         }
         s[w * Ls + (natural_in ? k : (int)bitrev((unsigned)k, a.log2L))] = v;
     }
-    if (kMode == 4 && threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
+    if (kMode == 4) pair_consts(ps, Ra, Rb);
     __syncthreads();
     // ---- transform ----
     float2 *out = s;                                       // where the result lies
@@ -371,15 +398,15 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
         const double *__restrict__ pb = Rb.phi + site0;
         float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps) + site0;
         float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps) + site0;
-        const float2 ca = split_f32(nu_shift(Ra)), cb = split_f32(nu_shift(Rb));
+        const float2 ca = ps.shift[0], cb = ps.shift[1];
 #pragma unroll 4
         for (int e = threadIdx.x; e < n; e += kFftThreads) {
             const int w = e / L, k = e - w * L;
             const float2 v = out[w * Ls + out_pos(k, a, true)];
-            ea[e] = refresh_site(pa[e], v.x, ca, ea[e], Ra, &s_err[0], err_a);
-            if (two) eb[e] = refresh_site(pb[e], v.y, cb, eb[e], Rb, &s_err[1], err_b);
+            ea[e] = refresh_site(pa[e], v.x, ca, ea[e], Ra, &ps.err[0], err_a);
+            if (two) eb[e] = refresh_site(pb[e], v.y, cb, eb[e], Rb, &ps.err[1], err_b);
         }
-        record_change(err_a, err_b, two, g == 0, Ra.ctr, Rb.ctr, s_err);
+        record_change(err_a, err_b, two, g == 0, Ra.ctr, Rb.ctr, ps);
     }
 }
 
@@ -586,6 +613,7 @@ struct Plane {
     static constexpr int R1 = L / 8, kT = fft_plane_threads<L>(), Ls = L + 1;
     static constexpr int kSmem = (L * Ls + L) * (int)sizeof(float2);
     float2 *s, *tw;
+    PairShared *ps;
 
     __device__ __forceinline__ float2 &at(int y, int x) const
     {
@@ -621,7 +649,7 @@ struct Plane {
     __device__ __forceinline__ void x_from_bits(const DevReplica &Ra, const DevReplica &Rb, bool two,
                                                 unsigned site0) const
     {
-        const float na = (float)Ra.nu, nb = (float)Rb.nu;
+        const float na = ps->nu[0], nb = ps->nu[1];
         for (int it = threadIdx.x; it < L * 8; it += kT) {
             const int b = it & 7, y = row_of(it >> 3);
             float2 v[R1];
@@ -743,13 +771,13 @@ struct Plane {
     // x, the inverse's second step, into eps of the plane at site0; the largest
     // changes of the thread's sites
     __device__ __forceinline__ void x_into_eps(const DevReplica &Ra, const DevReplica &Rb, bool two,
-                                               unsigned site0, unsigned long long *s_err,
-                                               float3 &err_a, float3 &err_b) const
+                                               unsigned site0, float3 &err_a,
+                                               float3 &err_b) const
     {
         const double *__restrict__ pa = Ra.phi + site0, *__restrict__ pb = Rb.phi + site0;
         float *__restrict__ ea = reinterpret_cast<float *>(Ra.eps) + site0;
         float *__restrict__ eb = reinterpret_cast<float *>(Rb.eps) + site0;
-        const float2 ca = split_f32(nu_shift(Ra)), cb = split_f32(nu_shift(Rb));
+        const float2 ca = ps->shift[0], cb = ps->shift[1];
         for (int it = threadIdx.x; it < L * 8; it += kT) {
             const int b = it & 7, y = row_of(it >> 3), site = y * L + b;
             float2 v[R1];
@@ -773,9 +801,9 @@ struct Plane {
 #pragma unroll
                 for (int k = 0; k < kBatch; ++k) {
                     const int e = site + 8 * (k0 + k);
-                    ea[e] = refresh_site(fa[k], v[k0 + k].x, ca, oa[k], Ra, &s_err[0], err_a);
+                    ea[e] = refresh_site(fa[k], v[k0 + k].x, ca, oa[k], Ra, &ps->err[0], err_a);
                     if (two)
-                        eb[e] = refresh_site(fb[k], v[k0 + k].y, cb, ob[k], Rb, &s_err[1], err_b);
+                        eb[e] = refresh_site(fb[k], v[k0 + k].y, cb, ob[k], Rb, &ps->err[1], err_b);
                 }
             }
         }
@@ -797,14 +825,14 @@ template <int L>
 __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_square_kernel(FftArgs a)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned long long s_err[2];
-    const Plane<L> P{s, s + L * Plane<L>::Ls};
+    __shared__ PairShared ps;
+    const Plane<L> P{s, s + L * Plane<L>::Ls, &ps};
     const int p = blockIdx.x;
     const DevReplica &Ra = a.reps[a.index[2 * p]];
     const bool two = 2 * p + 1 < a.R;
     const DevReplica &Rb = a.reps[a.index[two ? 2 * p + 1 : 2 * p]];
     P.twiddles(a.tw);
-    if (threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
+    pair_consts(ps, Ra, Rb);
     clear_change(two, Ra.ctr, Rb.ctr);
     __syncthreads();
     P.prefetch(Ra, 0u);
@@ -820,8 +848,8 @@ __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_square_kernel(FftA
     P.x_inverse1();
     __syncthreads();
     float3 err_a = make_float3(0.0f, 0.0f, 0.0f), err_b = err_a;
-    P.x_into_eps(Ra, Rb, two, 0u, s_err, err_a, err_b);
-    record_change(err_a, err_b, two, true, Ra.ctr, Rb.ctr, s_err);
+    P.x_into_eps(Ra, Rb, two, 0u, err_a, err_b);
+    record_change(err_a, err_b, two, true, Ra.ctr, Rb.ctr, ps);
 }
 
 // The cubic lattice in three launches over L x L planes: x and y of a z-plane
@@ -832,9 +860,9 @@ template <int L, int kStep>
 __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftArgs a)
 {
     extern __shared__ float2 s[];
-    __shared__ unsigned long long s_err[2];
+    __shared__ PairShared ps;
     constexpr int R1 = L / 8;
-    const Plane<L> P{s, s + L * Plane<L>::Ls};
+    const Plane<L> P{s, s + L * Plane<L>::Ls, &ps};
     const int p = blockIdx.x / L, o = blockIdx.x - p * L;
     const DevReplica &Ra = a.reps[a.index[2 * p]];
     const bool two = 2 * p + 1 < a.R;
@@ -842,7 +870,7 @@ __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftAr
     float2 *buf = a.buf + (size_t)p * L * L * L;
     const unsigned site0 = (unsigned)(o * L * L);
     P.twiddles(a.tw);
-    if (kStep == 2 && threadIdx.x < 2) s_err[threadIdx.x] = 0ull;
+    if (kStep != 1) pair_consts(ps, Ra, Rb);
     __syncthreads();
     if (kStep == 0) {
         if (o == 0) clear_change(two, Ra.ctr, Rb.ctr);
@@ -870,8 +898,8 @@ __global__ void __launch_bounds__(fft_plane_threads<L>()) fft_cubic_kernel(FftAr
         P.x_inverse1();
         __syncthreads();
         float3 err_a = make_float3(0.0f, 0.0f, 0.0f), err_b = err_a;
-        P.x_into_eps(Ra, Rb, two, site0, s_err, err_a, err_b);
-        record_change(err_a, err_b, two, o == 0, Ra.ctr, Rb.ctr, s_err);
+        P.x_into_eps(Ra, Rb, two, site0, err_a, err_b);
+        record_change(err_a, err_b, two, o == 0, Ra.ctr, Rb.ctr, ps);
     }
 }
 
