@@ -42,8 +42,8 @@ L2_FLUSH_BYTES = 256 << 20    # > 129 MB L2
 # CTAs per replica).  M changes which labels are drawn, not the bytes (the
 # state is loaded and stored once per launch): captures at M = 4096 and
 # 16384 gave 20.748 and 20.742 MB.
-TRAFFIC_CAPTURE = {"sources_sha256_16": "651cca43504ee42b", "bytes_per_launch": 20.752e6,
-                   "replicas": 304, "hops_per_replica": 1024, "M": 16384, "threads": 512,
+TRAFFIC_CAPTURE = {"sources_sha256_16": "ae8933914cf24ddd", "bytes_per_launch": 20.764e6,
+                   "replicas": 304, "hops_per_replica": 1024, "M": 4096, "threads": 256,
                    "cluster": 1}
 
 
@@ -153,7 +153,8 @@ def workload_config(args, R):
                        f"{args.M})"),
             "refresh": "every 1024 hops: eps from its definition by the convolution "
                        "theorem (binary32 FFTs, two replicas per complex "
-                       "transform, times DFT(1/r); phi added in binary64)",
+                       "transform, times DFT(1/r); phi added with all of its bits, one "
+                       "rounding to binary32)",
             "l2": "256 MB buffer zeroed between steps (outside the timed events)",
             "state": f"chains relaxed {args.relax_steps * HOPS_PER_STEP} hops from "
                      f"their random start, then {args.warmup} warm-up steps"}

@@ -312,7 +312,9 @@ int cg_observables(cg_handle *h, int replica, cg_obs *out);
  *     eps - phi = IDFT(DFT(n - nu) DFT(1/r)) on the periodic lattice,
  *     transforms in binary32 with two replicas per
  *     complex transform (DFT(1/r) is real), DFT(1/r) and the
- *     twiddles from binary64 on the host, phi added in binary64 (error below
+ *     twiddles from binary64 on the host, phi added with all of its bits (at
+ *     least as exactly as in binary64) and one rounding to binary32, which
+ *     the largest change is taken before (error below
  *     2e-5 up to L = 256 square and L = 64 cubic, measured against the
  *     definition);
  *   - otherwise, a group of replicas of one L whose N is a multiple of 128

@@ -205,8 +205,9 @@ cudaError_t launch_reset_refresh_err(const DevReplica *d_reps, const int *d_inde
 
 // Positions sorted by falling attempts per hop (rank by counting: at most a few
 // hundred replicas), and the claim table cleared.  A batch of two replicas per
-// SM lasts as long as its slowest SM: 304 of L = 128 at T = 0.01, 11.16 -> 10.62
-// ms per 1024 hops with heavy and light ones paired; this launch takes 5 us.
+// SM lasts as long as its slowest SM: 304 of L = 128 at T = 0.01 that run on, 10.30
+// ms per 1024 hops in replica order, 9.88 with heavy and light ones paired; this
+// launch takes 5 us.
 __global__ void __launch_bounds__(1024) pr_schedule_kernel(const DevReplica *__restrict__ reps,
                                                            const int *__restrict__ index,
                                                            int count, int *__restrict__ sched)

@@ -42,7 +42,8 @@ struct alignas(16) DevCounters {
 constexpr int kGuideBits = 12;
 constexpr int kGuide = 1 << kGuideBits;
 
-// Guide table of the single-hop lattice kernel (cg_pr_lattice.cuh): bucket
+// Guide table of the lattice kernels but for two-electron hops on clusters
+// (cg_pr_lattice.cuh): bucket
 // b = x1 >> (32 - kLatGuideBits) holds v - lat_guide_base(V) when every x1 of
 // the bucket selects the same vector v and that difference is in [0, 254],
 // else 255 (the kernel then searches the thresholds between the bounds of
@@ -159,8 +160,8 @@ __host__ __device__ inline SmemLayout smem_layout(int N, int tab_entries, int V,
     return s;
 }
 
-// Shared-memory carve-up of the single-hop lattice kernel (cg_pr_lattice.cuh)
-// with a guide table of 2^gbits entries.
+// Shared-memory carve-up of the lattice kernels but for two-electron hops on
+// clusters (cg_pr_lattice.cuh), with a guide table of 2^gbits entries.
 struct LatLayout {
     int off_eps, off_tinv, off_occ, off_guide, off_hint, off_thr, off_rec;
     int off_vr64, off_edx64, total;

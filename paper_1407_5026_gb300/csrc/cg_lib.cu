@@ -125,8 +125,9 @@ struct Tables {
     std::vector<float> r2_32;
     double *d_r2_64 = nullptr;
     float *d_r2_32 = nullptr;
-    // the FFT refresh (binary32 handles, power-of-two L): DFT(g) / N of the
-    // minimum-image 1/r (real: g is even) and the twiddles exp(-2 pi i k/L)
+    // the FFT refresh (groups of group_uses_fft; the first table of a side and
+    // dimension has them): DFT(g) / N of the minimum-image 1/r (real: g is even)
+    // and the twiddles exp(-2 pi i k/L)
     std::vector<float> ghat;
     std::vector<float2> tw;
     float *d_ghat = nullptr;
@@ -1407,7 +1408,8 @@ cg_handle *create_impl(int R, const cg_replica_desc *reps, const cg_opts *opts, 
 }
 
 // Rebuild eps of one group's replicas from scratch (binary64: the serial-order
-// kernel; binary32: the tensor-core contraction or the binary64 direct sum).
+// kernel; binary32: the transforms, the tensor-core contraction or the binary64
+// direct sum).
 int refresh_group(cg_handle *h, const Group &g, cudaStream_t st)
 {
     if (h->opts.precision != CG_FP32) {

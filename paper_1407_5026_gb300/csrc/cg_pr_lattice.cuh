@@ -23,10 +23,13 @@
 //   Update (step 3b): eps_l += 1/r_lj - 1/r_li for every l, with the table
 //   holding 0 at the origin so l = i and l = j need no special case.
 //
-// What bounds it (L = 128, T = 0.01, 304 replicas, two CTAs per SM): a label costs about 85 warp instructions per 32 labels, 47 of them on
-// the integer pipe and 24 on the multiplier, and time goes with their sum
-// (Philox alone is 40 of the 71); alone it runs at 266 G labels/s, 470 G being
-// the generator by itself.  More warps change nothing.  So the per-label work
+// What bounds it (L = 128, T = 0.01, 304 replicas, two CTAs per SM): 32 labels
+// cost 97 warp instructions (counted), 50 of them on the integer pipe, 28 on the
+// multiply pipe and 6 loads; Philox alone is 40 of the 78.  Half of the issue
+// slots are taken; fixed latencies, the chunks' barriers and shared-memory latency
+// come first among the waits.  Labels run at 120 G/s over a launch and 151 G/s
+// over the rejection phase, the generator by itself at 464.  More warps change
+// nothing.  So the per-label work
 // was cut: only a label whose theta holds and whose dH is below the cut (one in
 // a few hundred) reaches the exponential, the near-tie test and, in binary64,
 // the slow binary64 pipe (its dH is first bounded from the energies' high
@@ -35,10 +38,10 @@
 // no second barrier: the accepting warps write their proposals and lower a
 // shared minimum before the one that ends the chunk.
 // ms per run call of the kernel before (150 instructions per label, 512 threads
-// throughout) and of this one, same chains: L = 128 binary32 12.12 -> 9.66,
-// binary64 (152 replicas) 2.95 -> 1.94; 24 binary64 chains of L = 64 4.25 ->
-// 2.44; L = 32 to 96 mixed 3.16 -> 1.63; 32^3 2.24 -> 1.93; L = 64 with a fifth
-// pair labels 2.53 -> 1.92.  Four labels per lane in place of two gained
+// throughout) and of this one, same chains: L = 128 binary32 12.12 -> 9.77,
+// binary64 (152 replicas) 2.95 -> 1.36; 24 binary64 chains of L = 64 4.25 ->
+// 2.38; L = 32 to 96 mixed 3.16 -> 1.69; 32^3 2.24 -> 1.94; L = 64 with a fifth
+// pair labels 2.53 -> 1.89.  Four labels per lane in place of two gained
 // nothing (9.60 to 9.68 against 9.66; mixed 1.65 against 1.62), and neither did a search
 // without barriers, which evaluates labels past the accepting one.
 #pragma once
@@ -530,9 +533,9 @@ __device__ __forceinline__ bool lat_eval_toy(const LatConst &K, unsigned kb, con
 
 // The replica position this CTA runs: the first CTA on an SM takes one of the
 // heavier half of the order, the second the lighter one that matches it, so the
-// SMs' sums of attempts come out close (304 replicas of L = 128 at T = 0.01:
-// the largest sum is 1.10 of the mean; 1.32 in replica order, and the launch
-// lasts as long as its slowest SM).  The SM only sets the preferred position: a
+// SMs' sums of attempts come out close (304 replicas of L = 128 at T = 0.01, by
+// the launch's own attempts: the largest sum is 1.10 of the mean; 1.32 in replica
+// order, and the launch lasts as long as its slowest SM).  The SM only sets the preferred position: a
 // taken one passes on to the next, so every position is run exactly once
 // wherever the CTAs land.
 __device__ __forceinline__ int claim_replica(int *sched, int count, int n_sms)
@@ -648,7 +651,7 @@ pr_lattice(const DevReplica *__restrict__ reps, const int *__restrict__ index, R
 
     // binary64: the energies and the table in fixed point where that is exact
     // for every one of them (the configurations' W = 1 and 2 at half filling;
-    // a W that is no short binary fraction leaves small energies finer bits)
+    // a W that is no short binary fraction may leave small energies finer bits)
     bool fixed = false;
     if constexpr (kF64) {
         // from 1024 sites on: below, the update waits for latency, not for the

@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(FftArgs a, int ax
 // pair: its L x L complex values stay in shared memory (132 KiB at L = 128)
 // through all the transforms, where the passes above write and read them through
 // L2 between launches and run a barrier per radix-2 stage (304 replicas of
-// L = 128: 0.225 -> 0.085 ms).  Cubic lattices take three launches over planes
+// L = 128: 0.15 -> 0.05 ms on the device).  Cubic lattices take three launches over planes
 // instead of five passes (152 of 32^3: 0.243 -> 0.067 ms; 16 of 48^3: 0.104 ->
 // 0.050).  Sides that are neither 2^m nor 3 2^m take the place of
 // the tensor-core contraction (128 of L = 112, a resume with its copies: 329 ->
